@@ -32,9 +32,10 @@ int launch_core(dgfs::Plan& p, const void* f, void* Q, int batch, cudaStream_t s
   if (sum && (stage_node + batch > p.max_batch || !p.d_Qfull)) return DGFS_ERR_BUDGET;
   const size_t n3 = size_t(p.N) * p.N * p.N;
   void* Qfull = sum ? static_cast<char*>(p.d_Qfull) + size_t(stage_node) * p.s * p.s * n3 * dgfs::real_size(p) : Q;
-  int rc = p.precision == DGFS_FP32     ? dgfs::launch_f32(p, f, Qfull, batch, st, ws)
-           : p.precision == DGFS_BF16X3 ? dgfs::launch_bf16x3(p, f, Qfull, batch, st, ws)
-                                        : dgfs::launch_f64(p, f, Qfull, batch, st, ws);
+  auto* const run = p.precision == DGFS_BF16X3 ? dgfs::launch_bf16x3
+                    : p.precision == DGFS_FP32 ? (p.vss ? dgfs::launch_f32 : dgfs::launch_vhs_f32)
+                                               : (p.vss ? dgfs::launch_f64 : dgfs::launch_vhs_f64);
+  int rc = run(p, f, Qfull, batch, st, ws);
   if (rc != DGFS_OK) return rc;
   *launches += 1;
   if (p.flags & DGFS_CONSERVE) {
@@ -98,9 +99,9 @@ int dgfs_create_plan(const dgfs_plan_desc* desc, dgfs_plan* out) {
   int rc = dgfs::build_plan(desc, p);
   if (rc == DGFS_OK && cudaGetDevice(&p.device) != cudaSuccess) rc = DGFS_ERR_CUDA;
   if (rc == DGFS_OK)
-    rc = p.precision == DGFS_FP32     ? dgfs::configure_f32(p)
-         : p.precision == DGFS_BF16X3 ? dgfs::configure_bf16x3(p)
-                                      : dgfs::configure_f64(p);
+    rc = p.precision == DGFS_BF16X3 ? dgfs::configure_bf16x3(p)
+         : p.precision == DGFS_FP32 ? (p.vss ? dgfs::configure_f32(p) : dgfs::configure_vhs_f32(p))
+                                    : (p.vss ? dgfs::configure_f64(p) : dgfs::configure_vhs_f64(p));
   if (rc == DGFS_OK) rc = dgfs::upload_plan(p);
   if (rc != DGFS_OK) {
     dgfs::free_plan(p);

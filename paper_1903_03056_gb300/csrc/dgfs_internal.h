@@ -12,6 +12,20 @@
 
 #include "dgfs.h"
 
+// the grid sizes the kernels are built for
+#define DGFS_DISPATCH(T, N_, CALL) \
+  switch (N_) {                    \
+    case 4: return CALL(T, 4);     \
+    case 6: return CALL(T, 6);     \
+    case 8: return CALL(T, 8);     \
+    case 12: return CALL(T, 12);   \
+    case 16: return CALL(T, 16);   \
+    case 24: return CALL(T, 24);   \
+    case 32: return CALL(T, 32);   \
+    case 48: return CALL(T, 48);   \
+    default: return DGFS_ERR_UNSUPPORTED_N; \
+  }
+
 namespace dgfs {
 
 // One unit of gain work: the product sum P_rho(v) = sum_e w_e a_e(v) b_e(v) over the entries
@@ -24,6 +38,7 @@ struct TaskDesc {
   int out0, out1;
   int ent_off, n_ent;  // entries (sigma, weight) of this task
   int grp_off, n_grp;  // groups of entries sharing sigma_x
+  int face_off, n_face;  // faces of the VHS kernel: entries with a shift along x or y
 };
 
 struct GroupDesc {
@@ -36,12 +51,15 @@ struct KernelParams {
   int batch, s, n_tasks, n_rho, max_ent;
   const TaskDesc* tasks;
   const GroupDesc* groups;
+  const int* faces;       // face codes of the tasks: 2 e + kind, e the entry within its task, kind 0
+                          // (k_x = N/2) if sigma_x != 0, kind 1 (k_y = N/2) if sigma_y != 0
   const double* ent_w;    // [entries] sigma weight (x2 for halved self pairs)
   const void* phase;      // complex: [task][rho][max_ent][role 2][axis 3][N]
   const void* Fw;         // [s*s][n_rho][N^3]: w_rho F^(ij)(k, rho) / N^3, in the plan's real
                           // type (FP32 plans: each FP64 value rounded once)
   const void* Gm;         // [s*s][N^3]: G^(ij)-(k), in the plan's real type
-  void* scratch;          // complex: [clusters][SLOT][N^3]
+  void* scratch;          // complex: [clusters][slot]
+  size_t slot;            // complex values of workspace per cluster (VHS kernel)
   int phase_smem;         // 1: the task's phase block of the current rho is staged in smem;
                           // 2: only its z phases are
   unsigned* work_counter; // next work item (reset to 0 before every launch)
@@ -76,6 +94,7 @@ struct LaunchShape {
   size_t smem = 0;        // dynamic shared memory per CTA
   int phase_smem = 0;     // phases staged in shared memory
   int clusters = 0;       // resident clusters (persistent grid)
+  size_t slot = 0;        // complex values of workspace per cluster (VHS kernel)
   double share = 1.0;     // fraction of the resident clusters one launch may use
 };
 
@@ -103,6 +122,7 @@ struct Plan {
   std::vector<TaskDesc> tasks;
   std::vector<GroupDesc> groups;
   std::vector<double> ent_w;
+  std::vector<int> faces;       // face codes per task (KernelParams::faces)
   std::vector<int> ent_sigma;   // design index of each entry
   std::vector<int> ent_m;       // [entries][2] VSS table slot codes of the entry and its antipode
   std::vector<int> fslot;       // [M] VSS table slot code of each direction: 2 slot + conj bit
@@ -129,6 +149,7 @@ struct Plan {
   float* d_Gmf = nullptr;
   int* d_ent_m = nullptr;
   int* d_ent_ysh = nullptr;
+  int* d_faces = nullptr;
   double* d_Gm = nullptr;
   double* d_ent_w = nullptr;
   void* d_phase = nullptr;
@@ -188,6 +209,10 @@ void free_plan(Plan& p);
 // kernel configuration and launch, per precision (collision_f32.cu / collision_f64.cu)
 int configure_f32(Plan& p);
 int configure_f64(Plan& p);
+int configure_vhs_f32(Plan& p);
+int configure_vhs_f64(Plan& p);
+int launch_vhs_f32(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
+int launch_vhs_f64(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
 int launch_f32(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
 int launch_f64(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
 

@@ -18,6 +18,15 @@ template <> struct cplx_t<float> { using type = float2; };
 template <> struct cplx_t<double> { using type = double2; };
 template <typename T> using C = typename cplx_t<T>::type;
 
+// type of a real constant that multiplies a T (float for packed pairs of floats)
+template <typename T> struct real_const { using type = T; };
+template <typename T> using Const = typename real_const<T>::type;
+// a c and a c + b for a real constant c (packed types overload these)
+__device__ __forceinline__ float mulc(float a, float c) { return a * c; }
+__device__ __forceinline__ double mulc(double a, double c) { return a * c; }
+__device__ __forceinline__ float fmac(float a, float c, float b) { return a * c + b; }
+__device__ __forceinline__ double fmac(double a, double c, double b) { return a * c + b; }
+
 template <typename T> __device__ __forceinline__ C<T> mk(T x, T y) { C<T> r; r.x = x; r.y = y; return r; }
 template <typename T> __device__ __forceinline__ C<T> add(C<T> a, C<T> b) { return mk<T>(a.x + b.x, a.y + b.y); }
 template <typename T> __device__ __forceinline__ C<T> sub(C<T> a, C<T> b) { return mk<T>(a.x - b.x, a.y - b.y); }
@@ -28,6 +37,11 @@ template <typename T> __device__ __forceinline__ C<T> scale(C<T> a, T s) { retur
 // multiply by DIR * i
 template <typename T, int DIR> __device__ __forceinline__ C<T> mul_i(C<T> a) {
   return DIR > 0 ? mk<T>(-a.y, a.x) : mk<T>(a.y, -a.x);
+}
+
+// a + DIR i b
+template <typename T, int DIR> __device__ __forceinline__ C<T> add_i(C<T> a, C<T> b) {
+  return DIR > 0 ? mk<T>(a.x - b.y, a.y + b.x) : mk<T>(a.x + b.y, a.y - b.x);
 }
 
 // ---- compile-time cos / sin of 2 pi a / b -------------------------------------------
@@ -72,9 +86,9 @@ __device__ __forceinline__ C<T> twiddle(C<T> a) {
   } else if constexpr (4 * m == 3 * N) {
     return mul_i<T, -DIR>(a);
   } else {
-    constexpr T c = T(trig2pi(m, N, 0));
-    constexpr T s = T(DIR * trig2pi(m, N, 1));
-    return mk<T>(a.x * c - a.y * s, a.x * s + a.y * c);
+    constexpr Const<T> c = Const<T>(trig2pi(m, N, 0));
+    constexpr Const<T> s = Const<T>(DIR * trig2pi(m, N, 1));
+    return mk<T>(fmac(a.y, -s, mulc(a.x, c)), fmac(a.x, s, mulc(a.y, c)));
   }
 }
 
@@ -86,38 +100,41 @@ template <typename T, int DIR> __device__ __forceinline__ void dft2(C<T>* v) {
 }
 template <typename T, int DIR> __device__ __forceinline__ void dft4(C<T>* v) {
   const C<T> s02 = add<T>(v[0], v[2]), d02 = sub<T>(v[0], v[2]);
-  const C<T> s13 = add<T>(v[1], v[3]), d13 = mul_i<T, DIR>(sub<T>(v[1], v[3]));
+  const C<T> s13 = add<T>(v[1], v[3]), d13 = sub<T>(v[1], v[3]);
   v[0] = add<T>(s02, s13);
   v[2] = sub<T>(s02, s13);
-  v[1] = add<T>(d02, d13);
-  v[3] = sub<T>(d02, d13);
+  v[1] = add_i<T, DIR>(d02, d13);
+  v[3] = add_i<T, -DIR>(d02, d13);
 }
 template <typename T, int DIR> __device__ __forceinline__ void dft3(C<T>* v) {
-  constexpr T h = T(0.866025403784438646763723170752936183);  // sqrt(3)/2
+  constexpr Const<T> h = Const<T>(DIR * 0.866025403784438646763723170752936183);  // sqrt(3)/2
+  constexpr Const<T> half = Const<T>(-0.5);
   const C<T> t = add<T>(v[1], v[2]);
-  const C<T> d = mul_i<T, DIR>(sub<T>(v[1], v[2]));
-  const C<T> m = mk<T>(v[0].x - T(0.5) * t.x, v[0].y - T(0.5) * t.y);
+  const C<T> d = sub<T>(v[1], v[2]);
+  const C<T> m = mk<T>(fmac(t.x, half, v[0].x), fmac(t.y, half, v[0].y));
   v[0] = add<T>(v[0], t);
-  v[1] = mk<T>(m.x + h * d.x, m.y + h * d.y);
-  v[2] = mk<T>(m.x - h * d.x, m.y - h * d.y);
+  v[1] = mk<T>(fmac(d.y, -h, m.x), fmac(d.x, h, m.y));
+  v[2] = mk<T>(fmac(d.y, h, m.x), fmac(d.x, -h, m.y));
 }
 // 8-point DFT: two 4-point DFTs of the even and odd points joined by the eighth roots of unity
 // w = e^{DIR 2 pi i / 8}: X_k = E_k + w^k O_k, X_{k+4} = E_k - w^k O_k
 template <typename T, int DIR> __device__ __forceinline__ void dft8(C<T>* v) {
-  constexpr T r = T(0.707106781186547524400844362104849039);  // 1 / sqrt(2)
+  constexpr Const<T> r = Const<T>(0.707106781186547524400844362104849039);  // 1 / sqrt(2)
   C<T> e[4] = {v[0], v[2], v[4], v[6]};
   C<T> o[4] = {v[1], v[3], v[5], v[7]};
   dft4<T, DIR>(e);
   dft4<T, DIR>(o);
   // w^1 = (1 + DIR i) / sqrt 2, w^2 = DIR i, w^3 = (-1 + DIR i) / sqrt 2
-  o[1] = mk<T>(r * (o[1].x - DIR * o[1].y), r * (o[1].y + DIR * o[1].x));
-  o[2] = mul_i<T, DIR>(o[2]);
-  o[3] = mk<T>(r * (-o[3].x - DIR * o[3].y), r * (-o[3].y + DIR * o[3].x));
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    v[k] = add<T>(e[k], o[k]);
-    v[k + 4] = sub<T>(e[k], o[k]);
-  }
+  const C<T> o1 = add_i<T, DIR>(o[1], o[1]);   // (1 + DIR i) o_1
+  const C<T> o3 = add_i<T, -DIR>(o[3], o[3]);  // (1 - DIR i) o_3 = -(w^3 o_3) sqrt 2
+  v[0] = add<T>(e[0], o[0]);
+  v[4] = sub<T>(e[0], o[0]);
+  v[1] = mk<T>(fmac(o1.x, r, e[1].x), fmac(o1.y, r, e[1].y));
+  v[5] = mk<T>(fmac(o1.x, -r, e[1].x), fmac(o1.y, -r, e[1].y));
+  v[2] = add_i<T, DIR>(e[2], o[2]);
+  v[6] = add_i<T, -DIR>(e[2], o[2]);
+  v[3] = mk<T>(fmac(o3.x, -r, e[3].x), fmac(o3.y, -r, e[3].y));
+  v[7] = mk<T>(fmac(o3.x, r, e[3].x), fmac(o3.y, r, e[3].y));
 }
 template <typename T, int R, int DIR> __device__ __forceinline__ void dft_small(C<T>* v) {
   if constexpr (R == 2) dft2<T, DIR>(v);

@@ -403,6 +403,7 @@ int build_plan(const dgfs_plan_desc* d, Plan& p) {
   p.groups.clear();
   p.ent_w.clear();
   p.ent_sigma.clear();
+  p.faces.clear();
   p.ent_m.clear();
   p.ent_ysh.clear();
   p.max_ent = 0;
@@ -447,6 +448,11 @@ int build_plan(const dgfs_plan_desc* d, Plan& p) {
         }
       }
       tk.n_grp = int(p.groups.size()) - tk.grp_off;
+      tk.face_off = int(p.faces.size());
+      for (size_t k = 0; k < ent.size(); ++k)
+        for (int kind = 0; kind < 2; ++kind)
+          if (p.sigma[3 * size_t(ent[k].first) + kind] != 0.0) p.faces.push_back(2 * int(k) + kind);
+      tk.n_face = int(p.faces.size()) - tk.face_off;
       for (size_t k = 0; k < ent.size(); ++k) {
         const auto& e = ent[k];
         p.ent_w.push_back(e.second);
@@ -535,29 +541,57 @@ int upload_plan(Plan& p) {
     }
   // phase factors exp(i pi shift_d k / L) per task, radial node, entry, role, axis
   const int NT = int(p.tasks.size());
-  const size_t nph = size_t(NT) * NR * p.max_ent * 2 * 3 * N;
-  std::vector<std::complex<double>> ph(nph, std::complex<double>(0.0, 0.0));
-  for (int t = 0; t < NT; ++t) {
+  auto phase_of = [&](int t, int q, int e, int role, int ax, int n) {
     const TaskDesc& tk = p.tasks[t];
     const double mi = p.mass[tk.i], mj = p.mass[tk.j];
     const double ci = mi / (mi + mj), cj = mj / (mi + mj);
-    for (int q = 0; q < NR; ++q)
-      for (int e = 0; e < tk.n_ent; ++e) {
-        const double* sg = &p.sigma[3 * p.ent_sigma[tk.ent_off + e]];
-        const double rq = rho_of(tk.out0, q);
-        for (int role = 0; role < 2; ++role) {
-          const double c = role == 0 ? rq * cj : -rq * ci;
-          for (int ax = 0; ax < 3; ++ax) {
-            const double sh = c * sg[ax];
-            std::complex<double>* dst = &ph[((((size_t(t) * NR + q) * p.max_ent + e) * 2 + role) * 3 + ax) * N];
-            for (int n = 0; n < N; ++n) {
-              const double arg = kPi * sh * centred_mode(n, N) / p.L;
-              dst[n] = std::complex<double>(std::cos(arg), std::sin(arg));
-            }
+    const double rq = rho_of(tk.out0, q);
+    const double c = role == 0 ? rq * cj : -rq * ci;
+    const double sh = c * p.sigma[3 * size_t(p.ent_sigma[tk.ent_off + e]) + ax];
+    const double arg = kPi * sh * centred_mode(n, N) / p.L;
+    return std::complex<double>(std::cos(arg), std::sin(arg));
+  };
+  std::vector<std::complex<double>> ph;
+  if (p.vss || p.precision == DGFS_BF16X3) {
+    // [task][rho][entry][role][axis][N]
+    ph.assign(size_t(NT) * NR * p.max_ent * 2 * 3 * N, std::complex<double>(0.0, 0.0));
+    for (int t = 0; t < NT; ++t)
+      for (int q = 0; q < NR; ++q)
+        for (int e = 0; e < p.tasks[t].n_ent; ++e)
+          for (int role = 0; role < 2; ++role)
+            for (int ax = 0; ax < 3; ++ax)
+              for (int n = 0; n < N; ++n)
+                ph[((((size_t(t) * NR + q) * p.max_ent + e) * 2 + role) * 3 + ax) * N + n] = phase_of(t, q, e, role, ax, n);
+  } else {
+    // [task][rho][entry] blocks of the VHS kernel: x [N][role], y [N][role], z [role][N/2], then
+    // per role (cz, tz) and per role (tx, ty), c + i t the phase of the unpaired mode N/2; the x
+    // and y entries of that mode keep c alone; role 1's z phases, cz and tz carry the weight w_e
+    const size_t PB = 5 * size_t(N) + 4;
+    const int h = N / 2;
+    ph.assign(size_t(NT) * NR * p.max_ent * PB, std::complex<double>(0.0, 0.0));
+    for (int t = 0; t < NT; ++t)
+      for (int q = 0; q < NR; ++q)
+        for (int e = 0; e < p.tasks[t].n_ent; ++e) {
+          std::complex<double>* blk = &ph[((size_t(t) * NR + q) * p.max_ent + e) * PB];
+          for (int role = 0; role < 2; ++role) {
+            const double w = role == 0 ? 1.0 : p.ent_w[p.tasks[t].ent_off + e];
+            double tu[2];
+            for (int ax = 0; ax < 2; ++ax)
+              for (int n = 0; n < N; ++n) {
+                std::complex<double> z = phase_of(t, q, e, role, ax, n);
+                if (n == h) {
+                  tu[ax] = z.imag();
+                  z = z.real();
+                }
+                blk[size_t(ax) * 2 * N + 2 * n + role] = z;
+              }
+            for (int n = 0; n < h; ++n) blk[4 * N + role * h + n] = w * phase_of(t, q, e, role, 2, n);
+            blk[5 * N + role] = w * phase_of(t, q, e, role, 2, h);
+            blk[5 * N + 2 + role] = std::complex<double>(tu[0], tu[1]);
           }
         }
-      }
   }
+  const size_t nph = ph.size();
   std::vector<float> phf;
   std::vector<double> phd;
   std::vector<uint16_t> mats;
@@ -720,6 +754,7 @@ int upload_plan(Plan& p) {
   if ((rc = upload(p, p.tasks.data(), p.tasks.size(), (void**)&p.d_tasks, total))) return rc;
   if ((rc = upload(p, p.groups.data(), p.groups.size(), (void**)&p.d_groups, total))) return rc;
   if ((rc = upload(p, p.ent_ysh.data(), p.ent_ysh.size(), (void**)&p.d_ent_ysh, total))) return rc;
+  if (!p.faces.empty() && (rc = upload(p, p.faces.data(), p.faces.size(), (void**)&p.d_faces, total))) return rc;
   if (!mats.empty() && (rc = upload(p, mats.data(), mats.size(), (void**)&p.d_mats, total))) return rc;
   if (p.f32io()) {
     if ((rc = upload(p, phf.data(), phf.size(), &p.d_phase, total))) return rc;
@@ -757,7 +792,7 @@ void free_plan(Plan& p) {
   void* ptrs[] = {p.d_Fw,      p.d_Gm,      p.d_ent_w,   p.d_phase, p.d_tasks, p.d_groups, p.d_Fv,
                   p.d_scratch_raw, p.d_stage_f, p.d_stage_Q, p.d_cons, p.d_kappa, p.d_Qfull, p.d_ent_m,
                   p.d_counter, p.d_rk,      p.d_ent_ysh, p.d_Fwf,    p.d_Fvf,   p.d_Gmf,   p.d_mats,
-                  p.d_scratch2_raw, p.d_counter2};
+                  p.d_scratch2_raw, p.d_counter2, p.d_faces};
   if (p.home) {
     for (void* q : ptrs)
       if (q) cudaFreeAsync(q, p.home);
@@ -799,6 +834,7 @@ void free_plan(Plan& p) {
   p.d_counter = nullptr;
   p.d_rk = nullptr;
   p.d_mats = nullptr;
+  p.d_faces = nullptr;
 }
 
 }  // namespace dgfs

@@ -1,0 +1,629 @@
+// Persistent collision kernel for VHS plans (alpha = 1): one thread-block cluster per work item
+// (node b, task), real transforms throughout.
+//
+// Only Re Q is wanted, and for VHS the gain weight F(k, rho) and the loss weight G^-(k) are real
+// and even in k, so Q_ij = IDFT(sum_rho w F DFT(Re P_rho)) - f_i IDFT(G^- f_hat_j) holds with the
+// real part of the products alone:
+//
+//     Re P = sum_e w_e (Re a_e Re b_e - Im a_e Im b_e).
+//
+// f is real, so the shifted copies a_e, b_e would be real too but for the unpaired modes at index
+// N/2 of an axis: there the phase e^{i theta k} has no conjugate partner and leaves
+// c + i t = cos - i sin of theta N / 2.  Write the shift along one axis as R + i t Pi, R the
+// real shift (phase c at the unpaired mode) and Pi the projection on that mode, an alternating
+// sequence.  The product over the three axes gives
+//
+//     Re a = RxRyRz f - ty tz RxPyPz f - tx tz PxRyPz f - tx ty PxPyRz f
+//     Im a = tx PxRyRz f + ty RxPyRz f + tz RxRyPz f - tx ty tz PxPyPz f.
+//
+// Every term but the first lives on faces or edges of the mode cube, so a shifted copy costs one
+// real 3D transform and two real 2D ones (the faces k_x = N/2 and k_y = N/2; the face k_z = N/2
+// falls out of the y pass, see below) instead of a complex 3D transform: half the arithmetic and
+// half the workspace.
+//
+// Layouts.  A spectrum keeps columns c = 0..N/2-1 of the z modes; column 0 holds
+// X(k_z = 0) + i X(k_z = N/2) ("C form": every x and y pass is linear and maps each part to
+// itself, so the pair travels as one complex line).  Rows of N complex values hold two such half
+// rows: role 0 (species i, shift +) and role 1 (species j, shift -).  After the inverse y pass
+// column 0 is (a(k_z = 0), a(k_z = N/2)), two real numbers.  The product's spectrum splits column
+// 0 over k_y instead ("N form", row r of column 0: r = 1..N/2-1 is (k_y = r, k_z = 0), N/2 + r is
+// (k_y = r, k_z = N/2), row 0 holds X(0,0) + i X(N/2,0) and row N/2 holds X(0,N/2) + i X(N/2,N/2)),
+// since there the weights of the two parts differ.
+//
+// Per radial node the phases run as a pipeline over sigma_x groups: phase 0 transforms the faces of
+// all entries and runs step A of group 0; phase k runs step A of group k and step B of group
+// k - 1; one cluster barrier each.
+//   step A  x pass of both roles' half spectra (one thread per pencil, coalesced)
+//   step B  per plane x and entry: y phases, y pass of N/2 columns of either role (one line per
+//           thread), transpose through shared memory, z phases and the real z transform of both
+//           roles (one row per thread), and the product into P, N real values per thread
+//   step C  after the last group: P -> spectrum, Q_hat_ij += F_ij P_hat (and Q_hat_ji for a cross pair)
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "dgfs_internal.h"
+#include "group_sync.cuh"
+#include "real_line.cuh"
+
+namespace dgfs {
+
+// compile-time launch shape per (precision, N): cluster size, plane groups per CTA, CTAs per SM
+template <typename T, int N> struct VShape;
+#define DGFS_SHAPE3(TT, NN, CC, GG, MB)      \
+  template <> struct VShape<TT, NN> {        \
+    static constexpr int cluster = CC;       \
+    static constexpr int groups = GG;        \
+    static constexpr int min_blocks = MB;    \
+  };
+#define DGFS_SHAPE(TT, NN, CC, GG) DGFS_SHAPE3(TT, NN, CC, GG, 1)
+#include "vhs_shapes.h"
+#undef DGFS_SHAPE
+#undef DGFS_SHAPE3
+
+template <typename T, int N>
+struct VGeo {
+  static constexpr int h = N / 2;
+  static constexpr int N2 = N * N, HN2 = N * h;
+  static constexpr size_t N3 = size_t(N) * N * N, HN3 = size_t(N) * HN2;
+  static constexpr int PITCH = N + 1;
+  static constexpr int CL = VShape<T, N>::cluster;
+  static constexpr int GP = VShape<T, N>::groups;
+  static constexpr int MINB = VShape<T, N>::min_blocks;
+  static constexpr int THREADS = GP * N;
+  static constexpr int PLANES = N / CL;  // planes, and rows of pencils, per CTA
+  static_assert(N % CL == 0 && PLANES % GP == 0, "planes must split evenly over the cluster and its plane groups");
+  // P of a plane stays in the row's thread (FP64 N = 48: in shared memory, its line alone fills
+  // the registers); with one plane per group it lives there for the whole radial node, otherwise
+  // it is parked in the workspace between sigma_x groups
+  static constexpr bool PSM = sizeof(T) == 8 && N >= 48;
+  static constexpr bool KEEP = PLANES == GP;
+  // shared memory per group: one padded plane, the entry's row of the k_y face, P if PSM
+  static constexpr size_t GROUP_BYTES = (size_t(N) * PITCH + N) * sizeof(C<T>) + (PSM ? N2 * sizeof(T) : 0);
+  static constexpr size_t SMEM = GP * GROUP_BYTES;
+  // phase block of an entry (complex values): x [N][role], y [N][role], z [role][h] (role 1 times
+  // w_e), then per role (cz, tz) (role 1 times w_e) and per role (tx, ty)
+  static constexpr int PB = 5 * N + 4;
+  // workspace per cluster (complex values): f_hat of both species, two buffers of x-passed half
+  // spectra of both roles, P_hat, two gain accumulators, parked P; then per entry the two faces
+  // and the k_x-face's k_z = N/2 line
+  static constexpr size_t SLOT = 3 * N3 + 3 * HN3 + (KEEP ? 0 : HN3);
+  static constexpr size_t FACE = 2 * N2 + N;
+};
+
+// v[n] *= ph[2 n]: the shared phase e^{i theta k} of a line; mode 0 has phase 1 and the unpaired
+// mode N/2 the real factor c
+template <typename T, int N>
+__device__ __forceinline__ void shift_line(C<T> (&v)[N], const C<T>* ph) {
+#pragma unroll
+  for (int n = 1; n < N; ++n) v[n] = n == N / 2 ? scale<T>(v[n], ph[2 * n].x) : cmul<T>(v[n], ph[2 * n]);
+}
+
+// Real rows of both roles of a plane.  In FP32 the roles run packed, one register pair per value:
+// the two transforms share every twiddle, so one instruction serves both.
+template <typename T, int N> struct Rows {
+  T a[N], b[N];
+  // a_z, b_z
+  __device__ __forceinline__ C<T> at(int z) const { return mk<T>(a[z], b[z]); }
+};
+template <int N> struct Rows<float, N> {
+  F2 v[N];
+  __device__ __forceinline__ float2 at(int z) const { return unpack2(v[z]); }
+};
+
+// z transform of a row of both roles (row: role 0, row + N/2: role 1) with the z phases phz (null:
+// none), x0 and xh the values (role 0, role 1) of modes 0 and N/2
+template <int N>
+__device__ __forceinline__ void rows_c2r(const float2* row, const float2* phz, float2 x0, float2 xh, Rows<float, N>& y) {
+  constexpr int h = N / 2;
+  C2 x[h];
+#pragma unroll
+  for (int k = 1; k < h; ++k) {
+    float2 a = row[k], b = row[h + k];
+    if (phz != nullptr) {
+      a = cmul<float>(a, phz[k]);
+      b = cmul<float>(b, phz[h + k]);
+    }
+    x[k].x = pack2(a.x, b.x);
+    x[k].y = pack2(a.y, b.y);
+  }
+  c2r_line<F2, N>(x, pack2(x0.x, x0.y), pack2(xh.x, xh.y), y.v);
+}
+template <int N>
+__device__ __forceinline__ void rows_c2r(const double2* row, const double2* phz, double2 x0, double2 xh,
+                                         Rows<double, N>& y) {
+  constexpr int h = N / 2;
+  double2 x[h];
+#pragma unroll
+  for (int k = 1; k < h; ++k) x[k] = phz != nullptr ? cmul<double>(row[k], phz[k]) : row[k];
+  c2r_line<double, N>(x, x0.x, xh.x, y.a);
+#pragma unroll
+  for (int k = 1; k < h; ++k) x[k] = phz != nullptr ? cmul<double>(row[h + k], phz[h + k]) : row[h + k];
+  c2r_line<double, N>(x, x0.y, xh.y, y.b);
+}
+
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+// (s u + t w) + m in both halves
+__device__ __forceinline__ float2 face_sum(float s, float2 u, float t, float2 w, float2 m) {
+  return unpack2(fma2(pack2(s, s), pack2(u.x, u.y), fma2(pack2(t, t), pack2(w.x, w.y), pack2(m.x, m.y))));
+}
+__device__ __forceinline__ double2 face_sum(double s, double2 u, double t, double2 w, double2 m) {
+  return make_double2(fma(s, u.x, fma(t, w.x, m.x)), fma(s, u.y, fma(t, w.y, m.y)));
+}
+__device__ __forceinline__ float2 mul_each(float2 s, float2 v) { return unpack2(pack2(s.x, s.y) * pack2(v.x, v.y)); }
+__device__ __forceinline__ double2 mul_each(double2 s, double2 v) { return make_double2(s.x * v.x, s.y * v.y); }
+
+template <typename T, int N>
+__global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_kernel(const KernelParams p) {
+  using G = VGeo<T, N>;
+  using CT = C<T>;
+  constexpr int h = G::h, N2 = G::N2, HN2 = G::HN2, CL = G::CL, GP = G::GP, NT = G::THREADS, PITCH = G::PITCH;
+  constexpr int PB = G::PB;
+  constexpr size_t N3 = G::N3, HN3 = G::HN3;
+
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tid = threadIdx.x;
+  const int grp = tid / N;  // plane group
+  const int t = tid % N;    // line within the group: column (role, c) in y passes, row in z passes
+  const int role = t / h, c = t % h;
+  unsigned char* const gsm = smem_raw + size_t(grp) * G::GROUP_BYTES;
+  CT* const tb = reinterpret_cast<CT*>(gsm);  // padded plane; the pad column of rows 0, 1 carries a corner value
+  CT* const uyb = tb + N * PITCH;             // the entry's row of the k_y face
+  T* const pb = reinterpret_cast<T*>(uyb + N);
+  CT* const phs = reinterpret_cast<CT*>(smem_raw + G::SMEM);  // phase block of the current (task, rho)
+  const bool ph_smem = p.phase_smem != 0;
+
+  const int rank = CL == 1 ? 0 : int(cluster_rank());
+  const int cid = blockIdx.x / CL;
+  CT* const scr = reinterpret_cast<CT*>(p.scratch) + size_t(cid) * p.slot;
+  CT* const FS = scr;               // f_hat [k_x][k_y][species 0 | 1][c]
+  CT* const H0 = FS + N3;           // x-passed half spectra [x][k_y][role][c], two buffers
+  CT* const PV = H0 + 2 * N3;       // product spectrum [x][row][c] (N form)
+  CT* const QA = PV + HN3;          // gain accumulators [k_x][row][c] (N form)
+  CT* const QB = QA + HN3;
+  T* const PS = reinterpret_cast<T*>(QB + HN3);  // parked P [x][z][y]
+  CT* const FC = scr + G::SLOT;     // faces per entry: X [z][y], Y [x][z], line [y]; values (role 0, role 1)
+  const int plane0 = rank * G::PLANES;
+  const T inv_n3 = T(1) / T(N3);
+
+  // Work items (node, task) come from a counter: thread 0 of the rank-0 CTA takes the next item
+  // after the first barrier of the current one, when every CTA has read the current value.
+  __shared__ int s_next_item;
+  const int n_items = p.batch * p.n_tasks;
+  if (rank == 0 && tid == 0) s_next_item = int(atomicAdd(p.work_counter, 1u));
+  cluster_sync<CL>();
+  for (int item = CL == 1 ? s_next_item : ld_rank0(&s_next_item); item < n_items;
+       item = CL == 1 ? s_next_item : ld_rank0(&s_next_item)) {
+    const int b = item / p.n_tasks;
+    const int task = item % p.n_tasks;
+    const TaskDesc tk = p.tasks[task];
+    const T* fb = reinterpret_cast<const T*>(p.f) + size_t(b) * p.s * N3;
+    const bool self = tk.i == tk.j;
+
+    // ---- step 0: f_hat = N^-3 DFT(f) of species i (and j), half spectra in C form -----------
+    for (int xl = grp; xl < G::PLANES; xl += GP) {
+      const int x = plane0 + xl;
+      for (int sp = 0; sp < (self ? 1 : 2); ++sp) {
+        const T* src = fb + size_t(sp == 0 ? tk.i : tk.j) * N3 + size_t(x) * N2 + t * N;
+        T y[N];
+        CT z[h];
+#pragma unroll
+        for (int n = 0; n < N; ++n) y[n] = __ldg(src + n);
+        r2c_line<T, N>(y, z);
+#pragma unroll
+        for (int k = 0; k < h; ++k) tb[t * PITCH + sp * h + k] = z[k];
+      }
+      group_sync<N, GP>();
+      if (!self || role == 0) {
+        CT v[N];
+#pragma unroll
+        for (int r = 0; r < N; ++r) v[r] = tb[r * PITCH + t];
+        line_fft<T, N, -1>(v);
+#pragma unroll
+        for (int r = 0; r < N; ++r) st2<T>(FS + size_t(x) * N2 + r * N + t, v[r]);
+      }
+      group_sync<N, GP>();
+    }
+    cluster_sync<CL>();
+    if (rank == 0 && tid == 0) s_next_item = int(atomicAdd(p.work_counter, 1u));
+    if (!self || role == 0) {
+      for (int xl = grp; xl < G::PLANES; xl += GP) {
+        CT* const vol = FS + (plane0 + xl) * N + t;
+        CT v[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) v[n] = ld2<T>(vol + n * N2);
+        line_fft<T, N, -1>(v);
+#pragma unroll
+        for (int n = 0; n < N; ++n) st2<T>(vol + n * N2, scale<T>(v[n], inv_n3));
+      }
+    }
+    cluster_sync<CL>();
+    const CT* const Fr = FS + (self ? c : t);     // this thread's column of f_hat
+    const CT fe = ld2<T>(Fr + h * N2 + h * N);    // its value on the edge k_x = k_y = N/2
+
+    // ---- gain ---------------------------------------------------------------------------------
+    T P[G::PSM ? 1 : N];
+    for (int q = 0; q < p.n_rho; ++q) {
+      const CT* const phq = static_cast<const CT*>(p.phase) + (size_t(task) * p.n_rho + q) * p.max_ent * PB;
+      if (ph_smem) {
+        for (int u = tid; u < tk.n_ent * PB; u += NT) phs[u] = __ldg(phq + u);
+        __syncthreads();
+      }
+      const CT* const phb = ph_smem ? phs : phq;
+
+      // faces of the entries whose shift along the face's axis is not zero, spread over the
+      // cluster's CTAs first; code 2 e + kind.  kind 0: k_x = N/2 (y and z shifted), kind 1:
+      // k_y = N/2 (x and z shifted)
+      for (int f0 = 0; f0 < tk.n_face; f0 += CL * GP) {
+        // groups that share a barrier run the same number of rounds: one without a face of its own
+        // repeats the last and stores nothing
+        const int f = f0 + grp * CL + rank;
+        const bool live = f < tk.n_face;
+        if (N % 32 == 0 && !live) break;
+        const int code = p.faces[tk.face_off + (live ? f : tk.n_face - 1)];
+        const int e = code >> 1, kind = code & 1;
+        const CT* const pe = phb + e * PB;
+        CT* const fc = FC + size_t(e) * G::FACE;
+        {
+          const CT* const src = Fr + (kind == 0 ? h * N2 : h * N);
+          const int step = kind == 0 ? N : N2;
+          CT v[N];
+#pragma unroll
+          for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + r * step);
+          shift_line<T, N>(v, pe + (kind == 0 ? 2 * N : 0) + role);
+          line_fft<T, N, +1>(v);
+          group_sync<N, GP>();
+#pragma unroll
+          for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
+          group_sync<N, GP>();
+        }
+        const CT* const row = tb + t * PITCH;
+        const CT cta = pe[5 * N], ctb = pe[5 * N + 1], txa = pe[5 * N + 2], txb = pe[5 * N + 3];
+        const CT a0 = row[0], b0 = row[h];
+        Rows<T, N> y;
+        rows_c2r<N>(row, pe + 4 * N, mk<T>(a0.x, pe[4 * N + h].x * b0.x), mk<T>(cta.x * a0.y, ctb.x * b0.y), y);
+        const CT sc = kind == 0 ? mk<T>(txa.x, txb.x) : mk<T>(txa.y, txb.y);
+        if (!live) {
+        } else if (kind == 0) {
+#pragma unroll
+          for (int z = 0; z < N; ++z) st2<T>(fc + z * N + t, mul_each(sc, y.at(z)));
+          st2<T>(fc + 2 * N2 + t, mk<T>(sc.x * a0.y, sc.y * b0.y));
+        } else {
+#pragma unroll
+          for (int z = 0; z < N; ++z) st2<T>(fc + N2 + t * N + z, mul_each(sc, y.at(z)));
+        }
+      }
+
+      for (int k = 0; k <= tk.n_grp; ++k) {
+        // step A of group k: x pass of this thread's pencils with the group's x phases
+        if (k < tk.n_grp) {
+          const GroupDesc gd = p.groups[tk.grp_off + k];
+          CT* const dst = H0 + size_t(k & 1) * N3;
+          const CT* const phx = phb + gd.first * PB + role;
+          for (int xl = grp; xl < G::PLANES; xl += GP) {
+            const int r = plane0 + xl;
+            CT v[N];
+#pragma unroll
+            for (int n = 0; n < N; ++n) v[n] = ld2<T>(Fr + n * N2 + r * N);
+            shift_line<T, N>(v, phx);
+            line_fft<T, N, +1>(v);
+#pragma unroll
+            for (int n = 0; n < N; ++n) st2<T>(dst + n * N2 + r * N + t, v[n]);
+          }
+        }
+        // step B of group k - 1: this group's planes
+        if (k > 0) {
+          const GroupDesc gd = p.groups[tk.grp_off + k - 1];
+          const CT* const src = H0 + size_t((k - 1) & 1) * N3;
+          const bool fresh = k == 1, last = k == tk.n_grp;
+          for (int xl = grp; xl < G::PLANES; xl += GP) {
+            const int x = plane0 + xl;
+            const T sgx = (x & 1) ? T(-1) : T(1), sgy = (t & 1) ? T(-1) : T(1);
+            if constexpr (G::PSM) {
+              if (fresh || !G::KEEP) {
+#pragma unroll
+                for (int z = 0; z < N; ++z) pb[z * N + t] = fresh ? T(0) : __ldcg(PS + size_t(x) * N2 + z * N + t);
+              }
+            } else {
+              if (fresh || !G::KEEP) {
+#pragma unroll
+                for (int z = 0; z < N; ++z) P[z] = fresh ? T(0) : __ldcg(PS + size_t(x) * N2 + z * N + t);
+              }
+            }
+            for (int e = gd.first; e < gd.first + gd.count; ++e) {
+              const CT* const pe = phb + e * PB;
+              const CT* const fc = FC + size_t(e) * G::FACE;
+              // a shift of zero along an axis has no face there
+              const CT txa = pe[5 * N + 2], txb = pe[5 * N + 3];
+              const bool has_x = txa.x != T(0) || txb.x != T(0), has_y = txa.y != T(0) || txb.y != T(0);
+              const CT uy = has_y ? ld2<T>(fc + N2 + x * N + t) : mk<T>(0, 0);
+              const CT en = has_x ? ld2<T>(fc + 2 * N2 + t) : mk<T>(0, 0);
+              {
+                CT v[N];
+#pragma unroll
+                for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + size_t(x) * N2 + r * N + t);
+                const T corner = v[h].y;  // of column 0: f on the edge k_y = k_z = N/2
+                shift_line<T, N>(v, pe + 2 * N + role);
+                const CT txy = role == 0 ? txa : txb;
+                const T w = sgx * txy.x * txy.y;
+                v[h] = mk<T>(v[h].x - w * fe.x, v[h].y - w * fe.y);
+                line_fft<T, N, +1>(v);
+                group_sync<N, GP>();  // the previous entry's rows have been read
+#pragma unroll
+                for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
+                uyb[t] = uy;
+                if (c == 0) tb[role * PITCH + N] = mk<T>(corner, T(0));
+                group_sync<N, GP>();
+              }
+              const CT* const row = tb + t * PITCH;
+              const CT cta = pe[5 * N], ctb = pe[5 * N + 1];
+              const CT a0 = row[0], b0 = row[h];
+              const CT m = mk<T>(cta.y * a0.y, ctb.y * b0.y);
+              Rows<T, N> y;
+              rows_c2r<N>(row, pe + 4 * N, mk<T>(a0.x, pe[4 * N + h].x * b0.x),
+                          mk<T>(cta.x * a0.y - cta.y * (sgx * en.x + sgy * txa.y * tb[N].x),
+                                ctb.x * b0.y - ctb.y * (sgx * en.y + sgy * txb.y * tb[PITCH + N].x)),
+                          y);
+#pragma unroll
+              for (int z = 0; z < N; ++z) {
+                const CT ux = has_x ? ld2<T>(fc + z * N + t) : mk<T>(0, 0);
+                const CT im = face_sum(sgx, ux, sgy, uyb[z], (z & 1) ? mk<T>(-m.x, -m.y) : m);
+                const CT re = y.at(z);
+                if constexpr (G::PSM) pb[z * N + t] = fma_(-im.x, im.y, fma_(re.x, re.y, pb[z * N + t]));
+                else P[z] = fma_(-im.x, im.y, fma_(re.x, re.y, P[z]));
+              }
+            }
+            if (last) {
+              group_sync<N, GP>();
+              {
+                CT z[h];
+                T y[N];
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                  if constexpr (G::PSM) y[n] = pb[n * N + t]; else y[n] = P[n];
+                }
+                r2c_line<T, N>(y, z);
+#pragma unroll
+                for (int kz = 0; kz < h; ++kz) tb[t * PITCH + kz] = z[kz];
+              }
+              group_sync<N, GP>();
+              if (role == 0) {
+                CT v[N];
+#pragma unroll
+                for (int r = 0; r < N; ++r) v[r] = tb[r * PITCH + t];
+                line_fft<T, N, -1>(v);
+                CT* const dst = PV + size_t(x) * HN2 + c;
+                if (c != 0) {
+#pragma unroll
+                  for (int r = 0; r < N; ++r) st2<T>(dst + r * h, v[r]);
+                } else {  // C form -> N form
+                  st2<T>(dst, mk<T>(v[0].x, v[h].x));
+                  st2<T>(dst + h * h, mk<T>(v[0].y, v[h].y));
+#pragma unroll
+                  for (int r = 1; r < h; ++r) {
+                    const CT m = conj_<T>(v[N - r]);
+                    const CT d = sub<T>(v[r], m);
+                    st2<T>(dst + r * h, scale<T>(add<T>(v[r], m), T(0.5)));
+                    st2<T>(dst + (h + r) * h, mk<T>(T(0.5) * d.y, T(-0.5) * d.x));
+                  }
+                }
+              }
+            } else if constexpr (!G::KEEP) {
+#pragma unroll
+              for (int z = 0; z < N; ++z) {
+                T val;
+                if constexpr (G::PSM) val = pb[z * N + t]; else val = P[z];
+                __stcg(PS + size_t(x) * N2 + z * N + t, val);
+              }
+            }
+          }
+        }
+        cluster_sync<CL>();
+      }
+
+      // step C: x pass of the product spectrum, weights, accumulation
+      for (int u = tid; u < G::PLANES * h; u += NT) {
+        const int r = plane0 + u / h, cc = u % h;
+        const size_t pp = size_t(r) * h + cc;
+        CT v[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) v[n] = ld2<T>(PV + n * HN2 + pp);
+        line_fft<T, N, -1>(v);
+        // modes of the pencil (N form): column 0 holds k_z = 0 in rows 1..N/2-1 and k_z = N/2 above
+        // them; rows 0 and N/2 hold two real pencils, k_y = 0 and N/2, as one
+        const bool pair_row = cc == 0 && (r == 0 || r == h);
+        const int ky = cc == 0 && r >= h ? r - h : r;
+        const int kz = cc == 0 && r >= h ? h : cc;
+        for (int o = 0; o < 2; ++o) {
+          const int pair = o == 0 ? tk.out0 : tk.out1;
+          if (pair < 0) break;
+          const T* const Fw = static_cast<const T*>(p.Fw) + (size_t(pair) * p.n_rho + q) * N3 + ky * N + kz;
+          CT* const acc = (o == 0 ? QA : QB) + pp;
+          if (!pair_row) {
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+              CT val = scale<T>(v[n], __ldg(Fw + n * N2));
+              if (q > 0) val = add<T>(val, ld2<T>(acc + n * HN2));
+              st2<T>(acc + n * HN2, val);
+            }
+          } else {
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+              const T fa = __ldg(Fw + n * N2), fh = __ldg(Fw + n * N2 + h * N);
+              const T fp = T(0.5) * (fa + fh), fm = T(0.5) * (fa - fh);
+              const CT m = v[(N - n) % N];
+              CT val = mk<T>(fp * v[n].x + fm * m.x, fp * v[n].y - fm * m.y);
+              if (q > 0) val = add<T>(val, ld2<T>(acc + n * HN2));
+              st2<T>(acc + n * HN2, val);
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+
+    // ---- finish: Q_ij = IDFT(Q_hat) - f_i IDFT(G^- f_hat_j); role 0 the gain, role 1 the loss ----
+    for (int o = 0; o < 2; ++o) {
+      const int pair = o == 0 ? tk.out0 : tk.out1;
+      if (pair < 0) break;
+      const int io = o == 0 ? tk.i : tk.j;
+      const int jo = o == 0 ? tk.j : tk.i;
+      const CT* const acc = o == 0 ? QA : QB;
+      const CT* const Fj = FS + (jo == tk.i ? 0 : h);
+      const T* const Gm = static_cast<const T*>(p.Gm) + size_t(pair) * N3;
+      for (int xl = grp; xl < G::PLANES; xl += GP) {
+        const int r = plane0 + xl;
+        CT v[N];
+        if (role == 0) {
+#pragma unroll
+          for (int n = 0; n < N; ++n) v[n] = ld2<T>(acc + n * HN2 + r * h + c);
+        } else if (c != 0) {
+#pragma unroll
+          for (int n = 0; n < N; ++n) v[n] = scale<T>(ld2<T>(Fj + n * N2 + r * N + c), __ldg(Gm + n * N2 + r * N + c));
+        } else {  // C form: the two parts of column 0 have weights of their own
+          const int rm = r == 0 ? 0 : N - r;
+#pragma unroll
+          for (int n = 0; n < N; ++n) {
+            const T ga = __ldg(Gm + n * N2 + r * N), gh = __ldg(Gm + n * N2 + r * N + h);
+            const T gp = T(0.5) * (ga + gh), gm = T(0.5) * (ga - gh);
+            const CT a = ld2<T>(Fj + n * N2 + r * N), m = ld2<T>(Fj + ((N - n) % N) * N2 + rm * N);
+            v[n] = mk<T>(gp * a.x + gm * m.x, gp * a.y - gm * m.y);
+          }
+        }
+        line_fft<T, N, +1>(v);
+#pragma unroll
+        for (int n = 0; n < N; ++n) st2<T>(H0 + n * N2 + r * N + t, v[n]);
+      }
+      cluster_sync<CL>();
+      T* const Qout = reinterpret_cast<T*>(p.Q) + ((size_t(b) * p.s + io) * p.s + jo) * N3;
+      const T* const fi = fb + size_t(io) * N3;
+      for (int xl = grp; xl < G::PLANES; xl += GP) {
+        const int x = plane0 + xl;
+        const CT* const src = H0 + size_t(x) * N2;
+        {
+          CT v[N];
+          if (t != 0) {
+#pragma unroll
+            for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + r * N + t);
+          } else {  // N form -> C form
+            const CT a = ld2<T>(src), d = ld2<T>(src + h * N);
+            v[0] = mk<T>(a.x, d.x);
+            v[h] = mk<T>(a.y, d.y);
+#pragma unroll
+            for (int r = 1; r < h; ++r) {
+              const CT al = ld2<T>(src + r * N), be = ld2<T>(src + (h + r) * N);
+              v[r] = mk<T>(al.x - be.y, al.y + be.x);
+              v[N - r] = mk<T>(al.x + be.y, be.x - al.y);
+            }
+          }
+          line_fft<T, N, +1>(v);
+          group_sync<N, GP>();
+#pragma unroll
+          for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
+          group_sync<N, GP>();
+        }
+        const CT g0 = tb[t * PITCH], l0 = tb[t * PITCH + h];
+        Rows<T, N> y;
+        rows_c2r<N>(tb + t * PITCH, static_cast<const CT*>(nullptr), mk<T>(g0.x, l0.x), mk<T>(g0.y, l0.y), y);
+        group_sync<N, GP>();
+        // stage the row through shared memory for a coalesced store
+        T* const rb = reinterpret_cast<T*>(tb);
+#pragma unroll
+        for (int z = 0; z < N; ++z) {
+          const CT gl = y.at(z);
+          rb[t * PITCH + z] = gl.x - __ldg(fi + size_t(x) * N2 + t * N + z) * gl.y;
+        }
+        group_sync<N, GP>();
+#pragma unroll
+        for (int r = 0; r < N; ++r) Qout[size_t(x) * N2 + r * N + t] = rb[r * PITCH + t];
+        group_sync<N, GP>();
+      }
+      cluster_sync<CL>();
+    }
+  }
+  // no CTA leaves while another may still read its shared memory (the last item index)
+  if constexpr (CL > 1) cluster_sync<CL>();
+}
+
+template <typename T, int N>
+int vhs_configure_impl(Plan& pl) {
+  using G = VGeo<T, N>;
+  auto kern = vhs_kernel<T, N>;
+  // the phase block of the current (task, rho) goes to shared memory while MINB CTAs still fit
+  const size_t ph_bytes = size_t(pl.max_ent) * G::PB * sizeof(C<T>);
+  const int ph_mode = G::MINB * (G::SMEM + ph_bytes + 2048) <= size_t(226) * 1024 ? 1 : 0;
+  const size_t smem = G::SMEM + (ph_mode ? ph_bytes : 0);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+    return DGFS_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = G::CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(G::CL);
+  cfg.blockDim = dim3(G::THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters <= 0) {
+    cudaGetLastError();
+    return DGFS_ERR_CUDA;
+  }
+  pl.shape.cluster = G::CL;
+  pl.shape.groups = G::GP;
+  pl.shape.threads = G::THREADS;
+  pl.shape.smem = smem;
+  pl.shape.phase_smem = ph_mode;
+  pl.shape.clusters = clusters;
+  pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
+  pl.scratch_bytes = size_t(clusters) * pl.shape.slot * sizeof(C<T>);
+  return DGFS_OK;
+}
+
+template <typename T, int N>
+int vhs_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
+  using G = VGeo<T, N>;
+  KernelParams kp;
+  kp.f = f;
+  kp.Q = Q;
+  kp.batch = batch;
+  kp.s = pl.s;
+  kp.n_tasks = int(pl.tasks.size());
+  kp.n_rho = pl.N_rho;
+  kp.max_ent = pl.max_ent;
+  kp.tasks = pl.d_tasks;
+  kp.groups = pl.d_groups;
+  kp.faces = pl.d_faces;
+  kp.phase = pl.d_phase;
+  kp.Fw = pl.d_Fwf ? static_cast<const void*>(pl.d_Fwf) : static_cast<const void*>(pl.d_Fw);
+  kp.Gm = pl.d_Gmf ? static_cast<const void*>(pl.d_Gmf) : static_cast<const void*>(pl.d_Gm);
+  kp.scratch = pl.scratch_of(ws);
+  kp.slot = pl.shape.slot;
+  kp.phase_smem = pl.shape.phase_smem;
+  kp.work_counter = pl.counter_of(ws);
+  const int items = batch * kp.n_tasks;
+  int limit = int(pl.shape.clusters * pl.shape.share);
+  if (limit < 1) limit = 1;
+  const int clusters = items < limit ? items : limit;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = G::CL;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(clusters * G::CL);
+  cfg.blockDim = dim3(G::THREADS);
+  cfg.dynamicSmemBytes = pl.shape.smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaMemsetAsync(kp.work_counter, 0, sizeof(unsigned), st) != cudaSuccess) return DGFS_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, vhs_kernel<T, N>, kp) != cudaSuccess) return DGFS_ERR_CUDA;
+  return DGFS_OK;
+}
+
+}  // namespace dgfs
