@@ -163,7 +163,7 @@ int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, i
   if (!p.d_scratch2_raw) {
     // the second workspace (with its guard blocks) and work counter of the pipelined chunks
     if (cudaMallocAsync(&p.d_scratch2_raw, p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
-        cudaMallocAsync((void**)&p.d_counter2, 256, p.home) != cudaSuccess) {
+        cudaMallocAsync((void**)&p.d_counter2, p.counter_bytes(), p.home) != cudaSuccess) {
       cudaGetLastError();
       if (p.d_scratch2_raw) cudaFreeAsync(p.d_scratch2_raw, p.home);
       if (p.d_counter2) cudaFreeAsync(p.d_counter2, p.home);
@@ -176,7 +176,7 @@ int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, i
     if (cudaMemsetAsync(p.d_scratch2_raw, dgfs::Plan::kGuardByte, dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
         cudaMemsetAsync(static_cast<char*>(p.d_scratch2) + p.scratch_bytes, dgfs::Plan::kGuardByte,
                         dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
-        cudaMemsetAsync(p.d_counter2, 0, 256, p.home) != cudaSuccess || cudaStreamSynchronize(p.home) != cudaSuccess) {
+        cudaMemsetAsync(p.d_counter2, 0, p.counter_bytes(), p.home) != cudaSuccess || cudaStreamSynchronize(p.home) != cudaSuccess) {
       cudaGetLastError();
       return DGFS_ERR_CUDA;
     }
@@ -293,7 +293,7 @@ int dgfs_plan_bytes(dgfs_plan plan, int batch, size_t* tables, size_t* workspace
   if (workspace)
     *workspace = p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes + (p.d_Qfull ? size_t(p.max_batch) * p.s * p.s * n3 * dgfs::real_size(p) : 0) +
                  (batch > 0 ? size_t(batch) * (p.s + output_pairs(p)) * n3 * dgfs::real_size(p) +
-                                  p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes + 256
+                                  p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes + p.counter_bytes()
                             : 0);
   return DGFS_OK;
 }

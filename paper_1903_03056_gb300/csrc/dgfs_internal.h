@@ -60,6 +60,8 @@ struct KernelParams {
   const void* Gm;         // [s*s][N^3]: G^(ij)-(k), in the plan's real type
   void* scratch;          // complex: [clusters][slot]
   size_t slot;            // complex values of workspace per cluster (VHS kernel)
+  void* parts;            // complex: [item][rho][N^3 / 2] products of split work items (VHS kernel)
+  int chunks;             // chunks a work item's radial nodes are split into (VHS kernel)
   int phase_smem;         // 1: the task's phase block of the current rho is staged in smem;
                           // 2: only its z phases are
   unsigned* work_counter; // next work item (reset to 0 before every launch)
@@ -96,6 +98,18 @@ struct LaunchShape {
   int clusters = 0;       // resident clusters (persistent grid)
   size_t slot = 0;        // complex values of workspace per cluster (VHS kernel)
   double share = 1.0;     // fraction of the resident clusters one launch may use
+};
+
+// words of the counter array: 0 the work counter, 1 the device status, then (VHS kernel) the
+// clusters that have left and, from kDoneWord on, the finished chunks of every split item
+constexpr int kExitWord = 2, kDoneWord = 64;
+// products (one radial node of one item) the VHS workspace holds per resident cluster
+constexpr int kPartsPerCluster = 6;
+
+// one launch shape of the VHS kernel
+struct VhsShape {
+  int threads = 0, phase_smem = 0, clusters = 0;
+  size_t smem = 0;
 };
 
 struct Plan {
@@ -159,6 +173,10 @@ struct Plan {
 
   // workspace
   LaunchShape shape;
+  VhsShape vhs[2];                 // VHS plans: the batch shape and the wide one (clusters = 0: none)
+  size_t part_off = 0;             // VHS plans: the split items' products in the workspace (complex values)
+  int part_slots = 0;              // and how many there is room for
+  size_t counter_bytes() const { return (kDoneWord + size_t(part_slots)) * sizeof(unsigned); }
   void* d_scratch = nullptr;       // kGuardBytes into d_scratch_raw
   void* d_scratch_raw = nullptr;   // guard | workspace | guard
   static constexpr size_t kGuardBytes = 4096;

@@ -540,9 +540,14 @@ int upload_plan(Plan& p) {
       }
     }
   // phase factors exp(i pi shift_d k / L) per task, radial node, entry, role, axis
-  const int NT = int(p.tasks.size());
+  // the VHS kernel takes its tasks in order of falling cost
+  const bool vhs = !p.vss && p.precision != DGFS_BF16X3;
+  std::vector<TaskDesc> tasks = p.tasks;
+  if (vhs)
+    std::stable_sort(tasks.begin(), tasks.end(), [](const TaskDesc& a, const TaskDesc& c) { return a.n_ent > c.n_ent; });
+  const int NT = int(tasks.size());
   auto phase_of = [&](int t, int q, int e, int role, int ax, int n) {
-    const TaskDesc& tk = p.tasks[t];
+    const TaskDesc& tk = tasks[t];
     const double mi = p.mass[tk.i], mj = p.mass[tk.j];
     const double ci = mi / (mi + mj), cj = mj / (mi + mj);
     const double rq = rho_of(tk.out0, q);
@@ -552,12 +557,12 @@ int upload_plan(Plan& p) {
     return std::complex<double>(std::cos(arg), std::sin(arg));
   };
   std::vector<std::complex<double>> ph;
-  if (p.vss || p.precision == DGFS_BF16X3) {
+  if (!vhs) {
     // [task][rho][entry][role][axis][N]
     ph.assign(size_t(NT) * NR * p.max_ent * 2 * 3 * N, std::complex<double>(0.0, 0.0));
     for (int t = 0; t < NT; ++t)
       for (int q = 0; q < NR; ++q)
-        for (int e = 0; e < p.tasks[t].n_ent; ++e)
+        for (int e = 0; e < tasks[t].n_ent; ++e)
           for (int role = 0; role < 2; ++role)
             for (int ax = 0; ax < 3; ++ax)
               for (int n = 0; n < N; ++n)
@@ -571,10 +576,10 @@ int upload_plan(Plan& p) {
     ph.assign(size_t(NT) * NR * p.max_ent * PB, std::complex<double>(0.0, 0.0));
     for (int t = 0; t < NT; ++t)
       for (int q = 0; q < NR; ++q)
-        for (int e = 0; e < p.tasks[t].n_ent; ++e) {
+        for (int e = 0; e < tasks[t].n_ent; ++e) {
           std::complex<double>* blk = &ph[((size_t(t) * NR + q) * p.max_ent + e) * PB];
           for (int role = 0; role < 2; ++role) {
-            const double w = role == 0 ? 1.0 : p.ent_w[p.tasks[t].ent_off + e];
+            const double w = role == 0 ? 1.0 : p.ent_w[tasks[t].ent_off + e];
             double tu[2];
             for (int ax = 0; ax < 2; ++ax)
               for (int n = 0; n < N; ++n) {
@@ -751,7 +756,7 @@ int upload_plan(Plan& p) {
     }
   }
   if ((rc = upload(p, p.ent_w.data(), p.ent_w.size(), (void**)&p.d_ent_w, total))) return rc;
-  if ((rc = upload(p, p.tasks.data(), p.tasks.size(), (void**)&p.d_tasks, total))) return rc;
+  if ((rc = upload(p, tasks.data(), tasks.size(), (void**)&p.d_tasks, total))) return rc;
   if ((rc = upload(p, p.groups.data(), p.groups.size(), (void**)&p.d_groups, total))) return rc;
   if ((rc = upload(p, p.ent_ysh.data(), p.ent_ysh.size(), (void**)&p.d_ent_ysh, total))) return rc;
   if (!p.faces.empty() && (rc = upload(p, p.faces.data(), p.faces.size(), (void**)&p.d_faces, total))) return rc;
@@ -777,9 +782,9 @@ int upload_plan(Plan& p) {
     cudaGetLastError();
     return DGFS_ERR_CUDA;
   }
-  if ((rc = dalloc(p, (void**)&p.d_counter, 256))) return rc;
-  // work counter and device status word start at zero
-  if (cudaMemsetAsync(p.d_counter, 0, 256, p.home) != cudaSuccess) {
+  if ((rc = dalloc(p, (void**)&p.d_counter, p.counter_bytes()))) return rc;
+  // the counters and the device status word start at zero
+  if (cudaMemsetAsync(p.d_counter, 0, p.counter_bytes(), p.home) != cudaSuccess) {
     cudaGetLastError();
     return DGFS_ERR_CUDA;
   }

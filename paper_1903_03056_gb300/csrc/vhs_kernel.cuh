@@ -40,6 +40,8 @@
 //   step C  after the last group: P -> spectrum, Q_hat_ij += F_ij P_hat (and Q_hat_ji for a cross pair)
 #pragma once
 
+#include <cmath>
+
 #include <cuda_runtime.h>
 
 #include "dgfs_internal.h"
@@ -48,28 +50,43 @@
 
 namespace dgfs {
 
-// compile-time launch shape per (precision, N): cluster size, plane groups per CTA, CTAs per SM
-template <typename T, int N> struct VShape;
-#define DGFS_SHAPE3(TT, NN, CC, GG, MB)      \
-  template <> struct VShape<TT, NN> {        \
+// Launch shape per (precision, N, W): cluster size, plane groups per CTA, CTAs per SM the registers
+// are sized for.  W = 0 serves batches that fill the device; W = 1, where it differs, spreads one
+// work item over more SMs for small batches (one plane per group, clusters of 4 to 8 CTAs).
+template <typename T, int N, int W> struct VShape : VShape<T, N, 0> {};
+template <typename T, int N> struct HasWide {
+  static constexpr bool value = false;
+  static constexpr double slow = 1.0;
+};
+#define DGFS_VHS_SHAPE(TT, NN, CC, GG, MB)   \
+  template <> struct VShape<TT, NN, 0> {     \
     static constexpr int cluster = CC;       \
     static constexpr int groups = GG;        \
     static constexpr int min_blocks = MB;    \
   };
-#define DGFS_SHAPE(TT, NN, CC, GG) DGFS_SHAPE3(TT, NN, CC, GG, 1)
+#define DGFS_VHS_WIDE(TT, NN, CC, GG, MB, SLOW)    \
+  template <> struct VShape<TT, NN, 1> {     \
+    static constexpr int cluster = CC;       \
+    static constexpr int groups = GG;        \
+    static constexpr int min_blocks = MB;    \
+  };                                         \
+  template <> struct HasWide<TT, NN> {       \
+    static constexpr bool value = true;      \
+    static constexpr double slow = SLOW;     \
+  };
 #include "vhs_shapes.h"
-#undef DGFS_SHAPE
-#undef DGFS_SHAPE3
+#undef DGFS_VHS_SHAPE
+#undef DGFS_VHS_WIDE
 
-template <typename T, int N>
+template <typename T, int N, int W>
 struct VGeo {
   static constexpr int h = N / 2;
   static constexpr int N2 = N * N, HN2 = N * h;
   static constexpr size_t N3 = size_t(N) * N * N, HN3 = size_t(N) * HN2;
   static constexpr int PITCH = N + 1;
-  static constexpr int CL = VShape<T, N>::cluster;
-  static constexpr int GP = VShape<T, N>::groups;
-  static constexpr int MINB = VShape<T, N>::min_blocks;
+  static constexpr int CL = VShape<T, N, W>::cluster;
+  static constexpr int GP = VShape<T, N, W>::groups;
+  static constexpr int MINB = VShape<T, N, W>::min_blocks;
   static constexpr int THREADS = GP * N;
   static constexpr int PLANES = N / CL;  // planes, and rows of pencils, per CTA
   static_assert(N % CL == 0 && PLANES % GP == 0, "planes must split evenly over the cluster and its plane groups");
@@ -86,8 +103,8 @@ struct VGeo {
   static constexpr int PB = 5 * N + 4;
   // workspace per cluster (complex values): f_hat of both species, two buffers of x-passed half
   // spectra of both roles, P_hat, two gain accumulators, parked P; then per entry the two faces
-  // and the k_x-face's k_z = N/2 line
-  static constexpr size_t SLOT = 3 * N3 + 3 * HN3 + (KEEP ? 0 : HN3);
+  // and the k_x-face's k_z = N/2 line.  The same for every W of (T, N).
+  static constexpr size_t SLOT = 3 * N3 + 4 * HN3;
   static constexpr size_t FACE = 2 * N2 + N;
 };
 
@@ -155,9 +172,23 @@ __device__ __forceinline__ double2 face_sum(double s, double2 u, double t, doubl
 __device__ __forceinline__ float2 mul_each(float2 s, float2 v) { return unpack2(pack2(s.x, s.y) * pack2(v.x, v.y)); }
 __device__ __forceinline__ double2 mul_each(double2 s, double2 v) { return make_double2(s.x * v.x, s.y * v.y); }
 
-template <typename T, int N>
-__global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_kernel(const KernelParams p) {
-  using G = VGeo<T, N>;
+// Gain of one mode: Q_hat (+)= F P_hat.  A work item split over its radial nodes adds them up later
+// with these operations in the same order, so it gives the same bits.
+template <typename T>
+__device__ __forceinline__ C<T> add_gain(C<T> acc, T f, C<T> v, bool first) {
+  return first ? scale<T>(v, f) : mk<T>(fma_(v.x, f, acc.x), fma_(v.y, f, acc.y));
+}
+// a mode of two real pencils held as one, p_0 + i p_h with weights fa, fh: v its value, m that of -k_x
+template <typename T>
+__device__ __forceinline__ C<T> add_gain_pair(C<T> acc, T fa, T fh, C<T> v, C<T> m, bool first) {
+  const T fp = T(0.5) * (fa + fh), fm = T(0.5) * (fa - fh);
+  const C<T> w = mk<T>(fma_(fm, m.x, fp * v.x), fma_(-fm, m.y, fp * v.y));
+  return first ? w : add<T>(w, acc);
+}
+
+template <typename T, int N, int W>
+__global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) vhs_kernel(const KernelParams p) {
+  using G = VGeo<T, N, W>;
   using CT = C<T>;
   constexpr int h = G::h, N2 = G::N2, HN2 = G::HN2, CL = G::CL, GP = G::GP, NT = G::THREADS, PITCH = G::PITCH;
   constexpr int PB = G::PB;
@@ -188,16 +219,23 @@ __global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_ker
   const int plane0 = rank * G::PLANES;
   const T inv_n3 = T(1) / T(N3);
 
-  // Work items (node, task) come from a counter: thread 0 of the rank-0 CTA takes the next item
-  // after the first barrier of the current one, when every CTA has read the current value.
+  // Work items (task, node, chunk of radial nodes) come from a counter: thread 0 of the rank-0 CTA
+  // takes the next item after the first barrier of the current one, when every CTA has read the
+  // current value.  Tasks are in order of falling cost, so the last items are the short ones.
   __shared__ int s_next_item;
-  const int n_items = p.batch * p.n_tasks;
+  __shared__ int s_last;
+  const int n_items = p.batch * p.n_tasks * p.chunks;
   if (rank == 0 && tid == 0) s_next_item = int(atomicAdd(p.work_counter, 1u));
   cluster_sync<CL>();
   for (int item = CL == 1 ? s_next_item : ld_rank0(&s_next_item); item < n_items;
        item = CL == 1 ? s_next_item : ld_rank0(&s_next_item)) {
-    const int b = item / p.n_tasks;
-    const int task = item % p.n_tasks;
+    const int chunk = item % p.chunks;
+    const int whole = item / p.chunks;
+    const int b = whole % p.batch;
+    const int task = whole / p.batch;
+    const bool split = p.chunks > 1;
+    const int q0 = chunk * p.n_rho / p.chunks, q1 = (chunk + 1) * p.n_rho / p.chunks;
+    CT* const PT = static_cast<CT*>(p.parts) + size_t(whole) * p.n_rho * HN3;  // P_hat of every radial node
     const TaskDesc tk = p.tasks[task];
     const T* fb = reinterpret_cast<const T*>(p.f) + size_t(b) * p.s * N3;
     const bool self = tk.i == tk.j;
@@ -245,7 +283,7 @@ __global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_ker
 
     // ---- gain ---------------------------------------------------------------------------------
     T P[G::PSM ? 1 : N];
-    for (int q = 0; q < p.n_rho; ++q) {
+    for (int q = q0; q < q1; ++q) {
       const CT* const phq = static_cast<const CT*>(p.phase) + (size_t(task) * p.n_rho + q) * p.max_ent * PB;
       if (ph_smem) {
         for (int u = tid; u < tk.n_ent * PB; u += NT) phs[u] = __ldg(phq + u);
@@ -436,6 +474,11 @@ __global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_ker
         const bool pair_row = cc == 0 && (r == 0 || r == h);
         const int ky = cc == 0 && r >= h ? r - h : r;
         const int kz = cc == 0 && r >= h ? h : cc;
+        if (split) {
+#pragma unroll
+          for (int n = 0; n < N; ++n) st2<T>(PT + q * HN3 + n * HN2 + pp, v[n]);
+          continue;
+        }
         for (int o = 0; o < 2; ++o) {
           const int pair = o == 0 ? tk.out0 : tk.out1;
           if (pair < 0) break;
@@ -444,21 +487,58 @@ __global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_ker
           if (!pair_row) {
 #pragma unroll
             for (int n = 0; n < N; ++n) {
-              CT val = scale<T>(v[n], __ldg(Fw + n * N2));
-              if (q > 0) val = add<T>(val, ld2<T>(acc + n * HN2));
-              st2<T>(acc + n * HN2, val);
+              const CT old = q > 0 ? ld2<T>(acc + n * HN2) : mk<T>(0, 0);
+              st2<T>(acc + n * HN2, add_gain<T>(old, __ldg(Fw + n * N2), v[n], q == 0));
             }
           } else {
 #pragma unroll
             for (int n = 0; n < N; ++n) {
-              const T fa = __ldg(Fw + n * N2), fh = __ldg(Fw + n * N2 + h * N);
-              const T fp = T(0.5) * (fa + fh), fm = T(0.5) * (fa - fh);
-              const CT m = v[(N - n) % N];
-              CT val = mk<T>(fp * v[n].x + fm * m.x, fp * v[n].y - fm * m.y);
-              if (q > 0) val = add<T>(val, ld2<T>(acc + n * HN2));
-              st2<T>(acc + n * HN2, val);
+              const CT old = q > 0 ? ld2<T>(acc + n * HN2) : mk<T>(0, 0);
+              st2<T>(acc + n * HN2, add_gain_pair<T>(old, __ldg(Fw + n * N2), __ldg(Fw + n * N2 + h * N), v[n],
+                                                     v[(N - n) % N], q == 0));
             }
           }
+        }
+      }
+    }
+    if (split) {
+      // the cluster that stores the last of the item's products adds them up and finishes the item
+      __threadfence();
+      cluster_sync<CL>();
+      if (rank == 0 && tid == 0) {
+        unsigned* const done = p.work_counter + kDoneWord + whole;
+        s_last = atomicAdd(done, 1u) + 1 == unsigned(p.chunks) ? 1 : 0;
+        if (s_last) *done = 0;  // ready for the next launch
+        __threadfence();
+      }
+      cluster_sync<CL>();
+      if ((CL == 1 ? s_last : ld_rank0(&s_last)) == 0) {
+        cluster_sync<CL>();  // s_last has been read
+        continue;
+      }
+      __threadfence();
+      for (int u = tid; u < N * G::PLANES * h; u += NT) {  // element by element: every load independent
+        const int n = u / (G::PLANES * h), pp = plane0 * h + u % (G::PLANES * h);
+        const int r = pp / h, cc = pp % h;
+        const bool pair_row = cc == 0 && (r == 0 || r == h);
+        const int ky = cc == 0 && r >= h ? r - h : r;
+        const int kz = cc == 0 && r >= h ? h : cc;
+        const CT* const pv = PT + n * HN2 + pp;
+        const CT* const pm = PT + (n == 0 ? 0 : N - n) * HN2 + pp;
+        for (int o = 0; o < 2; ++o) {
+          const int pair = o == 0 ? tk.out0 : tk.out1;
+          if (pair < 0) break;
+          const T* const Fw = static_cast<const T*>(p.Fw) + size_t(pair) * p.n_rho * N3 + n * N2 + ky * N + kz;
+          CT acc = mk<T>(0, 0);
+          if (!pair_row) {
+#pragma unroll 8
+            for (int q = 0; q < p.n_rho; ++q) acc = add_gain<T>(acc, __ldg(Fw + q * N3), ld2<T>(pv + q * HN3), q == 0);
+          } else {
+            for (int q = 0; q < p.n_rho; ++q)
+              acc = add_gain_pair<T>(acc, __ldg(Fw + q * N3), __ldg(Fw + q * N3 + h * N), ld2<T>(pv + q * HN3),
+                                     ld2<T>(pm + q * HN3), q == 0);
+          }
+          st2<T>((o == 0 ? QA : QB) + n * HN2 + pp, acc);
         }
       }
     }
@@ -545,48 +625,128 @@ __global__ void __launch_bounds__(VGeo<T, N>::THREADS, VGeo<T, N>::MINB) vhs_ker
   }
   // no CTA leaves while another may still read its shared memory (the last item index)
   if constexpr (CL > 1) cluster_sync<CL>();
+  // every cluster has taken its last item once all have come here: the last one readies the counter
+  // for the next launch
+  if (rank == 0 && tid == 0 && atomicAdd(p.work_counter + kExitWord, 1u) + 1 == gridDim.x / CL) {
+    p.work_counter[0] = 0;
+    p.work_counter[kExitWord] = 0;
+  }
 }
 
-template <typename T, int N>
-int vhs_configure_impl(Plan& pl) {
-  using G = VGeo<T, N>;
-  auto kern = vhs_kernel<T, N>;
-  // the phase block of the current (task, rho) goes to shared memory while MINB CTAs still fit
+// dynamic shared memory of a shape; *ph_mode = 1 when the phase block of the current (task, rho) is
+// in it (while MINB CTAs still fit)
+template <typename T, int N, int W>
+size_t vhs_smem(const Plan& pl, int* ph_mode) {
+  using G = VGeo<T, N, W>;
   const size_t ph_bytes = size_t(pl.max_ent) * G::PB * sizeof(C<T>);
-  const int ph_mode = G::MINB * (G::SMEM + ph_bytes + 2048) <= size_t(226) * 1024 ? 1 : 0;
-  const size_t smem = G::SMEM + (ph_mode ? ph_bytes : 0);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+  *ph_mode = G::MINB * (G::SMEM + ph_bytes + 2048) <= size_t(226) * 1024 ? 1 : 0;
+  return G::SMEM + (*ph_mode ? ph_bytes : 0);
+}
+
+inline void vhs_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cluster, int clusters, const VhsShape& s,
+                       cudaStream_t st) {
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(clusters * cluster);
+  cfg.blockDim = dim3(s.threads);
+  cfg.dynamicSmemBytes = s.smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+}
+
+template <typename T, int N, int W>
+int vhs_configure_shape(Plan& pl) {
+  using G = VGeo<T, N, W>;
+  auto kern = vhs_kernel<T, N, W>;
+  VhsShape& s = pl.vhs[W];
+  s.threads = G::THREADS;
+  s.smem = vhs_smem<T, N, W>(pl, &s.phase_smem);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
     return DGFS_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = G::CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(G::CL);
-  cfg.blockDim = dim3(G::THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters <= 0) {
+  vhs_config(cfg, attr, G::CL, 1, s, nullptr);
+  if (cudaOccupancyMaxActiveClusters(&s.clusters, kern, &cfg) != cudaSuccess || s.clusters <= 0) {
     cudaGetLastError();
     return DGFS_ERR_CUDA;
   }
-  pl.shape.cluster = G::CL;
-  pl.shape.groups = G::GP;
-  pl.shape.threads = G::THREADS;
-  pl.shape.smem = smem;
-  pl.shape.phase_smem = ph_mode;
-  pl.shape.clusters = clusters;
-  pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
-  pl.scratch_bytes = size_t(clusters) * pl.shape.slot * sizeof(C<T>);
   return DGFS_OK;
 }
 
 template <typename T, int N>
+int vhs_configure_impl(Plan& pl) {
+  using G = VGeo<T, N, 0>;
+  if (int rc = vhs_configure_shape<T, N, 0>(pl)) return rc;
+  if constexpr (HasWide<T, N>::value) {
+    if (int rc = vhs_configure_shape<T, N, 1>(pl)) return rc;
+  }
+  pl.shape.cluster = G::CL;
+  pl.shape.groups = G::GP;
+  pl.shape.threads = G::THREADS;
+  pl.shape.smem = pl.vhs[0].smem;
+  pl.shape.clusters = pl.vhs[0].clusters;
+  pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
+  // one workspace per cluster of either shape, then the products of split items
+  int most = pl.vhs[0].clusters;
+  if (pl.vhs[1].clusters > most) most = pl.vhs[1].clusters;
+  pl.part_off = size_t(most) * pl.shape.slot;
+  pl.part_slots = kPartsPerCluster * most;
+  pl.scratch_bytes = (pl.part_off + size_t(pl.part_slots) * G::HN3) * sizeof(C<T>);
+  return DGFS_OK;
+}
+
+// How a launch of `items` work items (task, node) runs: the shape W and the number of chunks each
+// item's radial nodes are split into, by a cost model in units of one radial node of the dearest
+// task on a full device.  A chunk of `len` nodes costs len + 1/2 (its own f_hat).  Chunks go out one
+// by one, so a launch takes its share of the device, sum of costs / clusters, and about 0.38 of the
+// last chunk; a chunk on a nearly idle device runs at 0.6 of its cost.  Fitted to N = 24, 45 nodes
+// (W = 0: 1.42, 1.21, 1.11, 0.98, 1.10 ms with 1, 2, 4, 6, 12 chunks) and N = 32, 5 nodes, 3 species
+// (W = 0: 2.30, 1.22, 0.99, 1.11 ms with 1, 4, 8, 16; W = 1: 0.97, 0.74, 0.75, 0.84 with 1, 2, 4, 16).
+// The wide shape takes `slow` times longer per node and cluster-share of the device.  All products
+// of all items must fit the parts buffer.
+struct VhsRun {
+  int wide = 0, chunks = 1;
+};
+inline VhsRun vhs_plan_run(int items, int n_rho, int clusters0, int clusters1, double slow, double mean_cost,
+                           int part_slots) {
+  VhsRun best;
+  double best_t = 1e300;
+  for (int w = 0; w < 2; ++w) {
+    const int C = w == 0 ? clusters0 : clusters1;
+    if (C <= 0) continue;
+    const double unit = w == 0 ? 1.0 : slow * double(clusters1) / double(clusters0);
+    for (int s = 1; s <= n_rho; ++s) {
+      if (s > 1 && double(items) * n_rho > double(part_slots)) break;
+      const int len = (n_rho + s - 1) / s;
+      if (s > 1 && (n_rho + s - 2) / (s - 1) == len) continue;  // no shorter than with s - 1 chunks
+      const double one = 0.5 + len, share = double(items) * s * mean_cost * one / C + 0.38 * one;
+      const double t = (share > 0.6 * one ? share : 0.6 * one) * unit;
+      if (t < best_t * (1.0 - 1e-9)) {
+        best_t = t;
+        best.wide = w;
+        best.chunks = s;
+      }
+    }
+  }
+  return best;
+}
+
+template <typename T, int N, int W>
+int vhs_launch_shape(const Plan& pl, KernelParams& kp, int items, int limit, cudaStream_t st) {
+  using G = VGeo<T, N, W>;
+  const VhsShape& s = pl.vhs[W];
+  kp.phase_smem = s.phase_smem;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  vhs_config(cfg, attr, G::CL, items < limit ? items : limit, s, st);
+  return cudaLaunchKernelEx(&cfg, vhs_kernel<T, N, W>, kp) == cudaSuccess ? DGFS_OK : DGFS_ERR_CUDA;
+}
+
+template <typename T, int N>
 int vhs_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
-  using G = VGeo<T, N>;
   KernelParams kp;
   kp.f = f;
   kp.Q = Q;
@@ -603,27 +763,25 @@ int vhs_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStrea
   kp.Gm = pl.d_Gmf ? static_cast<const void*>(pl.d_Gmf) : static_cast<const void*>(pl.d_Gm);
   kp.scratch = pl.scratch_of(ws);
   kp.slot = pl.shape.slot;
-  kp.phase_smem = pl.shape.phase_smem;
+  kp.parts = static_cast<C<T>*>(pl.scratch_of(ws)) + pl.part_off;
   kp.work_counter = pl.counter_of(ws);
+  auto share_of = [&](int clusters) {
+    const int n = int(clusters * pl.shape.share);
+    return n < 1 ? 1 : n;
+  };
   const int items = batch * kp.n_tasks;
-  int limit = int(pl.shape.clusters * pl.shape.share);
-  if (limit < 1) limit = 1;
-  const int clusters = items < limit ? items : limit;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = G::CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(clusters * G::CL);
-  cfg.blockDim = dim3(G::THREADS);
-  cfg.dynamicSmemBytes = pl.shape.smem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaMemsetAsync(kp.work_counter, 0, sizeof(unsigned), st) != cudaSuccess) return DGFS_ERR_CUDA;
-  if (cudaLaunchKernelEx(&cfg, vhs_kernel<T, N>, kp) != cudaSuccess) return DGFS_ERR_CUDA;
-  return DGFS_OK;
+  const int c0 = share_of(pl.vhs[0].clusters), c1 = pl.vhs[1].clusters > 0 ? share_of(pl.vhs[1].clusters) : 0;
+  double cost = 0.0, most = 0.0;
+  for (const TaskDesc& t : pl.tasks) {
+    cost += t.n_ent;
+    most = t.n_ent > most ? t.n_ent : most;
+  }
+  const VhsRun run = vhs_plan_run(items, pl.N_rho, c0, c1, HasWide<T, N>::slow, cost / (kp.n_tasks * most), pl.part_slots);
+  kp.chunks = run.chunks;
+  if constexpr (HasWide<T, N>::value) {
+    if (run.wide) return vhs_launch_shape<T, N, 1>(pl, kp, items * run.chunks, c1, st);
+  }
+  return vhs_launch_shape<T, N, 0>(pl, kp, items * run.chunks, c0, st);
 }
 
 }  // namespace dgfs

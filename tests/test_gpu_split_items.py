@@ -1,0 +1,48 @@
+"""Small VHS batches run with their radial nodes split into chunks, and on some grids in a launch
+shape of their own; a node's result is bit for bit the one it has inside a batch that fills the
+device and runs unsplit."""
+
+import numpy as np
+import pytest
+
+from paper_1903_03056_gb300 import dgfs, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("N,batch", [(4, 20000), (6, 8000), (8, 4000), (12, 1500), (16, 1000), (24, 400),
+                                     (32, 400), (48, 140)])
+def test_a_node_alone_and_in_a_full_batch_give_the_same_bits(N, batch, precision):
+    import torch
+    dt = torch.float32 if precision == "fp32" else torch.float64
+    # N_rho = 5 does not divide into the chunks evenly; the full batch's products outnumber any
+    # parts buffer, so it runs unsplit
+    w = synth.Workload("split", 3, N, 5.0, (1.0, 2.1), 0.7, 1.0, 6, 5, "bimaxwellian", 0.05, 90)
+    few = torch.from_numpy(synth.batch_distribution(w)).to(device="cuda", dtype=dt)
+    full = few.repeat((batch + 2) // 3, 1, 1, 1, 1)[:batch].contiguous()
+    plan = dgfs.Plan(N, 5.0, [1.0, 2.1], 0.7, M=6, N_rho=5, precision=precision)
+    ref = plan.eval(full)
+    for b in (1, 2, 3):
+        assert torch.equal(plan.eval(few[:b].contiguous()), ref[:b])
+    plan.set_sm_share(0.1)  # fewer clusters: another split of the same items
+    assert torch.equal(plan.eval(few), ref[:3])
+    torch.cuda.synchronize()
+    assert plan.check()
+    plan.close()
+
+
+def test_a_split_evaluation_replays_from_a_graph():
+    import torch
+    w = synth.Workload("split", 2, 16, 5.0, (1.0, 2.1), 0.7, 1.0, 6, 5, "bimaxwellian", 0.05, 91)
+    f = torch.from_numpy(synth.batch_distribution(w)).to(device="cuda", dtype=torch.float32)
+    plan = dgfs.Plan(16, 5.0, [1.0, 2.1], 0.7, M=6, N_rho=5, precision="fp32")
+    ref = plan.eval(f)
+    Q = torch.zeros_like(ref)
+    g = plan.capture(f, Q)
+    for _ in range(3):
+        Q.fill_(np.nan)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(Q, ref)
+    plan.close()
