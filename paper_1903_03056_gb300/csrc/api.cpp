@@ -38,14 +38,17 @@ int launch_core(dgfs::Plan& p, const void* f, void* Q, int batch, cudaStream_t s
   int rc = run(p, f, Qfull, batch, st, ws);
   if (rc != DGFS_OK) return rc;
   *launches += 1;
+  double* lam = nullptr;
   if (p.flags & DGFS_CONSERVE) {
     dgfs::NvtxRange r2("dgfs conservation projection");
-    if ((rc = dgfs::launch_conserve(p, Qfull, batch, st)) != DGFS_OK) return rc;
+    // with the species sum the projection is applied there, from its multipliers
+    if (sum) lam = p.d_lam + size_t(stage_node) * p.cons.size() * 6;
+    if ((rc = dgfs::launch_conserve(p, Qfull, batch, lam, st)) != DGFS_OK) return rc;
     *launches += 1;
   }
   if (sum) {
     dgfs::NvtxRange r2("dgfs species sum");
-    if ((rc = dgfs::launch_species_sum(p, Qfull, Q, batch, st)) != DGFS_OK) return rc;
+    if ((rc = dgfs::launch_species_sum(p, Qfull, Q, batch, lam, st)) != DGFS_OK) return rc;
     *launches += 1;
   }
   return DGFS_OK;

@@ -155,6 +155,7 @@ struct Plan {
   // device tables
   ConsBlock* d_cons = nullptr;
   double* d_kappa = nullptr;
+  double* d_lam = nullptr;         // multipliers of the projection (DGFS_CONSERVE | DGFS_SUM_SPECIES)
   void* d_Qfull = nullptr;         // full operators staged for DGFS_SUM_SPECIES
   double* d_Fw = nullptr;
   double2* d_Fv = nullptr;         // VSS gain weights (complex)
@@ -265,9 +266,11 @@ int launch_bf16x3(const Plan& p, const void* f, void* Q, int batch, cudaStream_t
 // SSP-RK2 stage combinations (stepper.cu): stage 1 f1 = f + dt r; stage 2 f = (f + f1 + dt r)/2
 int launch_rk_stage(const Plan& p, int stage, void* f, void* f1, const void* r, double dt, size_t n, cudaStream_t st);
 
-// conservation projection (in place on Q[batch][s][s][N^3]) and species sum (conserve.cu)
-int launch_conserve(const Plan& p, void* Q, int batch, cudaStream_t st);
-int launch_species_sum(const Plan& p, const void* Qfull, void* Qsum, int batch, cudaStream_t st);
+// conservation projection of Q[batch][s][s][N^3] and species sum (conserve.cu).  lam = null projects
+// Q in place; otherwise the multipliers go to lam [batch][block][6] and Q stays, and the species
+// sum given the same lam subtracts the projection
+int launch_conserve(const Plan& p, void* Q, int batch, double* lam, cudaStream_t st);
+int launch_species_sum(const Plan& p, const void* Qfull, void* Qsum, int batch, const double* lam, cudaStream_t st);
 
 }  // namespace dgfs
 

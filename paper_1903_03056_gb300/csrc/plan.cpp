@@ -771,6 +771,8 @@ int upload_plan(Plan& p) {
   p.table_bytes = total;
   if ((p.flags & DGFS_SUM_SPECIES) && p.max_batch > 0) {
     if ((rc = dalloc(p, &p.d_Qfull, size_t(p.max_batch) * s * s * N3 * real_size(p)))) return rc;
+    if (!p.cons.empty() && (rc = dalloc(p, (void**)&p.d_lam, size_t(p.max_batch) * p.cons.size() * 6 * sizeof(double))))
+      return rc;
   }
   // the workspace between two guard blocks of a fixed byte pattern: dgfs_plan_check reads
   // them back to detect a kernel write outside the workspace
@@ -797,7 +799,7 @@ void free_plan(Plan& p) {
   void* ptrs[] = {p.d_Fw,      p.d_Gm,      p.d_ent_w,   p.d_phase, p.d_tasks, p.d_groups, p.d_Fv,
                   p.d_scratch_raw, p.d_stage_f, p.d_stage_Q, p.d_cons, p.d_kappa, p.d_Qfull, p.d_ent_m,
                   p.d_counter, p.d_rk,      p.d_ent_ysh, p.d_Fwf,    p.d_Fvf,   p.d_Gmf,   p.d_mats,
-                  p.d_scratch2_raw, p.d_counter2, p.d_faces};
+                  p.d_scratch2_raw, p.d_counter2, p.d_faces, p.d_lam};
   if (p.home) {
     for (void* q : ptrs)
       if (q) cudaFreeAsync(q, p.home);
@@ -840,6 +842,7 @@ void free_plan(Plan& p) {
   p.d_rk = nullptr;
   p.d_mats = nullptr;
   p.d_faces = nullptr;
+  p.d_lam = nullptr;
 }
 
 }  // namespace dgfs
