@@ -110,22 +110,6 @@ struct Geo {
   static constexpr int SLOT = 2 + 2 * NBV + 4;
 };
 
-// Hint that [p, p + bytes) (16-byte aligned, a multiple of 16 bytes) is read soon: one bulk
-// prefetch into L2, so the loads that follow meet L2 rather than DRAM latency.  The workspace
-// of all clusters exceeds L2, so a volume written in one phase is partly evicted before it is
-// read in the next.
-__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// Order this thread's generic-proxy accesses to global memory before later async-proxy (bulk
-// copy) accesses: the workspace planes are written with ordinary stores and read back by bulk
-// copies after a barrier.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
-
 // transpose a plane held as column t (x[r] = V[r][t]) into row t (x[c] = V[t][c]) and back
 template <typename T, int N, int GP>
 __device__ __forceinline__ void cols_to_rows(C<T> (&x)[N], C<T>* tb, int t) {

@@ -568,32 +568,25 @@ int upload_plan(Plan& p) {
               for (int n = 0; n < N; ++n)
                 ph[((((size_t(t) * NR + q) * p.max_ent + e) * 2 + role) * 3 + ax) * N + n] = phase_of(t, q, e, role, ax, n);
   } else {
-    // [task][rho][entry] blocks of the VHS kernel: x [N][role], y [N][role], z [role][N/2], then
-    // per role (cz, tz) and per role (tx, ty), c + i t the phase of the unpaired mode N/2; the x
-    // and y entries of that mode keep c alone; role 1's z phases, cz and tz carry the weight w_e
-    const size_t PB = 5 * size_t(N) + 4;
+    // [task][rho][entry] blocks of the VHS kernel: x [N/2][role], y [N/2][role], z [role][N/2] (role 1
+    // times the weight w_e), then (w_e, 0) and a pad.  Modes 1..N/2-1 (their negatives take the
+    // conjugate); the slot of mode 0, whose phase is 1, holds the unpaired mode's c + i t
+    const size_t PB = 3 * size_t(N) + 2;
     const int h = N / 2;
     ph.assign(size_t(NT) * NR * p.max_ent * PB, std::complex<double>(0.0, 0.0));
     for (int t = 0; t < NT; ++t)
       for (int q = 0; q < NR; ++q)
         for (int e = 0; e < tasks[t].n_ent; ++e) {
           std::complex<double>* blk = &ph[((size_t(t) * NR + q) * p.max_ent + e) * PB];
-          for (int role = 0; role < 2; ++role) {
-            const double w = role == 0 ? 1.0 : p.ent_w[tasks[t].ent_off + e];
-            double tu[2];
-            for (int ax = 0; ax < 2; ++ax)
-              for (int n = 0; n < N; ++n) {
-                std::complex<double> z = phase_of(t, q, e, role, ax, n);
-                if (n == h) {
-                  tu[ax] = z.imag();
-                  z = z.real();
-                }
-                blk[size_t(ax) * 2 * N + 2 * n + role] = z;
-              }
-            for (int n = 0; n < h; ++n) blk[4 * N + role * h + n] = w * phase_of(t, q, e, role, 2, n);
-            blk[5 * N + role] = w * phase_of(t, q, e, role, 2, h);
-            blk[5 * N + 2 + role] = std::complex<double>(tu[0], tu[1]);
-          }
+          const double we = p.ent_w[tasks[t].ent_off + e];
+          for (int role = 0; role < 2; ++role)
+            for (int n = 0; n < h; ++n) {
+              const int mode = n == 0 ? h : n;
+              blk[2 * n + role] = phase_of(t, q, e, role, 0, mode);
+              blk[N + 2 * n + role] = phase_of(t, q, e, role, 1, mode);
+              blk[2 * N + role * h + n] = (role == 0 ? 1.0 : we) * phase_of(t, q, e, role, 2, mode);
+            }
+          blk[3 * N] = we;
         }
   }
   const size_t nph = ph.size();

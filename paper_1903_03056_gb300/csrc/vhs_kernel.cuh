@@ -47,6 +47,7 @@
 #include "dgfs_internal.h"
 #include "group_sync.cuh"
 #include "real_line.cuh"
+#include "tcgen05.cuh"
 
 namespace dgfs {
 
@@ -95,25 +96,67 @@ struct VGeo {
   // it is parked in the workspace between sigma_x groups
   static constexpr bool PSM = sizeof(T) == 8 && N >= 48;
   static constexpr bool KEEP = PLANES == GP;
+  // L2 prefetch of a group's next plane one plane ahead (measured: N = 32 -1.8 %, 48 -0.8 %, smaller
+  // grids, whose workspaces mostly stay in L2, +0.5 to 1.4 %)
+  static constexpr bool PF = sizeof(T) == 4 && N >= 32;
+  // Tensor memory (FP32): each thread owns a lane, TMEM holds its raw line of the current plane (read
+  // once per sigma_x group, used by every entry of it) and the parked P of its planes.  Neither then
+  // goes through L2 or the L1 data path again.  Used while the CTAs an SM holds fit its 512 columns.
+  static constexpr int PPG = PLANES / GP;
+  static constexpr int SETS = (THREADS + 127) / 128;  // warps that share a lane quarter
+  static constexpr int alloc_of(int cols) { return cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512; }
+  static constexpr bool fits(int cols) { return cols > 0 && cols <= 512 && MINB * alloc_of(cols) <= 512; }
+  static constexpr bool TMOK = sizeof(T) == 4 && N % 8 == 0 && N >= 16 && N <= 32 && THREADS % 32 == 0 && W == 0;
+  static constexpr int P_COLS = KEEP ? 0 : PPG * N;
+  static constexpr bool TMP = TMOK && !KEEP && fits(SETS * P_COLS);
+  static constexpr bool TMR = TMOK && fits(SETS * (2 * N + (TMP ? P_COLS : 0)));
+  static constexpr int TM_SET = (TMR ? 2 * N : 0) + (TMP ? P_COLS : 0);  // columns of a thread
+  static constexpr int TM_ALLOC = TM_SET > 0 ? alloc_of(SETS * TM_SET) : 0;
   // shared memory per group: one padded plane, the entry's row of the k_y face, P if PSM
-  static constexpr size_t GROUP_BYTES = (size_t(N) * PITCH + N) * sizeof(C<T>) + (PSM ? N2 * sizeof(T) : 0);
+  // (FP32: the groups' stride is 2 N words modulo 32, so that the lanes of a warp that spans two
+  // groups hit distinct banks: N = 24)
+  static constexpr size_t GROUP_BASE = (size_t(N) * PITCH + N) * sizeof(C<T>) + (PSM ? N2 * sizeof(T) : 0);
+  static constexpr size_t GROUP_BYTES =
+      GROUP_BASE + (sizeof(T) == 4 ? size_t((2 * N + 32 - int(GROUP_BASE / 4 % 32)) % 32) * 4 : 0);
+  static_assert(GROUP_BYTES % 16 == 0, "16-byte accesses");
   static constexpr size_t SMEM = GP * GROUP_BYTES;
-  // phase block of an entry (complex values): x [N][role], y [N][role], z [role][h] (role 1 times
-  // w_e), then per role (cz, tz) (role 1 times w_e) and per role (tx, ty)
-  static constexpr int PB = 5 * N + 4;
-  // workspace per cluster (complex values): f_hat of both species, two buffers of x-passed half
-  // spectra of both roles, P_hat, two gain accumulators, parked P; then per entry the two faces
+  // phase block of an entry (complex values): x [h][role], y [h][role], z [role][h] (role 1 times
+  // w_e), then (w_e, 0) and a pad.  Mode 0 needs no phase: its slot holds c + i t, the unpaired mode's
+  static constexpr int PB = 3 * N + 2;
+  // workspace per cluster (complex values): f_hat of both species, NBH buffers of x-passed
+  // half spectra of both roles, P_hat, two gain accumulators, parked P; then per entry the two faces
   // and the k_x-face's k_z = N/2 line.  The same for every W of (T, N).
-  static constexpr size_t SLOT = 3 * N3 + 4 * HN3;
+  static constexpr bool SPLIT = CL > 1 && (sizeof(T) == 8 || N >= 48);
+  static constexpr int NBH = SPLIT ? 3 : 2;
+  static constexpr size_t SLOT = (1 + 3) * N3 + 4 * HN3;
   static constexpr size_t FACE = 2 * N2 + N;
 };
 
-// v[n] *= ph[2 n]: the shared phase e^{i theta k} of a line; mode 0 has phase 1 and the unpaired
-// mode N/2 the real factor c
+// v[n] *= e^{i theta k_n}, ph[2 n] the phase of mode n: mode -n (entry N - n) takes its conjugate, the
+// unpaired mode the real factor c, mode 0 none
 template <typename T, int N>
 __device__ __forceinline__ void shift_line(C<T> (&v)[N], const C<T>* ph) {
+  v[N / 2] = scale<T>(v[N / 2], ph[0].x);
 #pragma unroll
-  for (int n = 1; n < N; ++n) v[n] = n == N / 2 ? scale<T>(v[n], ph[2 * n].x) : cmul<T>(v[n], ph[2 * n]);
+  for (int n = 1; n < N / 2; ++n) {
+    const C<T> f = ph[2 * n], a = v[n], b = v[N - n];
+    v[n] = mk<T>(a.x * f.x - a.y * f.y, a.x * f.y + a.y * f.x);
+    v[N - n] = mk<T>(b.x * f.x + b.y * f.y, b.y * f.x - b.x * f.y);
+  }
+}
+
+// whether an entry (phase block pe) has a shift along x, and with it a k_x face
+template <typename T> __device__ __forceinline__ bool has_face(const C<T>* pe) { return pe[0].y != T(0) || pe[1].y != T(0); }
+
+// two neighbouring complex values (index i even) with one 16-byte access
+__device__ __forceinline__ void load_two(const float2* p, float2& a, float2& b) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  a = make_float2(q.x, q.y);
+  b = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void load_two(const double2* p, double2& a, double2& b) {
+  a = p[0];
+  b = p[1];
 }
 
 // Real rows of both roles of a plane.  In FP32 the roles run packed, one register pair per value:
@@ -134,12 +177,22 @@ template <int N>
 __device__ __forceinline__ void rows_c2r(const float2* row, const float2* phz, float2 x0, float2 xh, Rows<float, N>& y) {
   constexpr int h = N / 2;
   C2 x[h];
+  float2 fa[2], fb[2];
 #pragma unroll
   for (int k = 1; k < h; ++k) {
     float2 a = row[k], b = row[h + k];
     if (phz != nullptr) {
-      a = cmul<float>(a, phz[k]);
-      b = cmul<float>(b, phz[h + k]);
+      if constexpr (h % 2 == 0) {  // the phases two at a time (every block starts on 16 bytes)
+        if (k == 1 || k % 2 == 0) {
+          load_two(phz + (k & ~1), fa[0], fa[1]);
+          load_two(phz + h + (k & ~1), fb[0], fb[1]);
+        }
+        a = cmul<float>(a, fa[k & 1]);
+        b = cmul<float>(b, fb[k & 1]);
+      } else {
+        a = cmul<float>(a, phz[k]);
+        b = cmul<float>(b, phz[h + k]);
+      }
     }
     x[k].x = pack2(a.x, b.x);
     x[k].y = pack2(a.y, b.y);
@@ -186,6 +239,36 @@ __device__ __forceinline__ C<T> add_gain_pair(C<T> acc, T fa, T fh, C<T> v, C<T>
   return first ? w : add<T>(w, acc);
 }
 
+// n consecutive TMEM columns of the thread's lane (n a multiple of 8; every thread of the warp takes
+// part).  A load waits for its data inside its asm statement; a store is waited for at once, since the
+// next access of these columns may come soon.
+template <int n>
+__device__ __forceinline__ void tm_load(uint32_t ta, float* v) {
+  if constexpr (n >= 32) {
+    tc::tmem_ld32w(ta, v);
+    if constexpr (n > 32) tm_load<n - 32>(ta + 32, v + 32);
+  } else if constexpr (n >= 16) {
+    tc::tmem_ld16w(ta, v);
+    if constexpr (n > 16) tm_load<n - 16>(ta + 16, v + 16);
+  } else {
+    tc::tmem_ld8w(ta, v);
+  }
+}
+template <int n>
+__device__ __forceinline__ void tm_store_part(uint32_t ta, const float* v) {
+  if constexpr (n >= 16) {
+    tc::tmem_st16p(ta, v);
+    if constexpr (n > 16) tm_store_part<n - 16>(ta + 16, v + 16);
+  } else {
+    tc::tmem_st8(ta, v);
+  }
+}
+template <int n>
+__device__ __forceinline__ void tm_store(uint32_t ta, const float* v) {
+  tm_store_part<n>(ta, v);
+  tc::tmem_wait_st();
+}
+
 template <typename T, int N, int W>
 __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) vhs_kernel(const KernelParams p) {
   using G = VGeo<T, N, W>;
@@ -206,12 +289,27 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
   CT* const phs = reinterpret_cast<CT*>(smem_raw + G::SMEM);  // phase block of the current (task, rho)
   const bool ph_smem = p.phase_smem != 0;
 
+  // TMEM: warp 0 allocates the CTA's columns; warp w reaches lanes 32 (w % 4) .. + 31
+  __shared__ uint32_t s_tmem;
+  uint32_t tm_raw = 0, tm_p = 0;
+  if constexpr (G::TM_ALLOC > 0) {
+    if (tid < 32) {
+      tc::tmem_alloc(&s_tmem, G::TM_ALLOC);
+      tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    tm_raw = s_tmem + (uint32_t(32 * ((tid / 32) & 3)) << 16) + uint32_t((tid / 128) * G::TM_SET);
+    tm_p = tm_raw + (G::TMR ? 2 * N : 0);
+  }
+
   const int rank = CL == 1 ? 0 : int(cluster_rank());
   const int cid = blockIdx.x / CL;
   CT* const scr = reinterpret_cast<CT*>(p.scratch) + size_t(cid) * p.slot;
   CT* const FS = scr;               // f_hat [k_x][k_y][species 0 | 1][c]
-  CT* const H0 = FS + N3;           // x-passed half spectra [x][k_y][role][c], two buffers
-  CT* const PV = H0 + 2 * N3;       // product spectrum [x][row][c] (N form)
+  CT* const H0 = FS + N3;           // x-passed half spectra [x][k_y][role][c], NBH buffers
+  CT* const PV = H0 + G::NBH * N3;       // product spectrum [x][row][c] (N form)
   CT* const QA = PV + HN3;          // gain accumulators [k_x][row][c] (N form)
   CT* const QB = QA + HN3;
   T* const PS = reinterpret_cast<T*>(QB + HN3);  // parked P [x][z][y]
@@ -310,7 +408,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
           CT v[N];
 #pragma unroll
           for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + r * step);
-          shift_line<T, N>(v, pe + (kind == 0 ? 2 * N : 0) + role);
+          shift_line<T, N>(v, pe + (kind == 0 ? N : 0) + role);
           line_fft<T, N, +1>(v);
           group_sync<N, GP>();
 #pragma unroll
@@ -318,11 +416,11 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
           group_sync<N, GP>();
         }
         const CT* const row = tb + t * PITCH;
-        const CT cta = pe[5 * N], ctb = pe[5 * N + 1], txa = pe[5 * N + 2], txb = pe[5 * N + 3];
+        const CT cta = pe[2 * N], ctb = pe[2 * N + h];
         const CT a0 = row[0], b0 = row[h];
         Rows<T, N> y;
-        rows_c2r<N>(row, pe + 4 * N, mk<T>(a0.x, pe[4 * N + h].x * b0.x), mk<T>(cta.x * a0.y, ctb.x * b0.y), y);
-        const CT sc = kind == 0 ? mk<T>(txa.x, txb.x) : mk<T>(txa.y, txb.y);
+        rows_c2r<N>(row, pe + 2 * N, mk<T>(a0.x, pe[3 * N].x * b0.x), mk<T>(cta.x * a0.y, ctb.x * b0.y), y);
+        const CT sc = mk<T>(pe[kind == 0 ? 0 : N].y, pe[kind == 0 ? 1 : N + 1].y);
         if (!live) {
         } else if (kind == 0) {
 #pragma unroll
@@ -338,7 +436,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
         // step A of group k: x pass of this thread's pencils with the group's x phases
         if (k < tk.n_grp) {
           const GroupDesc gd = p.groups[tk.grp_off + k];
-          CT* const dst = H0 + size_t(k & 1) * N3;
+          CT* const dst = H0 + size_t(k % G::NBH) * N3;
           const CT* const phx = phb + gd.first * PB + role;
           for (int xl = grp; xl < G::PLANES; xl += GP) {
             const int r = plane0 + xl;
@@ -351,13 +449,19 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
             for (int n = 0; n < N; ++n) st2<T>(dst + n * N2 + r * N + t, v[n]);
           }
         }
+        // split barrier: step B of group k - 1 covers the other CTAs' lag in step A of group k
+        const bool halves = G::SPLIT && k > 0 && k < tk.n_grp;
+        if (halves) cluster_arrive();
         // step B of group k - 1: this group's planes
         if (k > 0) {
           const GroupDesc gd = p.groups[tk.grp_off + k - 1];
-          const CT* const src = H0 + size_t((k - 1) & 1) * N3;
+          const CT* const src = H0 + size_t((k - 1) % G::NBH) * N3;
           const bool fresh = k == 1, last = k == tk.n_grp;
           for (int xl = grp; xl < G::PLANES; xl += GP) {
             const int x = plane0 + xl;
+            if constexpr (G::PF) {
+              if (t == 0 && xl + GP < G::PLANES) prefetch_l2(src + size_t(x + GP) * N2, N2 * sizeof(CT));
+            }
             const T sgx = (x & 1) ? T(-1) : T(1), sgy = (t & 1) ? T(-1) : T(1);
             if constexpr (G::PSM) {
               if (fresh || !G::KEEP) {
@@ -365,27 +469,43 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
                 for (int z = 0; z < N; ++z) pb[z * N + t] = fresh ? T(0) : __ldcg(PS + size_t(x) * N2 + z * N + t);
               }
             } else {
-              if (fresh || !G::KEEP) {
+              if (fresh) {
 #pragma unroll
-                for (int z = 0; z < N; ++z) P[z] = fresh ? T(0) : __ldcg(PS + size_t(x) * N2 + z * N + t);
+                for (int z = 0; z < N; ++z) P[z] = T(0);
+              } else if constexpr (G::TMP) {
+                __syncwarp();
+                tm_load<N>(tm_p + uint32_t((xl / GP) * N), reinterpret_cast<float*>(P));
+              } else if constexpr (!G::KEEP) {
+#pragma unroll
+                for (int z = 0; z < N; ++z) P[z] = __ldcg(PS + size_t(x) * N2 + z * N + t);
               }
             }
             for (int e = gd.first; e < gd.first + gd.count; ++e) {
               const CT* const pe = phb + e * PB;
               const CT* const fc = FC + size_t(e) * G::FACE;
               // a shift of zero along an axis has no face there
-              const CT txa = pe[5 * N + 2], txb = pe[5 * N + 3];
-              const bool has_x = txa.x != T(0) || txb.x != T(0), has_y = txa.y != T(0) || txb.y != T(0);
-              const CT uy = has_y ? ld2<T>(fc + N2 + x * N + t) : mk<T>(0, 0);
-              const CT en = has_x ? ld2<T>(fc + 2 * N2 + t) : mk<T>(0, 0);
+              const T txa = pe[0].y, txb = pe[1].y, tya = pe[N].y, tyb = pe[N + 1].y;
+              const bool has_x = has_face<T>(pe), has_y = tya != T(0) || tyb != T(0);
+              const CT uy = has_y ? __ldca(fc + N2 + x * N + t) : mk<T>(0, 0);
+              const CT en = has_x ? __ldca(fc + 2 * N2 + t) : mk<T>(0, 0);
               {
                 CT v[N];
+                if (!G::TMR || e == gd.first) {
 #pragma unroll
-                for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + size_t(x) * N2 + r * N + t);
+                  for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + size_t(x) * N2 + r * N + t);
+                  if constexpr (G::TMR) {
+                    if (gd.count > 1) {
+                      __syncwarp();
+                      tm_store<2 * N>(tm_raw, reinterpret_cast<const float*>(v));
+                    }
+                  }
+                } else if constexpr (G::TMR) {
+                  __syncwarp();
+                  tm_load<2 * N>(tm_raw, reinterpret_cast<float*>(v));
+                }
                 const T corner = v[h].y;  // of column 0: f on the edge k_y = k_z = N/2
-                shift_line<T, N>(v, pe + 2 * N + role);
-                const CT txy = role == 0 ? txa : txb;
-                const T w = sgx * txy.x * txy.y;
+                shift_line<T, N>(v, pe + N + role);
+                const T w = sgx * (role == 0 ? txa * tya : txb * tyb);
                 v[h] = mk<T>(v[h].x - w * fe.x, v[h].y - w * fe.y);
                 line_fft<T, N, +1>(v);
                 group_sync<N, GP>();  // the previous entry's rows have been read
@@ -396,21 +516,27 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
                 group_sync<N, GP>();
               }
               const CT* const row = tb + t * PITCH;
-              const CT cta = pe[5 * N], ctb = pe[5 * N + 1];
+              const CT cta = pe[2 * N], ctb = pe[2 * N + h];
               const CT a0 = row[0], b0 = row[h];
               const CT m = mk<T>(cta.y * a0.y, ctb.y * b0.y);
               Rows<T, N> y;
-              rows_c2r<N>(row, pe + 4 * N, mk<T>(a0.x, pe[4 * N + h].x * b0.x),
-                          mk<T>(cta.x * a0.y - cta.y * (sgx * en.x + sgy * txa.y * tb[N].x),
-                                ctb.x * b0.y - ctb.y * (sgx * en.y + sgy * txb.y * tb[PITCH + N].x)),
+              rows_c2r<N>(row, pe + 2 * N, mk<T>(a0.x, pe[3 * N].x * b0.x),
+                          mk<T>(cta.x * a0.y - cta.y * (sgx * en.x + sgy * tya * tb[N].x),
+                                ctb.x * b0.y - ctb.y * (sgx * en.y + sgy * tyb * tb[PITCH + N].x)),
                           y);
 #pragma unroll
-              for (int z = 0; z < N; ++z) {
-                const CT ux = has_x ? ld2<T>(fc + z * N + t) : mk<T>(0, 0);
-                const CT im = face_sum(sgx, ux, sgy, uyb[z], (z & 1) ? mk<T>(-m.x, -m.y) : m);
-                const CT re = y.at(z);
-                if constexpr (G::PSM) pb[z * N + t] = fma_(-im.x, im.y, fma_(re.x, re.y, pb[z * N + t]));
-                else P[z] = fma_(-im.x, im.y, fma_(re.x, re.y, P[z]));
+              for (int z = 0; z < N; z += 2) {
+                CT uz[2];
+                load_two(uyb + z, uz[0], uz[1]);
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                  // read by every plane of the CTA: through L1
+                  const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
+                  const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
+                  const CT re = y.at(z + d);
+                  if constexpr (G::PSM) pb[(z + d) * N + t] = fma_(-im.x, im.y, fma_(re.x, re.y, pb[(z + d) * N + t]));
+                  else P[z + d] = fma_(-im.x, im.y, fma_(re.x, re.y, P[z + d]));
+                }
               }
             }
             if (last) {
@@ -448,6 +574,9 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
                   }
                 }
               }
+            } else if constexpr (G::TMP) {
+              __syncwarp();
+              tm_store<N>(tm_p + uint32_t((xl / GP) * N), reinterpret_cast<const float*>(P));
             } else if constexpr (!G::KEEP) {
 #pragma unroll
               for (int z = 0; z < N; ++z) {
@@ -458,7 +587,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
             }
           }
         }
-        cluster_sync<CL>();
+        if (halves) cluster_wait(); else cluster_sync<CL>();
       }
 
       // step C: x pass of the product spectrum, weights, accumulation
@@ -623,6 +752,12 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
       cluster_sync<CL>();
     }
   }
+  if constexpr (G::TM_ALLOC > 0) {
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (tid < 32) tc::tmem_dealloc(s_tmem, G::TM_ALLOC);
+  }
   // no CTA leaves while another may still read its shared memory (the last item index)
   if constexpr (CL > 1) cluster_sync<CL>();
   // every cluster has taken its last item once all have come here: the last one readies the counter
@@ -633,14 +768,16 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
   }
 }
 
-// dynamic shared memory of a shape; *ph_mode = 1 when the phase block of the current (task, rho) is
-// in it (while MINB CTAs still fit)
+// dynamic shared memory of a shape: the plane buffers and, while MINB CTAs still fit, the phase block
+// of the current (task, rho)
 template <typename T, int N, int W>
-size_t vhs_smem(const Plan& pl, int* ph_mode) {
+size_t vhs_smem(const Plan& pl, VhsShape& s) {
   using G = VGeo<T, N, W>;
-  const size_t ph_bytes = size_t(pl.max_ent) * G::PB * sizeof(C<T>);
-  *ph_mode = G::MINB * (G::SMEM + ph_bytes + 2048) <= size_t(226) * 1024 ? 1 : 0;
-  return G::SMEM + (*ph_mode ? ph_bytes : 0);
+  const size_t limit = size_t(226) * 1024 / G::MINB - 2048;  // per CTA while MINB CTAs still fit
+  const size_t ph_bytes = (size_t(pl.max_ent) * G::PB + 1) / 2 * 2 * sizeof(C<T>);
+  s.phase_smem = G::SMEM + ph_bytes <= limit ? 1 : 0;
+  const size_t used = G::SMEM + (s.phase_smem ? ph_bytes : 0);
+  return used;
 }
 
 inline void vhs_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cluster, int clusters, const VhsShape& s,
@@ -663,7 +800,7 @@ int vhs_configure_shape(Plan& pl) {
   auto kern = vhs_kernel<T, N, W>;
   VhsShape& s = pl.vhs[W];
   s.threads = G::THREADS;
-  s.smem = vhs_smem<T, N, W>(pl, &s.phase_smem);
+  s.smem = vhs_smem<T, N, W>(pl, s);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
     return DGFS_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
@@ -672,6 +809,34 @@ int vhs_configure_shape(Plan& pl) {
   if (cudaOccupancyMaxActiveClusters(&s.clusters, kern, &cfg) != cudaSuccess || s.clusters <= 0) {
     cudaGetLastError();
     return DGFS_ERR_CUDA;
+  }
+  if constexpr (G::TM_ALLOC > 0) {
+    // The occupancy calculator grants a kernel that allocates tensor memory one CTA per SM; the
+    // device co-schedules what registers, shared memory and threads allow.
+    cudaFuncAttributes fa;
+    int dev = 0, sms = 0;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return DGFS_ERR_CUDA;
+    if (G::CL > 1) {
+      // A CTA that waits for columns inside a cluster must not wait for another waiting cluster:
+      // each CTA asks for at least its columns' share of the SM's shared memory, so whatever mix of
+      // such kernels an SM holds, their columns fit.  (A kernel without clusters waits for nobody
+      // once it has its columns.)
+      const size_t least = (size_t(228) * 1024 * G::TM_ALLOC + 511) / 512 - 1024 - fa.sharedSizeBytes;
+      if (s.smem < least) s.smem = least;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
+        return DGFS_ERR_CUDA;
+    }
+    const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
+    int most = 65536 / (regs_warp * ((G::THREADS + 31) / 32));
+    const int by_smem = int(size_t(228) * 1024 / (s.smem + fa.sharedSizeBytes + 1024));
+    if (by_smem < most) most = by_smem;
+    if (2048 / G::THREADS < most) most = 2048 / G::THREADS;
+    if (512 / G::TM_ALLOC < most) most = 512 / G::TM_ALLOC;
+    if (most < 1) return DGFS_ERR_CUDA;
+    const int cap = most * sms / G::CL;
+    if (cap > s.clusters) s.clusters = cap;
   }
   return DGFS_OK;
 }

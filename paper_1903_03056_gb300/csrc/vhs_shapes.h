@@ -9,14 +9,14 @@ DGFS_VHS_SHAPE(float, 12, 1, 12, 1)
 DGFS_VHS_SHAPE(float, 16, 1, 8, 4)
 DGFS_VHS_SHAPE(float, 24, 1, 8, 2)
 DGFS_VHS_SHAPE(float, 32, 2, 4, 3)
-DGFS_VHS_SHAPE(float, 48, 8, 2, 4)
+DGFS_VHS_SHAPE(float, 48, 4, 4, 2)
 DGFS_VHS_SHAPE(double, 4, 1, 4, 1)
 DGFS_VHS_SHAPE(double, 6, 1, 6, 1)
 DGFS_VHS_SHAPE(double, 8, 1, 8, 1)
 DGFS_VHS_SHAPE(double, 12, 1, 12, 1)
 DGFS_VHS_SHAPE(double, 16, 1, 8, 1)
 DGFS_VHS_SHAPE(double, 24, 6, 4, 1)
-DGFS_VHS_SHAPE(double, 32, 8, 4, 2)
+DGFS_VHS_SHAPE(double, 32, 4, 4, 2)
 DGFS_VHS_SHAPE(double, 48, 4, 1, 1)
 
 // ... and how many times longer the wide shape takes per radial node on a full device (measured:
