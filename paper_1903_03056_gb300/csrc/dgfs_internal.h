@@ -38,11 +38,13 @@ struct TaskDesc {
   int out0, out1;
   int ent_off, n_ent;  // entries (sigma, weight) of this task
   int grp_off, n_grp;  // groups of entries sharing sigma_x
+  int any_zero;        // some group has sigma_x = 0
   int face_off, n_face;  // faces of the VHS kernel: entries with a shift along x or y
 };
 
 struct GroupDesc {
   int first, count;  // entry range within the task, all with the same sigma_x
+  int zero;          // 1 when that is 0: the x pass is the same for every radial node
 };
 
 struct KernelParams {

@@ -443,11 +443,19 @@ int build_plan(const dgfs_plan_desc* d, Plan& p) {
       for (int e = 1; e <= int(ent.size()); ++e) {
         if (e == int(ent.size()) || p.vss ||
             std::fabs(p.sigma[3 * ent[e].first] - p.sigma[3 * ent[first].first]) > 1e-12) {
-          p.groups.push_back({first, e - first});
+          p.groups.push_back({first, e - first, 0});
           first = e;
         }
       }
       tk.n_grp = int(p.groups.size()) - tk.grp_off;
+      tk.any_zero = 0;
+      for (int g = 0; g < tk.n_grp; ++g) {
+        GroupDesc& gd = p.groups[size_t(tk.grp_off) + g];
+        gd.zero = 1;
+        for (int e = gd.first; e < gd.first + gd.count; ++e)
+          if (p.sigma[3 * size_t(ent[e].first)] != 0.0) gd.zero = 0;
+        tk.any_zero |= gd.zero;
+      }
       tk.face_off = int(p.faces.size());
       for (size_t k = 0; k < ent.size(); ++k)
         for (int kind = 0; kind < 2; ++kind)

@@ -124,11 +124,11 @@ struct VGeo {
   // w_e), then (w_e, 0) and a pad.  Mode 0 needs no phase: its slot holds c + i t, the unpaired mode's
   static constexpr int PB = 3 * N + 2;
   // workspace per cluster (complex values): f_hat of both species, NBH buffers of x-passed
-  // half spectra of both roles, P_hat, two gain accumulators, parked P; then per entry the two faces
+  // half spectra of both roles, one more for the group with sigma_x = 0, P_hat, two gain accumulators, parked P; then per entry the two faces
   // and the k_x-face's k_z = N/2 line.  The same for every W of (T, N).
   static constexpr bool SPLIT = CL > 1 && (sizeof(T) == 8 || N >= 48);
   static constexpr int NBH = SPLIT ? 3 : 2;
-  static constexpr size_t SLOT = (1 + 3) * N3 + 4 * HN3;
+  static constexpr size_t SLOT = (2 + 3) * N3 + 4 * HN3;
   static constexpr size_t FACE = 2 * N2 + N;
 };
 
@@ -309,7 +309,8 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
   CT* const scr = reinterpret_cast<CT*>(p.scratch) + size_t(cid) * p.slot;
   CT* const FS = scr;               // f_hat [k_x][k_y][species 0 | 1][c]
   CT* const H0 = FS + N3;           // x-passed half spectra [x][k_y][role][c], NBH buffers
-  CT* const PV = H0 + G::NBH * N3;       // product spectrum [x][row][c] (N form)
+  CT* const HZ = H0 + G::NBH * N3;  // the same for the group with sigma_x = 0, kept for all radial nodes
+  CT* const PV = HZ + N3;       // product spectrum [x][row][c] (N form)
   CT* const QA = PV + HN3;          // gain accumulators [k_x][row][c] (N form)
   CT* const QB = QA + HN3;
   T* const PS = reinterpret_cast<T*>(QB + HN3);  // parked P [x][z][y]
@@ -359,6 +360,11 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
         line_fft<T, N, -1>(v);
 #pragma unroll
         for (int r = 0; r < N; ++r) st2<T>(FS + size_t(x) * N2 + r * N + t, v[r]);
+        // without a shift along x the x passes there and back cancel
+        if (tk.any_zero) {
+#pragma unroll
+          for (int r = 0; r < N; ++r) st2<T>(HZ + size_t(x) * N2 + r * N + t, scale<T>(v[r], T(1) / T(N2)));
+        }
       }
       group_sync<N, GP>();
     }
@@ -434,7 +440,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
 
       for (int k = 0; k <= tk.n_grp; ++k) {
         // step A of group k: x pass of this thread's pencils with the group's x phases
-        if (k < tk.n_grp) {
+        if (k < tk.n_grp && !p.groups[tk.grp_off + k].zero) {
           const GroupDesc gd = p.groups[tk.grp_off + k];
           CT* const dst = H0 + size_t(k % G::NBH) * N3;
           const CT* const phx = phb + gd.first * PB + role;
@@ -455,7 +461,9 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
         // step B of group k - 1: this group's planes
         if (k > 0) {
           const GroupDesc gd = p.groups[tk.grp_off + k - 1];
-          const CT* const src = H0 + size_t((k - 1) % G::NBH) * N3;
+          const bool zero = gd.zero != 0;
+          const CT* const src = zero ? HZ : H0 + size_t((k - 1) % G::NBH) * N3;
+          const int col = zero && self ? c : t;  // (a self pair's roles share the unshifted columns)
           const bool fresh = k == 1, last = k == tk.n_grp;
           for (int xl = grp; xl < G::PLANES; xl += GP) {
             const int x = plane0 + xl;
@@ -492,7 +500,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) v
                 CT v[N];
                 if (!G::TMR || e == gd.first) {
 #pragma unroll
-                  for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + size_t(x) * N2 + r * N + t);
+                  for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + size_t(x) * N2 + r * N + col);
                   if constexpr (G::TMR) {
                     if (gd.count > 1) {
                       __syncwarp();
