@@ -33,8 +33,8 @@ int launch_core(dgfs::Plan& p, const void* f, void* Q, int batch, cudaStream_t s
   const size_t n3 = size_t(p.N) * p.N * p.N;
   void* Qfull = sum ? static_cast<char*>(p.d_Qfull) + size_t(stage_node) * p.s * p.s * n3 * dgfs::real_size(p) : Q;
   auto* const run = p.precision == DGFS_BF16X3 ? dgfs::launch_bf16x3
-                    : p.precision == DGFS_FP32 ? (p.vss ? dgfs::launch_f32 : dgfs::launch_vhs_f32)
-                                               : (p.vss ? dgfs::launch_f64 : dgfs::launch_vhs_f64);
+                    : p.precision == DGFS_FP32 ? (p.vss ? dgfs::launch_vss_f32 : dgfs::launch_f32)
+                                               : (p.vss ? dgfs::launch_vss_f64 : dgfs::launch_f64);
   int rc = run(p, f, Qfull, batch, st, ws);
   if (rc != DGFS_OK) return rc;
   *launches += 1;
@@ -103,8 +103,8 @@ int dgfs_create_plan(const dgfs_plan_desc* desc, dgfs_plan* out) {
   if (rc == DGFS_OK && cudaGetDevice(&p.device) != cudaSuccess) rc = DGFS_ERR_CUDA;
   if (rc == DGFS_OK)
     rc = p.precision == DGFS_BF16X3 ? dgfs::configure_bf16x3(p)
-         : p.precision == DGFS_FP32 ? (p.vss ? dgfs::configure_f32(p) : dgfs::configure_vhs_f32(p))
-                                    : (p.vss ? dgfs::configure_f64(p) : dgfs::configure_vhs_f64(p));
+         : p.precision == DGFS_FP32 ? (p.vss ? dgfs::configure_vss_f32(p) : dgfs::configure_f32(p))
+                                    : (p.vss ? dgfs::configure_vss_f64(p) : dgfs::configure_f64(p));
   if (rc == DGFS_OK) rc = dgfs::upload_plan(p);
   if (rc != DGFS_OK) {
     dgfs::free_plan(p);

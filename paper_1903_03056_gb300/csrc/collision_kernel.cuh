@@ -1,316 +1,392 @@
-// Persistent collision kernel: one thread-block cluster per work item (node b, task).
+// Persistent collision kernel: one thread-block cluster per work item (node b, task), on real
+// transforms.
 //
-// For a task (i, j) the cluster evaluates, for every radial node rho_q (Sec. 4):
+// Only Re Q is wanted, and for VHS (alpha = 1) the gain weight F(k, rho) and the loss weight G^-(k) are real
+// and even in k, so Q_ij = IDFT(sum_rho w F DFT(Re P_rho)) - f_i IDFT(G^- f_hat_j) holds with the
+// real part of the products alone:
 //
-//   step A  pencil pass along x: for the entries of one sigma_x group, the spectra
-//           f_hat_i e^{+i pi rho c_j k_x sigma_x / L} and f_hat_j e^{-i pi rho c_i k_x sigma_x / L}
-//           are inverse-transformed along x (the x phase is shared by the group);
-//   step B  plane pass over (y, z): per entry, the y and z phases are applied, the inverse
-//           transforms along y and z finish a_e and b_e on the plane, and
-//           P += w_e a_e b_e accumulates in registers (entries with the previous entry's
-//           sigma_y reuse its y pass where a third plane buffer fits); after the last group
-//           P is transformed forward along z and y;
-//   step C  pencil pass along x: forward transform of P, then Q_hat^+_(ij) += w_rho F^(ij) P_hat
-//           (and Q_hat^+_(ji) += w_rho F^(ji) P_hat for a cross pair).
+//     Re P = sum_e w_e (Re a_e Re b_e - Im a_e Im b_e).
 //
-// then finishes Q_ij = Re IFFT(Q_hat^+_ij) - f_i Re IFFT(G^(ij)- f_hat_j) (the loss
-// convolution of Sec. 4) and writes it.  The 3D transforms are split into a pencil pass
-// (x, strided by N^2) and a plane pass (y, z, contiguous), each line transformed in the
-// registers of one thread; the planes of a volume are spread over the cluster's CTAs and the
-// pencils likewise, with cluster barriers between passes.  The volumes live in a per-cluster
-// workspace accessed through L2 only; when the workspaces of all resident clusters exceed L2
-// (N >= 24) part of them streams through HBM, and each plane is prefetched into L2 one read
-// ahead of its use.
+// f is real, so the shifted copies a_e, b_e would be real too but for the unpaired modes at index
+// N/2 of an axis: there the phase e^{i theta k} has no conjugate partner and leaves
+// c + i t = cos - i sin of theta N / 2.  Write the shift along one axis as R + i t Pi, R the
+// real shift (phase c at the unpaired mode) and Pi the projection on that mode, an alternating
+// sequence.  The product over the three axes gives
+//
+//     Re a = RxRyRz f - ty tz RxPyPz f - tx tz PxRyPz f - tx ty PxPyRz f
+//     Im a = tx PxRyRz f + ty RxPyRz f + tz RxRyPz f - tx ty tz PxPyPz f.
+//
+// Every term but the first lives on faces or edges of the mode cube, so a shifted copy costs one
+// real 3D transform and two real 2D ones (the faces k_x = N/2 and k_y = N/2; the face k_z = N/2
+// falls out of the y pass, see below) instead of a complex 3D transform: half the arithmetic and
+// half the workspace.
+//
+// Layouts.  A spectrum keeps columns c = 0..N/2-1 of the z modes; column 0 holds
+// X(k_z = 0) + i X(k_z = N/2) ("C form": every x and y pass is linear and maps each part to
+// itself, so the pair travels as one complex line).  Rows of N complex values hold two such half
+// rows: role 0 (species i, shift +) and role 1 (species j, shift -).  After the inverse y pass
+// column 0 is (a(k_z = 0), a(k_z = N/2)), two real numbers.  The product's spectrum splits column
+// 0 over k_y instead ("N form", row r of column 0: r = 1..N/2-1 is (k_y = r, k_z = 0), N/2 + r is
+// (k_y = r, k_z = N/2), row 0 holds X(0,0) + i X(N/2,0) and row N/2 holds X(0,N/2) + i X(N/2,N/2)),
+// since there the weights of the two parts differ.
+//
+// Per radial node the phases run as a pipeline over sigma_x groups: phase 0 transforms the faces of
+// all entries and runs step A of group 0; phase k runs step A of group k and step B of group
+// k - 1; one cluster barrier each.
+//   step A  x pass of both roles' half spectra (one thread per pencil, coalesced)
+//   step B  per plane x and entry: y phases, y pass of N/2 columns of either role (one line per
+//           thread), transpose through shared memory, z phases and the real z transform of both
+//           roles (one row per thread), and the product into P, N real values per thread
+//   step C  after the last group: P -> spectrum, Q_hat_ij += F_ij P_hat (and Q_hat_ji for a cross pair)
+//
+// VSS (alpha != 1, W = 2): F depends on sigma and is complex, so every entry's product, now complex
+// (Im a Re b + Re a Im b beside the real part), is transformed forward by itself in step B, and step C
+// runs two phases behind step A, entry by entry, on the half space of its Hermitian part (vss_step_c).
+// Groups hold one or two entries.
+//
+// Measured on the GB300 against the complex-transform kernel this one replaced: 4096 nodes of N = 32
+// FP32 285 -> 144.6 ms, 3001 of N = 24 75.1 -> 36.5, 8192 of N = 16 28.7 -> 16.2, 61 three-species nodes
+// of N = 48 86.0 -> 36.0, 61 nodes of N = 32 FP64 201 -> 85.7, VSS 37 three-species nodes of N = 48
+// (M = 32) 339 -> 161 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
+// FMA pipes run half their cycles (N = 16: the L1 data path three quarters), the stalls are L2 loads
+// of the x-passed spectra, whose workspaces together exceed L2 from N = 24 on.
 #pragma once
+
+#include <cmath>
 
 #include <cuda_runtime.h>
 
 #include "dgfs_internal.h"
-#include "fft_line.cuh"
 #include "group_sync.cuh"
+#include "real_line.cuh"
 #include "tcgen05.cuh"
 
 namespace dgfs {
 
-// compile-time launch shape per (precision, N): cluster size, plane groups per CTA, CTAs per SM
-template <typename T, int N> struct Shape;
-#define DGFS_SHAPE3(TT, NN, CC, GG, MB)                              \
-  template <> struct Shape<TT, NN> {                                 \
-    static constexpr int cluster = CC;                               \
-    static constexpr int groups = GG;                                \
-    static constexpr int min_blocks = MB;                            \
+// Launch shape per (precision, N, W): cluster size, plane groups per CTA, CTAs per SM the registers
+// are sized for.  W = 0 serves batches that fill the device; W = 1, where it differs, spreads one
+// work item over more SMs for small batches (one plane per group, clusters of 4 to 8 CTAs).
+template <typename T, int N, int W> struct VShape : VShape<T, N, 0> {};
+template <typename T, int N> struct HasWide {
+  static constexpr bool value = false;
+  static constexpr double slow = 1.0;
+};
+#define DGFS_SHAPE3(TT, NN, CC, GG, MB)   \
+  template <> struct VShape<TT, NN, 0> {     \
+    static constexpr int cluster = CC;       \
+    static constexpr int groups = GG;        \
+    static constexpr int min_blocks = MB;    \
   };
-#define DGFS_SHAPE(TT, NN, CC, GG) DGFS_SHAPE3(TT, NN, CC, GG, 1)
+#define DGFS_VSS(TT, NN, CC, GG, MB)   \
+  template <> struct VShape<TT, NN, 2> {     \
+    static constexpr int cluster = CC;       \
+    static constexpr int groups = GG;        \
+    static constexpr int min_blocks = MB;    \
+  };
+#define DGFS_WIDE(TT, NN, CC, GG, MB, SLOW)    \
+  template <> struct VShape<TT, NN, 1> {     \
+    static constexpr int cluster = CC;       \
+    static constexpr int groups = GG;        \
+    static constexpr int min_blocks = MB;    \
+  };                                         \
+  template <> struct HasWide<TT, NN> {       \
+    static constexpr bool value = true;      \
+    static constexpr double slow = SLOW;     \
+  };
 #include "tuned_shapes.h"
-#undef DGFS_SHAPE
 #undef DGFS_SHAPE3
+#undef DGFS_WIDE
+#undef DGFS_VSS
 
-template <typename T, int N>
-struct Geo {
-  static constexpr int N2 = N * N;
-  static constexpr int N3 = N * N * N;
-  static constexpr int PITCH = N + 1;  // padded smem row (complex elements)
-  // P accumulates in registers when a second line of N complex values still fits (FP32 up to
-  // N = 48: ~50 bytes of spills there, and one plane buffer per group less; measured 8-10 %
-  // faster than P in shared memory at N = 48)
-  static constexpr bool PREG = (sizeof(T) == 4 && N <= 48) || N <= 16;
-  static constexpr int CL = Shape<T, N>::cluster;
-  static constexpr int GP = Shape<T, N>::groups;
-  static constexpr int MINB = Shape<T, N>::min_blocks;  // CTAs per SM the registers are sized for
+template <typename T, int N, int W>
+struct VGeo {
+  static constexpr int h = N / 2;
+  static constexpr int N2 = N * N, HN2 = N * h;
+  static constexpr size_t N3 = size_t(N) * N * N, HN3 = size_t(N) * HN2;
+  static constexpr int PITCH = N + 1;
+  static constexpr int CL = VShape<T, N, W>::cluster;
+  static constexpr int GP = VShape<T, N, W>::groups;
+  static constexpr int MINB = VShape<T, N, W>::min_blocks;
   static constexpr int THREADS = GP * N;
-  static constexpr int PLANES = N / CL;       // planes per CTA
-  static constexpr int PENCILS = N2 / CL;     // pencils per CTA
-  static_assert(PLANES % GP == 0, "planes must split evenly over plane groups");
-  static_assert(N2 % CL == 0, "pencils must split evenly over the cluster");
-  static constexpr size_t BUF = size_t(N) * PITCH * sizeof(C<T>);  // one padded plane
-  // CTAs an SM holds at once: the register budget's count, or two when a CTA of at most 128
-  // threads (at up to 256 registers each) and two plane buffers per group leave room
-  static constexpr int RES =
-      MINB > 1 ? MINB : (THREADS <= 128 && 2 * (GP * 2 * BUF + 1024) <= 228 * 1024 ? 2 : 1);
-  // y-pass sharing: entries of a group with equal sigma_y reuse the y pass of both shifted
-  // volumes, kept in a transpose buffer per role; needs P in registers and a third buffer per
-  // group that still leaves RES CTAs per SM with 8 KB for the z phases.  Measured on the
-  // 8192-node N = 16 batch: FP32 -4 %, FP64 -11 %; at N = 24 and 32 the third buffer takes
-  // the room of the phase block and of L1 and the kernel ran 5-8 % slower, so it stays off.
-  static constexpr bool YSH = N <= 16 && PREG && RES * (GP * 3 * BUF + 1024 + 8 * 1024) <= 228 * 1024;
-  // Tensor-memory accumulators: the sigma sum P of each of a group's planes and the role-0 line
-  // a_e live in TMEM columns (2N FP32 columns per line) instead of registers and shared memory,
-  // which leaves the registers to the line transform and keeps P on chip across the sigma_x
-  // groups of a radial node.  FP32, groups of one whole warp and at most 128 threads (each
-  // thread owns one TMEM lane), and the allocations of the CTAs an SM holds within its 512
-  // columns.
-  static constexpr int PPG = PLANES / GP;  // planes per group
-  static constexpr int TM_COLS = 2 * N * (PPG + 1);
-  static constexpr int TM_ALLOC =
-      TM_COLS <= 32 ? 32 : TM_COLS <= 64 ? 64 : TM_COLS <= 128 ? 128 : TM_COLS <= 256 ? 256 : 512;
-  static constexpr bool TM = sizeof(T) == 4 && N % 32 == 0 && THREADS <= 128 && !YSH &&
-                             TM_COLS <= 512 && RES * TM_ALLOC <= 512;
-  // smem planes per plane group: transpose (role 0), a, then P (!PREG) or the role-1 transpose;
-  // with TMEM accumulators the transpose buffer only
-  static constexpr int NBUF = TM ? 1 : (PREG && !YSH) ? 2 : 3;
-  static constexpr size_t SMEM = size_t(GP) * NBUF * BUF;
-  // L2 prefetch of the workspace reads (measured: a gain from N = 24 on, where the clusters'
-  // workspaces together exceed L2; a loss at N = 16); bulk prefetches need whole 16-byte rows
-  static constexpr bool PF = N >= 24 && (PENCILS * sizeof(C<T>)) % 16 == 0;
-  // staged plane pass (step B): the two plane buffers of a group take turns receiving the next
-  // shifted plane by a bulk copy, issued one (entry, role) ahead of its use, so the plane's
-  // L2/HBM latency overlaps the transforms of the previous role instead of stalling the loads
-  // (P in registers, no y-pass sharing or TMEM accumulators, N >= 24; a plane is a whole
-  // number of 16-byte rows)
-  static constexpr bool STAGE = !TM && PREG && !YSH && N >= 24 && (N2 * sizeof(C<T>)) % 16 == 0 && (BUF % 16) == 0;
-  // Buffers of the shifted-volume pair: three for clusters of several CTAs, whose VHS phases
-  // split the cluster barrier (a CTA arrives when its step A is written and waits at the end
-  // of the phase, so a CTA may still read pair k-1 while another writes pair k+1), two otherwise.
-  // Measured at N = 32: 2-CTA clusters 2.6 % faster with the split; the TMEM shape (8-CTA
-  // clusters) as fast without it, and the third buffer raised its DRAM traffic from 28 to 45 GB
-  // per 288-node launch (L2 hit rate 86 % -> 74 %), so TMEM shapes keep two.
-  static constexpr int NBV = CL > 1 && !TM ? 3 : 2;
-  // workspace volumes per cluster: f_hat_i, f_hat_j, the NBV pairs of shifted volumes, two P
-  // volumes (the second used by the VSS pipeline), two gain accumulators
-  static constexpr int SLOT = 2 + 2 * NBV + 4;
+  static constexpr int PLANES = N / CL;  // planes, and rows of pencils, per CTA
+  static_assert(N % CL == 0 && PLANES % GP == 0, "planes must split evenly over the cluster and its plane groups");
+  // P of a plane stays in the row's thread (FP64 N = 48: in shared memory, its line alone fills
+  // the registers); with one plane per group it lives there for the whole radial node, otherwise
+  // it is parked in the workspace between sigma_x groups
+  static constexpr bool PSM = sizeof(T) == 8 && N >= 48 && W != 2;
+  // W = 2: VSS (sigma-dependent weights).  Groups hold one or two entries; each entry's product is
+  // complex and transformed forward by itself
+  static constexpr bool VSS = W == 2;
+  static constexpr bool KEEP = PLANES == GP;
+  // L2 prefetch of a group's next plane one plane ahead (measured: N = 32 -1.8 %, 48 -0.8 %, smaller
+  // grids, whose workspaces mostly stay in L2, +0.5 to 1.4 %)
+  static constexpr bool PF = sizeof(T) == 4 && N >= 32;
+  // Tensor memory (FP32): each thread owns a lane, TMEM holds its raw line of the current plane (read
+  // once per sigma_x group, used by every entry of it) and the parked P of its planes.  Neither then
+  // goes through L2 or the L1 data path again.  Used while the CTAs an SM holds fit its 512 columns.
+  static constexpr int PPG = PLANES / GP;
+  static constexpr int SETS = (THREADS + 127) / 128;  // warps that share a lane quarter
+  static constexpr int alloc_of(int cols) { return cols <= 32 ? 32 : cols <= 64 ? 64 : cols <= 128 ? 128 : cols <= 256 ? 256 : 512; }
+  static constexpr bool fits(int cols) { return cols > 0 && cols <= 512 && MINB * alloc_of(cols) <= 512; }
+  static constexpr bool TMOK = sizeof(T) == 4 && N % 8 == 0 && N >= 16 && N <= 32 && THREADS % 32 == 0 && W == 0;
+  static constexpr int P_COLS = KEEP ? 0 : PPG * N;
+  static constexpr bool TMP = TMOK && !KEEP && fits(SETS * P_COLS);
+  static constexpr bool TMR = TMOK && fits(SETS * (2 * N + (TMP ? P_COLS : 0)));
+  static constexpr int TM_SET = (TMR ? 2 * N : 0) + (TMP ? P_COLS : 0);  // columns of a thread
+  static constexpr int TM_ALLOC = TM_SET > 0 ? alloc_of(SETS * TM_SET) : 0;
+  // shared memory per group: one padded plane, the entry's row of the k_y face, P if PSM
+  // (FP32: the groups' stride is 2 N words modulo 32, so that the lanes of a warp that spans two
+  // groups hit distinct banks: N = 24)
+  static constexpr size_t GROUP_BASE = (size_t(N) * PITCH + N) * sizeof(C<T>) + (PSM ? N2 * sizeof(T) : 0);
+  static constexpr size_t GROUP_BYTES =
+      GROUP_BASE + (sizeof(T) == 4 ? size_t((2 * N + 32 - int(GROUP_BASE / 4 % 32)) % 32) * 4 : 0);
+  static_assert(GROUP_BYTES % 16 == 0, "16-byte accesses");
+  static constexpr size_t SMEM = GP * GROUP_BYTES;
+  // phase block of an entry (complex values): x [h][role], y [h][role], z [role][h] (role 1 times
+  // w_e), then (w_e, 0) and a pad.  Mode 0 needs no phase: its slot holds c + i t, the unpaired mode's
+  static constexpr int PB = 3 * N + 2;
+  // workspace per cluster (complex values): f_hat of both species, NBH buffers of x-passed
+  // half spectra of both roles, one more for the group with sigma_x = 0, P_hat, two gain accumulators, parked P; then per entry the two faces
+  // and the k_x-face's k_z = N/2 line.  The same for every W of (T, N).
+  static constexpr bool SPLIT = CL > 1 && (sizeof(T) == 8 || N >= 48) && !VSS;
+  static constexpr int NBH = SPLIT ? 3 : 2;
+  // VSS: complex product spectra [x][k_y][k_z] of up to two entries a group, double buffered, and
+  // accumulators per k_x: pencils [k_y][0..N/2], then (k_y = N/2, k_z = N/2+1..N-1)
+  static constexpr size_t PVN = VSS ? 4 * N3 : HN3;
+  static constexpr int QROW = VSS ? N * (h + 1) + h - 1 : HN2;
+  static constexpr size_t QN = VSS ? (size_t(N) * QROW + 1) / 2 * 2 : HN3;
+  static constexpr size_t SLOT = VSS ? (2 + 2) * N3 + PVN + 2 * QN : (2 + 3) * N3 + 4 * HN3;
+  static constexpr size_t FACE = 2 * N2 + N;
 };
 
-// transpose a plane held as column t (x[r] = V[r][t]) into row t (x[c] = V[t][c]) and back
-template <typename T, int N, int GP>
-__device__ __forceinline__ void cols_to_rows(C<T> (&x)[N], C<T>* tb, int t) {
-  constexpr int P = N + 1;
+// v[n] *= e^{i theta k_n}, ph[2 n] the phase of mode n: mode -n (entry N - n) takes its conjugate, the
+// unpaired mode the real factor c, mode 0 none
+template <typename T, int N>
+__device__ __forceinline__ void shift_line(C<T> (&v)[N], const C<T>* ph) {
+  v[N / 2] = scale<T>(v[N / 2], ph[0].x);
 #pragma unroll
-  for (int r = 0; r < N; ++r) tb[r * P + t] = x[r];
-  group_sync<N, GP>();
-#pragma unroll
-  for (int c = 0; c < N; ++c) x[c] = tb[t * P + c];
-  group_sync<N, GP>();
-}
-template <typename T, int N, int GP>
-__device__ __forceinline__ void rows_to_cols(C<T> (&x)[N], C<T>* tb, int t) {
-  constexpr int P = N + 1;
-#pragma unroll
-  for (int c = 0; c < N; ++c) tb[t * P + c] = x[c];
-  group_sync<N, GP>();
-#pragma unroll
-  for (int r = 0; r < N; ++r) x[r] = tb[r * P + t];
-  group_sync<N, GP>();
+  for (int n = 1; n < N / 2; ++n) {
+    const C<T> f = ph[2 * n], a = v[n], b = v[N - n];
+    v[n] = mk<T>(a.x * f.x - a.y * f.y, a.x * f.y + a.y * f.x);
+    v[N - n] = mk<T>(b.x * f.x + b.y * f.y, b.y * f.x - b.x * f.y);
+  }
 }
 
-// A line of N complex FP32 values in 2N consecutive TMEM columns of the thread's lane (16
-// columns per access; every thread of the warp takes part).  The load waits for its data inside
-// the same asm statement, so no use of the registers can move ahead of the wait.
-__device__ __forceinline__ void tm_ld16w(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];\n\ttcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
+// whether an entry (phase block pe) has a shift along x, and with it a k_x face
+template <typename T> __device__ __forceinline__ bool has_face(const C<T>* pe) { return pe[0].y != T(0) || pe[1].y != T(0); }
+
+// two neighbouring complex values (index i even) with one 16-byte access
+__device__ __forceinline__ void load_two(const float2* p, float2& a, float2& b) {
+  const float4 q = *reinterpret_cast<const float4*>(p);
+  a = make_float2(q.x, q.y);
+  b = make_float2(q.z, q.w);
+}
+__device__ __forceinline__ void load_two(const double2* p, double2& a, double2& b) {
+  a = p[0];
+  b = p[1];
+}
+
+// Real rows of both roles of a plane.  In FP32 the roles run packed, one register pair per value:
+// the two transforms share every twiddle, so one instruction serves both.
+template <typename T, int N> struct Rows {
+  T a[N], b[N];
+  // a_z, b_z
+  __device__ __forceinline__ C<T> at(int z) const { return mk<T>(a[z], b[z]); }
+};
+template <int N> struct Rows<float, N> {
+  F2 v[N];
+  __device__ __forceinline__ float2 at(int z) const { return unpack2(v[z]); }
+};
+
+// z transform of a row of both roles (row: role 0, row + N/2: role 1) with the z phases phz (null:
+// none), x0 and xh the values (role 0, role 1) of modes 0 and N/2
+template <int N>
+__device__ __forceinline__ void rows_c2r(const float2* row, const float2* phz, float2 x0, float2 xh, Rows<float, N>& y) {
+  constexpr int h = N / 2;
+  C2 x[h];
+  float2 fa[2], fb[2];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int k = 1; k < h; ++k) {
+    float2 a = row[k], b = row[h + k];
+    if (phz != nullptr) {
+      if constexpr (h % 2 == 0) {  // the phases two at a time (every block starts on 16 bytes)
+        if (k == 1 || k % 2 == 0) {
+          load_two(phz + (k & ~1), fa[0], fa[1]);
+          load_two(phz + h + (k & ~1), fb[0], fb[1]);
+        }
+        a = cmul<float>(a, fa[k & 1]);
+        b = cmul<float>(b, fb[k & 1]);
+      } else {
+        a = cmul<float>(a, phz[k]);
+        b = cmul<float>(b, phz[h + k]);
+      }
+    }
+    x[k].x = pack2(a.x, b.x);
+    x[k].y = pack2(a.y, b.y);
+  }
+  c2r_line<F2, N>(x, pack2(x0.x, x0.y), pack2(xh.x, xh.y), y.v);
 }
 template <int N>
-__device__ __forceinline__ void tm_store_line(uint32_t ta, const C<float> (&v)[N]) {
+__device__ __forceinline__ void rows_c2r(const double2* row, const double2* phz, double2 x0, double2 xh,
+                                         Rows<double, N>& y) {
+  constexpr int h = N / 2;
+  double2 x[h];
 #pragma unroll
-  for (int ch = 0; ch < N / 8; ++ch) {
-    float f[16];
+  for (int k = 1; k < h; ++k) x[k] = phz != nullptr ? cmul<double>(row[k], phz[k]) : row[k];
+  c2r_line<double, N>(x, x0.x, xh.x, y.a);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      f[2 * j] = v[8 * ch + j].x;
-      f[2 * j + 1] = v[8 * ch + j].y;
-    }
-    tc::tmem_st16(ta + uint32_t(16 * ch), f);
-  }
-}
-template <int N>
-__device__ __forceinline__ void tm_load_line(uint32_t ta, C<float> (&v)[N]) {
-#pragma unroll
-  for (int ch = 0; ch < N / 8; ++ch) {
-    float f[16];
-    tm_ld16w(ta + uint32_t(16 * ch), f);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v[8 * ch + j] = mk<float>(f[2 * j], f[2 * j + 1]);
-  }
+  for (int k = 1; k < h; ++k) x[k] = phz != nullptr ? cmul<double>(row[h + k], phz[h + k]) : row[h + k];
+  c2r_line<double, N>(x, x0.y, xh.y, y.b);
 }
 
-// v[r] *= ph[r] for a phase array of N complex values.  Every phase array starts on a multiple
-// of N complex values (N even), so FP32 phases can be read two at a time with 16-byte loads
-// (broadcast reads: the arrays are the same for every thread of a group).  Measured: 1.3 % and
-// 0.8 % faster at N = 24 and 16; at N = 32 and 48 the line transform's register allocation
-// came out 2-3 % slower, so there the phases are read one at a time.
-template <typename T, int N>
-__device__ __forceinline__ void mul_phases(C<T> (&v)[N], const C<T>* ph) {
-  if constexpr (sizeof(T) == 4 && N % 2 == 0 && N <= 24) {
-#pragma unroll
-    for (int r = 0; r < N; r += 2) {
-      const float4 q = *reinterpret_cast<const float4*>(ph + r);
-      v[r] = cmul<T>(v[r], mk<T>(q.x, q.y));
-      v[r + 1] = cmul<T>(v[r + 1], mk<T>(q.z, q.w));
-    }
+__device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_(double a, double b, double c) { return fma(a, b, c); }
+
+// (s u + t w) + m in both halves
+__device__ __forceinline__ float2 face_sum(float s, float2 u, float t, float2 w, float2 m) {
+  return unpack2(fma2(pack2(s, s), pack2(u.x, u.y), fma2(pack2(t, t), pack2(w.x, w.y), pack2(m.x, m.y))));
+}
+__device__ __forceinline__ double2 face_sum(double s, double2 u, double t, double2 w, double2 m) {
+  return make_double2(fma(s, u.x, fma(t, w.x, m.x)), fma(s, u.y, fma(t, w.y, m.y)));
+}
+__device__ __forceinline__ float2 mul_each(float2 s, float2 v) { return unpack2(pack2(s.x, s.y) * pack2(v.x, v.y)); }
+__device__ __forceinline__ double2 mul_each(double2 s, double2 v) { return make_double2(s.x * v.x, s.y * v.y); }
+
+// Gain of one mode: Q_hat (+)= F P_hat.  A work item split over its radial nodes adds them up later
+// with these operations in the same order, so it gives the same bits.
+template <typename T>
+__device__ __forceinline__ C<T> add_gain(C<T> acc, T f, C<T> v, bool first) {
+  return first ? scale<T>(v, f) : mk<T>(fma_(v.x, f, acc.x), fma_(v.y, f, acc.y));
+}
+// a mode of two real pencils held as one, p_0 + i p_h with weights fa, fh: v its value, m that of -k_x
+template <typename T>
+__device__ __forceinline__ C<T> add_gain_pair(C<T> acc, T fa, T fh, C<T> v, C<T> m, bool first) {
+  const T fp = T(0.5) * (fa + fh), fm = T(0.5) * (fa - fh);
+  const C<T> w = mk<T>(fma_(fm, m.x, fp * v.x), fma_(-fm, m.y, fp * v.y));
+  return first ? w : add<T>(w, acc);
+}
+
+// n consecutive TMEM columns of the thread's lane (n a multiple of 8; every thread of the warp takes
+// part).  A load waits for its data inside its asm statement; a store is waited for at once, since the
+// next access of these columns may come soon.
+template <int n>
+__device__ __forceinline__ void tm_load(uint32_t ta, float* v) {
+  if constexpr (n >= 32) {
+    tc::tmem_ld32w(ta, v);
+    if constexpr (n > 32) tm_load<n - 32>(ta + 32, v + 32);
+  } else if constexpr (n >= 16) {
+    tc::tmem_ld16w(ta, v);
+    if constexpr (n > 16) tm_load<n - 16>(ta + 16, v + 16);
   } else {
-#pragma unroll
-    for (int r = 0; r < N; ++r) v[r] = cmul<T>(v[r], ph[r]);
+    tc::tmem_ld8w(ta, v);
   }
 }
-
-// Two-pass transform of a plane: the first line pass, the transpose (columns to rows when
-// COLS_FIRST, rows to columns otherwise), an optional per-element phase, the second line pass.
-// For N >= 32 the passes run as a two-trip loop over one copy of the unrolled line transform,
-// which keeps the kernel's instruction footprint small (measured: +3% at N = 32 and 48); the
-// smaller transforms are faster unrolled.
-template <typename T, int N, int GP, int DIR, bool COLS_FIRST>
-__device__ __forceinline__ void plane_pass2(C<T> (&v)[N], C<T>* tb, int t, const C<T>* ph2) {
-  auto between = [&]() {
-    if constexpr (COLS_FIRST) cols_to_rows<T, N, GP>(v, tb, t); else rows_to_cols<T, N, GP>(v, tb, t);
-    if (ph2 != nullptr) mul_phases<T, N>(v, ph2);
-  };
-  if constexpr (N >= 32) {
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      if (pass == 1) between();
-      fft_line<T, N, DIR>(v);
-    }
+template <int n>
+__device__ __forceinline__ void tm_store_part(uint32_t ta, const float* v) {
+  if constexpr (n >= 16) {
+    tc::tmem_st16p(ta, v);
+    if constexpr (n > 16) tm_store_part<n - 16>(ta + 16, v + 16);
   } else {
-    fft_line<T, N, DIR>(v);
-    between();
-    fft_line<T, N, DIR>(v);
+    tc::tmem_st8(ta, v);
   }
 }
-
-template <typename T, int N>
-__device__ __forceinline__ const C<T>* phase_ptr(const KernelParams& p, int task, int q, int e,
-                                                  int role, int axis) {
-  const C<T>* ph = reinterpret_cast<const C<T>*>(p.phase);
-  return ph + ((((size_t(task) * p.n_rho + q) * p.max_ent + e) * 2 + role) * 3 + axis) * N;
+template <int n>
+__device__ __forceinline__ void tm_store(uint32_t ta, const float* v) {
+  tm_store_part<n>(ta, v);
+  tc::tmem_wait_st();
 }
 
-template <typename T, int N>
-__global__ void __launch_bounds__(Geo<T, N>::THREADS, Geo<T, N>::MINB) collision_kernel(const KernelParams p) {
-  using G = Geo<T, N>;
+// Step C of one VSS entry: x pass of its complex product spectrum P_hat and Q_hat += F P_hat.  Only the
+// real part of IDFT(Q_hat) is wanted, that is Herm(Q_hat)(k) = (Q_hat(k) + conj Q_hat(-k)) / 2, so the half
+// space k_z = 0..N/2 is enough.  F(-k) = conj F(k) except where k has an unpaired mode N/2: a pencil
+// (k_y, k_z) off those faces needs Herm(P_hat) alone, adds its partner (-k_y, -k_z) before the transform,
+// and weights only its element k_x = N/2 apart (two alternating sums over x).  The pencils with k_y or
+// k_z = N/2 keep Q_hat itself, partner included, until the finish.
+template <typename T, int N, int W>
+__device__ __forceinline__ void vss_step_c(const KernelParams& p, const TaskDesc& tk, int q, int e, const C<T>* PV,
+                                           C<T>* QA, C<T>* QB, int plane0, int tid) {
+  using G = VGeo<T, N, W>;
   using CT = C<T>;
-  constexpr int N2 = G::N2, N3 = G::N3, CL = G::CL, GP = G::GP, NT = G::THREADS;
-  constexpr int PITCH = G::PITCH;
+  constexpr int h = G::h, N2 = G::N2, QS = G::QROW, HP = h + 1;
+  const int c0 = p.ent_m[2 * (tk.ent_off + e)], c1 = p.ent_m[2 * (tk.ent_off + e) + 1];
+  const bool self_sum = tk.i == tk.j && c1 >= 0;
+  const bool first = q == 0 && e == 0;
+  const int own = G::PLANES * HP;
+  const int all = own + (plane0 <= h && h < plane0 + G::PLANES ? h - 1 : 0);
+  for (int u = tid; u < all; u += G::THREADS) {
+    const int r = u < own ? plane0 + u / HP : h, kz = u < own ? u % HP : HP + u - own;
+    const int at = u < own ? r * HP + kz : N * HP + u - own;
+    const int rm = r == 0 ? 0 : N - r, km = kz == 0 ? 0 : N - kz;
+    const bool inner = kz < h && r != h;
+    const CT* const pv = PV + r * N + kz;
+    const CT* const pm = PV + rm * N + km;
+    CT v[N];
+    CT av = mk<T>(0, 0), am = mk<T>(0, 0);
+    if (inner) {
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        const CT a = ld2<T>(pv + n * N2), m = ld2<T>(pm + n * N2);
+        const T s = (n & 1) ? T(-1) : T(1);
+        av = mk<T>(fma_(s, a.x, av.x), fma_(s, a.y, av.y));
+        am = mk<T>(fma_(s, m.x, am.x), fma_(s, m.y, am.y));
+        v[n] = mk<T>(T(0.5) * (a.x + m.x), T(0.5) * (a.y - m.y));
+      }
+    } else {
+#pragma unroll
+      for (int n = 0; n < N; ++n) v[n] = ld2<T>(pv + n * N2);
+    }
+    line_fft<T, N, -1>(v);
+    for (int o = 0; o < 2; ++o) {
+      const int pair = o == 0 ? tk.out0 : tk.out1;
+      if (pair < 0) break;
+      // the slot of the output's direction, conjugated where it holds the antipode's weight; a halved
+      // self pair takes F(sigma) + F(-sigma) (FP32 tables hold the sum)
+      const int code = o == 0 ? c0 : c1;
+      const CT* const F = static_cast<const CT*>(p.Fv) + ((size_t(pair) * p.n_rho + q) * p.n_fslot + (code >> 1)) * G::N3;
+      auto weight = [&](int n, int row, int col) {
+        const CT f = __ldg(F + n * N2 + row * N + col);
+        if (sizeof(T) == 8 && self_sum) return mk<T>(f.x + f.x, T(0));
+        return mk<T>(f.x, (code & 1) ? -f.y : f.y);
+      };
+      CT* const acc = (o == 0 ? QA : QB) + at;
+#pragma unroll
+      for (int n = 0; n < N; ++n) {
+        CT val = cmul<T>(v[n], weight(n, r, kz));
+        if (n == h && inner) {
+          const CT x = cmul<T>(weight(h, r, kz), av), z = cmul<T>(weight(h, rm, km), am);
+          val = mk<T>(T(0.5) * (x.x + z.x), T(0.5) * (x.y - z.y));
+        }
+        if (!first) val = add<T>(val, ld2<T>(acc + n * QS));
+        st2<T>(acc + n * QS, val);
+      }
+    }
+  }
+}
+
+template <typename T, int N, int W>
+__global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) collision_kernel(const KernelParams p) {
+  using G = VGeo<T, N, W>;
+  using CT = C<T>;
+  constexpr int h = G::h, N2 = G::N2, HN2 = G::HN2, CL = G::CL, GP = G::GP, NT = G::THREADS, PITCH = G::PITCH;
+  constexpr int PB = G::PB;
+  constexpr size_t N3 = G::N3, HN3 = G::HN3;
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x;
   const int grp = tid / N;  // plane group
-  const int t = tid % N;    // line within the plane group
-  CT* tb = reinterpret_cast<CT*>(smem_raw) + size_t(grp) * G::NBUF * N * PITCH;
-  CT* ab = tb + N * PITCH;
-  CT* pb = ab + N * PITCH;  // used only when !PREG
-  CT* const tbB = pb;       // used only when YSH: transpose buffer of role 1
-  // phase block of the current (task, rho): [entry][role][axis][N], when staged in smem
-  CT* const phs = reinterpret_cast<CT*>(smem_raw) + size_t(GP) * G::NBUF * N * PITCH;
-  // phase block in shared memory: 1 = all axes, 2 = the z phases only (YSH shapes, where the
-  // x and y phases are read once per group or per unshared entry)
+  const int t = tid % N;    // line within the group: column (role, c) in y passes, row in z passes
+  const int role = t / h, c = t % h;
+  unsigned char* const gsm = smem_raw + size_t(grp) * G::GROUP_BYTES;
+  CT* const tb = reinterpret_cast<CT*>(gsm);  // padded plane; the pad column of rows 0, 1 carries a corner value
+  CT* const uyb = tb + N * PITCH;             // the entry's row of the k_y face
+  T* const pb = reinterpret_cast<T*>(uyb + N);
+  CT* const phs = reinterpret_cast<CT*>(smem_raw + G::SMEM);  // phase block of the current (task, rho)
   const bool ph_smem = p.phase_smem != 0;
-  const bool ph_zonly = G::YSH && p.phase_smem == 2;
 
-  const int rank = CL == 1 ? 0 : int(cluster_rank());
-  const int cid = blockIdx.x / CL;
-  CT* scr = reinterpret_cast<CT*>(p.scratch) + size_t(cid) * G::SLOT * N3;
-  CT* const FI = scr;
-  CT* const FJ = scr + N3;
-  CT* const HA0 = scr + 2 * N3;               // shifted volumes of role 0: HA0 + b N^3
-  CT* const HB0 = scr + (2 + G::NBV) * N3;    // and of role 1
-  CT* const PV = scr + (2 + 2 * G::NBV) * N3;
-  CT* const PV1 = PV + N3;
-  CT* const QA = PV + 2 * N3;
-  CT* const QB = PV + 3 * N3;
-  const bool vss = p.vss != 0;
-  const int plane0 = rank * G::PLANES;
-  const int pencil0 = rank * G::PENCILS;
-  const T inv_n3 = T(1) / T(N3);
-
-  // Work items (node, task) are taken from a counter: thread 0 of the rank-0 CTA takes the
-  // next item and the cluster reads it from that CTA's shared memory after a cluster barrier,
-  // so clusters that start late (other kernels holding SMs) find no work left instead of
-  // owning a share of it.  The value for the next item is taken after the first barrier of
-  // the current one, when every CTA has read the current value.
-  __shared__ int s_next_item;
-  const int n_items = p.batch * p.n_tasks;
-
-  // Staged plane pass: one mbarrier per plane buffer of each group (tb = buffer 0, ab =
-  // buffer 1), armed by the group's first thread for one bulk copy of N^2 complex values.
-  // Every thread of the group keeps the same bookkeeping: fill_par bit b is the parity of
-  // buffer b's next completion, fill_out bit b a copy in flight.  A wait gives up after about
-  // a second: the status word beside the work counter records it, and the group stops issuing
-  // and waiting (its results are then invalid, which the status reports).
-  __shared__ __align__(8) uint64_t s_fill[2 * GP];
-  unsigned fill_par = 0, fill_out = 0;
-  bool stalled = false;
-  if constexpr (G::STAGE) {
-    if (tid == 0) {
-      for (int b = 0; b < 2 * GP; ++b) tc::mbar_init(&s_fill[b], 1);
-      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-  }
-  // start a bulk copy of the plane at src into buffer bi (called by every thread of the group
-  // after the buffer's last readers have passed a group barrier behind a proxy fence)
-  auto fill = [&](int bi, const CT* src) {
-    if (stalled) return;
-    if (t == 0) {
-      uint64_t* bar = &s_fill[2 * grp + bi];
-      tc::mbar_expect_tx(bar, unsigned(N2 * sizeof(CT)));
-      tc::bulk_g2s(bi ? ab : tb, src, unsigned(N2 * sizeof(CT)), bar);
-    }
-    fill_out |= 1u << bi;
-  };
-  auto wait_fill = [&](int bi) {
-    if (stalled) return;
-    if (tc::mbar_wait_bounded(&s_fill[2 * grp + bi], (fill_par >> bi) & 1u, 2000000000LL)) {
-      fill_par ^= 1u << bi;
-      fill_out &= ~(1u << bi);
-    } else {
-      stalled = true;
-      atomicOr(p.work_counter + 1, 2u);
-    }
-  };
-
-  // TMEM accumulators: warp 0 allocates the CTA's columns; thread t of warp w reaches lane
-  // 32 (w % 4) + t
+  // TMEM: warp 0 allocates the CTA's columns; warp w reaches lanes 32 (w % 4) .. + 31
   __shared__ uint32_t s_tmem;
-  uint32_t tm_row = 0;
-  if constexpr (G::TM) {
+  uint32_t tm_raw = 0, tm_p = 0;
+  if constexpr (G::TM_ALLOC > 0) {
     if (tid < 32) {
       tc::tmem_alloc(&s_tmem, G::TM_ALLOC);
       tc::tmem_relinquish();
@@ -318,498 +394,527 @@ __global__ void __launch_bounds__(Geo<T, N>::THREADS, Geo<T, N>::MINB) collision
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    tm_row = s_tmem + (uint32_t(32 * ((tid / 32) & 3)) << 16);
+    tm_raw = s_tmem + (uint32_t(32 * ((tid / 32) & 3)) << 16) + uint32_t((tid / 128) * G::TM_SET);
+    tm_p = tm_raw + (G::TMR ? 2 * N : 0);
   }
 
+  const int rank = CL == 1 ? 0 : int(cluster_rank());
+  const int cid = blockIdx.x / CL;
+  CT* const scr = reinterpret_cast<CT*>(p.scratch) + size_t(cid) * p.slot;
+  CT* const FS = scr;               // f_hat [k_x][k_y][species 0 | 1][c]
+  CT* const H0 = FS + N3;           // x-passed half spectra [x][k_y][role][c], NBH buffers
+  CT* const HZ = H0 + G::NBH * N3;  // the same for the group with sigma_x = 0, kept for all radial nodes
+  CT* const PV = HZ + N3;       // product spectrum [x][row][c] (N form)
+  CT* const QA = PV + G::PVN;          // gain accumulators [k_x][row][c] (N form)
+  CT* const QB = QA + G::QN;
+  T* const PS = reinterpret_cast<T*>(QB + HN3);  // parked P [x][z][y]
+  CT* const FC = scr + G::SLOT;     // faces per entry: X [z][y], Y [x][z], line [y]; values (role 0, role 1)
+  const int plane0 = rank * G::PLANES;
+  const T inv_n3 = T(1) / T(N3);
+
+  // Work items (task, node, chunk of radial nodes) come from a counter: thread 0 of the rank-0 CTA
+  // takes the next item after the first barrier of the current one, when every CTA has read the
+  // current value.  Tasks are in order of falling cost, so the last items are the short ones.
+  __shared__ int s_next_item;
+  __shared__ int s_last;
+  const int n_items = p.batch * p.n_tasks * p.chunks;
   if (rank == 0 && tid == 0) s_next_item = int(atomicAdd(p.work_counter, 1u));
   cluster_sync<CL>();
   for (int item = CL == 1 ? s_next_item : ld_rank0(&s_next_item); item < n_items;
        item = CL == 1 ? s_next_item : ld_rank0(&s_next_item)) {
-    const int b = item / p.n_tasks;
-    const int task = item % p.n_tasks;
+    const int chunk = item % p.chunks;
+    const int whole = item / p.chunks;
+    const int b = whole % p.batch;
+    const int task = whole / p.batch;
+    const bool split = p.chunks > 1;
+    const int q0 = chunk * p.n_rho / p.chunks, q1 = (chunk + 1) * p.n_rho / p.chunks;
+    CT* const PT = static_cast<CT*>(p.parts) + size_t(whole) * p.n_rho * HN3;  // P_hat of every radial node
     const TaskDesc tk = p.tasks[task];
     const T* fb = reinterpret_cast<const T*>(p.f) + size_t(b) * p.s * N3;
-    const int nspec = tk.j == tk.i ? 1 : 2;
+    const bool self = tk.i == tk.j;
 
-    // ---- step 0: Fourier coefficients f_hat = N^-3 FFT(f) of species i (and j) ----------
+    // ---- step 0: f_hat = N^-3 DFT(f) of species i (and j), half spectra in C form -----------
     for (int xl = grp; xl < G::PLANES; xl += GP) {
       const int x = plane0 + xl;
-      for (int sp = 0; sp < nspec; ++sp) {
-        const T* src = fb + size_t(sp == 0 ? tk.i : tk.j) * N3 + size_t(x) * N2;
+      for (int sp = 0; sp < (self ? 1 : 2); ++sp) {
+        const T* src = fb + size_t(sp == 0 ? tk.i : tk.j) * N3 + size_t(x) * N2 + t * N;
+        T y[N];
+        CT z[h];
+#pragma unroll
+        for (int n = 0; n < N; ++n) y[n] = __ldg(src + n);
+        r2c_line<T, N>(y, z);
+#pragma unroll
+        for (int k = 0; k < h; ++k) tb[t * PITCH + sp * h + k] = z[k];
+      }
+      group_sync<N, GP>();
+      if (!self || role == 0) {
         CT v[N];
 #pragma unroll
-        for (int c = 0; c < N; ++c) v[c] = mk<T>(__ldg(src + t * N + c), T(0));
-        plane_pass2<T, N, GP, -1, false>(v, tb, t, nullptr);
-        CT* dst = (sp == 0 ? FI : FJ) + size_t(x) * N2;
+        for (int r = 0; r < N; ++r) v[r] = tb[r * PITCH + t];
+        line_fft<T, N, -1>(v);
 #pragma unroll
-        for (int r = 0; r < N; ++r) st2<T>(dst + r * N + t, v[r]);
+        for (int r = 0; r < N; ++r) st2<T>(FS + size_t(x) * N2 + r * N + t, v[r]);
+        // without a shift along x the x passes there and back cancel
+        if (tk.any_zero) {
+#pragma unroll
+          for (int r = 0; r < N; ++r) st2<T>(HZ + size_t(x) * N2 + r * N + t, scale<T>(v[r], T(1) / T(N2)));
+        }
       }
+      group_sync<N, GP>();
     }
     cluster_sync<CL>();
     if (rank == 0 && tid == 0) s_next_item = int(atomicAdd(p.work_counter, 1u));
-    for (int u = tid; u < nspec * G::PENCILS; u += NT) {
-      const int sp = u / G::PENCILS;
-      const int pp = pencil0 + u % G::PENCILS;
-      CT* vol = sp == 0 ? FI : FJ;
-      CT v[N];
-#pragma unroll
-      for (int n = 0; n < N; ++n) v[n] = ld2<T>(vol + n * N2 + pp);
-      fft_line<T, N, -1>(v);
-#pragma unroll
-      for (int n = 0; n < N; ++n) st2<T>(vol + n * N2 + pp, scale<T>(v[n], inv_n3));
-    }
-    cluster_sync<CL>();
-    const CT* FJs = nspec == 2 ? FJ : FI;
-
-    // ---- gain: radial nodes, sigma_x groups, entries ----------------------------------------
-    // Phase k runs step A of group k (into buffer k&1) and step B of group k-1 (from buffer
-    // (k-1)&1); one cluster barrier per phase, n_grp + 1 phases per radial node.  With VSS
-    // every group is one entry whose product is transformed forward on its own: step B of
-    // entry k-1 writes P volume (k-1)&1 and step C of entry k-2 weights P volume (k-2)&1 by
-    // F(k, rho, sigma) in the same phase (n_grp + 2 phases).
-    for (int q = 0; q < p.n_rho; ++q) {
-      const CT* const phq = phase_ptr<T, N>(p, task, q, 0, 0, 0);
-      if (ph_zonly) {
-        for (int u = tid; u < tk.n_ent * 2 * N; u += NT) phs[u] = __ldg(phq + ((u / N) * 3 + 2) * N + u % N);
-        __syncthreads();
-      } else if (ph_smem) {
-        for (int u = tid; u < tk.n_ent * 6 * N; u += NT) phs[u] = __ldg(phq + u);
-        __syncthreads();
-      }
-      const CT* const phb = ph_smem && !ph_zonly ? phs : phq;  // x and y phases
-      const int n_phase = tk.n_grp + (vss ? 2 : 1);
-      // Split cluster barrier (VHS, CL > 1): the CTA arrives once its step A of the phase is
-      // written and waits at the end of the phase, so its step B covers the other CTAs' lag.
-      // Pair k is written in phase k and read in phase k + 1, so with three buffers the pair
-      // written in phase k + 1 is one that no CTA reads after arriving in phase k.  The VSS
-      // pipeline's step B writes P volumes other CTAs read in the next phase: one full barrier.
-      const bool split = G::NBV == 3 && !vss;
-      const int nbv = split ? 3 : 2;
-      for (int k = 0; k < n_phase; ++k) {
-        if constexpr (G::STAGE) {
-          // step B of this phase starts on planes written before the last cluster barrier:
-          // copy the first entry's two planes now, so that they land during step A
-          if (k > 0 && k <= tk.n_grp) {
-            fence_proxy_async_global();
-            tc::fence_async_smem();
-            group_sync<N, GP>();
-            const size_t x0 = size_t(plane0 + grp) * N2;
-            fill(0, HA0 + size_t((k - 1) % nbv) * N3 + x0);
-            fill(1, HB0 + size_t((k - 1) % nbv) * N3 + x0);
-          }
-        }
-        if (k < tk.n_grp) {
-          const GroupDesc gd = p.groups[tk.grp_off + k];
-          CT* const dA = HA0 + size_t(k % nbv) * N3;
-          CT* const dB = HB0 + size_t(k % nbv) * N3;
-          // step A: x-pencils with the group's shared x phase.  The CTA's pencils of f_hat_i
-          // and f_hat_j are N rows of PENCILS contiguous elements each; prefetch them first.
-          if constexpr (G::PF) {
-            for (int u = tid; u < 2 * N; u += NT)
-              prefetch_l2((u < N ? FI : FJs) + size_t(u % N) * N2 + pencil0, G::PENCILS * sizeof(CT));
-          }
-          for (int u = tid; u < 2 * G::PENCILS; u += NT) {
-            const int role = u / G::PENCILS;
-            const int pp = pencil0 + u % G::PENCILS;
-            const CT* src = role == 0 ? FI : FJs;
-            const CT* ph = phb + ((gd.first * 2 + role) * 3 + 0) * N;
-            CT v[N];
-#pragma unroll
-            for (int n = 0; n < N; ++n) v[n] = ld2<T>(src + n * N2 + pp);
-            mul_phases<T, N>(v, ph);
-            fft_line<T, N, +1>(v);
-            CT* dst = role == 0 ? dA : dB;
-#pragma unroll
-            for (int n = 0; n < N; ++n) st2<T>(dst + n * N2 + pp, v[n]);
-          }
-          // the next phase reads these planes with bulk copies
-          if constexpr (G::STAGE) fence_proxy_async_global();
-        }
-        if constexpr (CL > 1) {
-          if (split && k < tk.n_grp) cluster_arrive();
-        }
-        if (G::STAGE && k > 0 && k <= tk.n_grp) {
-          const int gi = k - 1;
-          const GroupDesc gd = p.groups[tk.grp_off + gi];
-          const CT* const sA = HA0 + size_t(gi % nbv) * N3;
-          const CT* const sB = HB0 + size_t(gi % nbv) * N3;
-          const bool last = vss || gi == tk.n_grp - 1;
-          const bool fresh = vss || gi == 0;
-          CT* const PVw = (vss && (gi & 1)) ? PV1 : PV;
-          const int e_end = gd.first + gd.count;
-          // staged step B.  Role 0 of an entry reads buffer `cur` and leaves a_e in it; role 1
-          // reads the other buffer.  After role 1's transpose its buffer takes the next
-          // entry's role-0 plane; after the product, `cur` takes the next entry's role-1 plane.
-          // Every entry of the group reads the same two planes (the x pass is shared).
-          int cur = 0;
-          for (int xl = grp; xl < G::PLANES; xl += GP) {
-            const int x = plane0 + xl;
-            CT P[N];
-#pragma unroll
-            for (int c = 0; c < N; ++c) P[c] = fresh ? mk<T>(0, 0) : ld2<T>(PV + x * N2 + c * N + t);
-            for (int e = gd.first; e < e_end; ++e) {
-              const T w = T(p.ent_w[tk.ent_off + e]);
-              CT v[N];
-#pragma unroll 1
-              for (int role = 0; role < 2; ++role) {
-                const int bi = role == 0 ? cur : 1 - cur;
-                CT* const B = bi ? ab : tb;
-                const CT* phy = phb + ((e * 2 + role) * 3 + 1) * N;
-                const CT* phz = phb + ((e * 2 + role) * 3 + 2) * N;
-                wait_fill(bi);
-                // column t of the plane as copied (unpadded rows), with the y phase
-#pragma unroll
-                for (int r = 0; r < N; ++r) v[r] = B[r * N + t];
-                mul_phases<T, N>(v, phy);
-                group_sync<N, GP>();  // every column read: the buffer is re-laid out in place
-#pragma unroll 1
-                for (int pass = 0; pass < 2; ++pass) {
-                  if (pass == 1) {
-#pragma unroll
-                    for (int r = 0; r < N; ++r) B[r * PITCH + t] = v[r];
-                    group_sync<N, GP>();
-#pragma unroll
-                    for (int c = 0; c < N; ++c) v[c] = B[t * PITCH + c];
-                    mul_phases<T, N>(v, phz);
-                    if (role == 1) {
-                      // the buffer is free: the next entry's role-0 plane
-                      const CT* nxt = e + 1 < e_end ? sA + size_t(x) * N2
-                                    : xl + GP < G::PLANES ? sA + size_t(x + GP) * N2 : nullptr;
-                      tc::fence_async_smem();
-                      group_sync<N, GP>();
-                      if (nxt != nullptr) fill(bi, nxt);
-                    }
-                  }
-                  fft_line<T, N, +1>(v);
-                }
-                if (role == 0) {
-#pragma unroll
-                  for (int c = 0; c < N; ++c) B[t * PITCH + c] = v[c];
-                }
-              }
-              const CT* A0 = cur ? ab : tb;
-#pragma unroll
-              for (int c = 0; c < N; ++c) {
-                const CT ab_ = cmul<T>(A0[t * PITCH + c], v[c]);
-                P[c] = mk<T>(P[c].x + w * ab_.x, P[c].y + w * ab_.y);
-              }
-              if (e + 1 < e_end) {
-                tc::fence_async_smem();
-                group_sync<N, GP>();
-                fill(cur, sB + size_t(x) * N2);
-              }
-              cur = 1 - cur;
-            }
-            // the last entry's role-0 buffer (1 - cur) is free once every row has been read
-            CT* const Pb = cur ? tb : ab;
-            if (last) {
-              plane_pass2<T, N, GP, -1, false>(P, Pb, t, nullptr);
-#pragma unroll
-              for (int r = 0; r < N; ++r) st2<T>(PVw + x * N2 + r * N + t, P[r]);
-            } else {
-#pragma unroll
-              for (int c = 0; c < N; ++c) st2<T>(PV + x * N2 + c * N + t, P[c]);
-            }
-            if (xl + GP < G::PLANES) {
-              tc::fence_async_smem();
-              group_sync<N, GP>();
-              fill(1 - cur, sB + size_t(x + GP) * N2);
-            }
-          }
-        } else if (k > 0 && k <= tk.n_grp) {
-          const int gi = k - 1;
-          const GroupDesc gd = p.groups[tk.grp_off + gi];
-          const CT* const sA = HA0 + size_t(gi % nbv) * N3;
-          const CT* const sB = HB0 + size_t(gi % nbv) * N3;
-          // step B: (y, z) planes
-          const bool last = vss || gi == tk.n_grp - 1;
-          const bool fresh = vss || gi == 0;
-          CT* const PVw = (vss && (gi & 1)) ? PV1 : PV;
-          // each plane is prefetched one (plane, entry, role) read ahead of its use
-          constexpr bool PF = G::PF;
-          if (PF && t == 0) prefetch_l2(sA + size_t(plane0 + grp) * N2, N2 * sizeof(CT));
-          for (int xl = grp; xl < G::PLANES; xl += GP) {
-            const int x = plane0 + xl;
-            // TMEM columns of this plane's P and of a_e (TMEM accumulators)
-            const uint32_t tp = tm_row + uint32_t(((xl - grp) / GP) * 2 * N);
-            const uint32_t ta = tm_row + uint32_t(G::PPG * 2 * N);
-            CT P[G::PREG && !G::TM ? N : 1];
-            if constexpr (G::TM) {
-              // P stays in TMEM from the first group of the radial node to the last
-            } else if constexpr (G::PREG) {
-#pragma unroll
-              for (int c = 0; c < N; ++c) P[c] = fresh ? mk<T>(0, 0) : ld2<T>(PV + x * N2 + c * N + t);
-            } else {
-#pragma unroll
-              for (int c = 0; c < N; ++c) pb[t * PITCH + c] = fresh ? mk<T>(0, 0) : ld2<T>(PV + x * N2 + c * N + t);
-            }
-            for (int e = gd.first; e < gd.first + gd.count; ++e) {
-              const T w = T(p.ent_w[tk.ent_off + e]);
-              // with YSH, an entry whose sigma_y equals the previous entry's in the group reads
-              // the y pass of both volumes back from the role's transpose buffer
-              const bool reuse = G::YSH && e > gd.first && p.ent_ysh[tk.ent_off + e] != 0;
-              CT v[N];
-              for (int role = 0; role < 2; ++role) {
-                const CT* vol = (role == 0 ? sA : sB) + size_t(x) * N2;
-                const CT* phy = phb + ((e * 2 + role) * 3 + 1) * N;
-                const CT* phz = ph_zonly ? phs + (e * 2 + role) * N : phb + ((e * 2 + role) * 3 + 2) * N;
-                if (PF && t == 0 && !reuse) {
-                  // next plane read: the other role, the next entry that does not reuse, or
-                  // the group's next plane
-                  const CT* nxt = nullptr;
-                  if (role == 0) {
-                    nxt = sB + size_t(x) * N2;
-                  } else {
-                    int en = e + 1;
-                    if constexpr (G::YSH) {
-                      while (en < gd.first + gd.count && p.ent_ysh[tk.ent_off + en] != 0) ++en;
-                    }
-                    if (en < gd.first + gd.count) nxt = sA + size_t(x) * N2;
-                    else if (xl + GP < G::PLANES) nxt = sA + size_t(x + GP) * N2;
-                  }
-                  if (nxt != nullptr) prefetch_l2(nxt, N2 * sizeof(CT));
-                }
-                if constexpr (G::YSH) {
-                  CT* const yb = role == 0 ? tb : tbB;
-                  constexpr int P_ = PITCH;
-                  if (!reuse) {
-#pragma unroll
-                    for (int r = 0; r < N; ++r) v[r] = ld2<T>(vol + r * N + t);
-                    mul_phases<T, N>(v, phy);
-                  }
-                  // pass 0: y transform of the column (skipped on reuse); pass 1: z transform
-                  // of row t read back from the role's buffer, with the entry's z phase
-#pragma unroll 1
-                  for (int pass = reuse ? 1 : 0; pass < 2; ++pass) {
-                    if (pass == 1) {
-                      if (!reuse) {
-                        group_sync<N, GP>();  // the previous rows of yb have been read
-#pragma unroll
-                        for (int r = 0; r < N; ++r) yb[r * P_ + t] = v[r];
-                        group_sync<N, GP>();
-                      }
-#pragma unroll
-                      for (int c = 0; c < N; ++c) v[c] = yb[t * P_ + c];
-                      mul_phases<T, N>(v, phz);
-                    }
-                    fft_line<T, N, +1>(v);
-                  }
-                } else {
-#pragma unroll
-                  for (int r = 0; r < N; ++r) v[r] = ld2<T>(vol + r * N + t);
-                  mul_phases<T, N>(v, phy);
-                  plane_pass2<T, N, GP, +1, true>(v, tb, t, phz);
-                }
-                if (role == 0) {
-                  if constexpr (G::TM) {
-                    __syncwarp();
-                    tm_store_line<N>(ta, v);
-                  } else {
-#pragma unroll
-                    for (int c = 0; c < N; ++c) ab[t * PITCH + c] = v[c];
-                  }
-                }
-              }
-              if constexpr (G::TM) {
-                // P += w a_e b_e in chunks of 8 values (the first entry of the radial node's first
-                // group writes P)
-                const bool p_first = fresh && e == gd.first;
-                __syncwarp();
-                tc::tmem_wait_st();
-#pragma unroll
-                for (int ch = 0; ch < N / 8; ++ch) {
-                  float a16[16], p16[16];
-                  tm_ld16w(ta + uint32_t(16 * ch), a16);
-                  if (!p_first) tm_ld16w(tp + uint32_t(16 * ch), p16);
-#pragma unroll
-                  for (int j = 0; j < 8; ++j) {
-                    const CT ab_ = cmul<T>(mk<T>(a16[2 * j], a16[2 * j + 1]), v[8 * ch + j]);
-                    // one rounding per update, as P + w ab in registers (P = 0 at the start)
-                    p16[2 * j] = fmaf(w, ab_.x, p_first ? 0.f : p16[2 * j]);
-                    p16[2 * j + 1] = fmaf(w, ab_.y, p_first ? 0.f : p16[2 * j + 1]);
-                  }
-                  tc::tmem_st16(tp + uint32_t(16 * ch), p16);
-                }
-              } else if constexpr (G::PREG) {
-#pragma unroll
-                for (int c = 0; c < N; ++c) {
-                  const CT a = ab[t * PITCH + c];
-                  const CT ab_ = cmul<T>(a, v[c]);
-                  P[c] = mk<T>(P[c].x + w * ab_.x, P[c].y + w * ab_.y);
-                }
-              } else {
-#pragma unroll
-                for (int c = 0; c < N; ++c) {
-                  const CT a = ab[t * PITCH + c];
-                  const CT ab_ = cmul<T>(a, v[c]);
-                  const CT o = pb[t * PITCH + c];
-                  pb[t * PITCH + c] = mk<T>(o.x + w * ab_.x, o.y + w * ab_.y);
-                }
-              }
-            }
-            if (last) {
-              CT v[N];
-              if constexpr (G::TM) {
-                __syncwarp();
-                tc::tmem_wait_st();
-                tm_load_line<N>(tp, v);
-              } else {
-#pragma unroll
-                for (int c = 0; c < N; ++c) {
-                  if constexpr (G::PREG) v[c] = P[c]; else v[c] = pb[t * PITCH + c];
-                }
-              }
-              plane_pass2<T, N, GP, -1, false>(v, tb, t, nullptr);
-#pragma unroll
-              for (int r = 0; r < N; ++r) st2<T>(PVw + x * N2 + r * N + t, v[r]);
-            } else if constexpr (!G::TM) {
-#pragma unroll
-              for (int c = 0; c < N; ++c) {
-                CT val;
-                if constexpr (G::PREG) val = P[c]; else val = pb[t * PITCH + c];
-                st2<T>(PV + x * N2 + c * N + t, val);
-              }
-            }
-          }
-        }
-        if (vss && k >= 2) {
-          // step C (VSS) of entry k-2: forward x transform, Q_hat^+ += F(k, rho, sigma) P_hat;
-          // for a halved self pair F(sigma) + F(-sigma), for the reused (j,i) pair F^(ji)(-sigma)
-          const int e = k - 2;
-          const CT* const PVr = (e & 1) ? PV1 : PV;
-          const int c0 = p.ent_m[2 * (tk.ent_off + e)], c1 = p.ent_m[2 * (tk.ent_off + e) + 1];
-          const bool self_sum = tk.i == tk.j && c1 >= 0;
-          const bool first = q == 0 && e == 0;
-          for (int u = tid; u < G::PENCILS; u += NT) {
-            const int pp = pencil0 + u;
-            CT v[N];
-#pragma unroll
-            for (int n = 0; n < N; ++n) v[n] = ld2<T>(PVr + n * N2 + pp);
-            fft_line<T, N, -1>(v);
-            for (int o = 0; o < 2; ++o) {
-              const int pair = o == 0 ? tk.out0 : tk.out1;
-              if (pair < 0) break;
-              // slot code of this output's direction: 2 slot + 1 when the slot holds the
-              // antipode's weight (read conjugated)
-              const int code = o == 0 ? c0 : c1;
-              const size_t fo = ((size_t(pair) * p.n_rho + q) * p.n_fslot + (code >> 1)) * N3;
-              const T sgn = (code & 1) ? T(-1) : T(1);
-              CT* acc = o == 0 ? QA : QB;
-              if constexpr (sizeof(T) == 4) {
-                // FP32 table; a self pair's slot already holds F(sigma) + F(-sigma)
-                const float2* F0 = static_cast<const float2*>(p.Fv) + fo;
-#pragma unroll
-                for (int n = 0; n < N; ++n) {
-                  const float2 fw = __ldg(F0 + n * N2 + pp);
-                  CT val = cmul<T>(v[n], mk<T>(fw.x, sgn * fw.y));
-                  if (!first) val = add<T>(val, ld2<T>(acc + n * N2 + pp));
-                  st2<T>(acc + n * N2 + pp, val);
-                }
-              } else {
-                const double2* F0 = static_cast<const double2*>(p.Fv) + fo;
-#pragma unroll
-                for (int n = 0; n < N; ++n) {
-                  double2 fw = __ldg(F0 + n * N2 + pp);
-                  // a halved self pair takes F(sigma) + F(-sigma) = F + conj F
-                  fw = self_sum ? make_double2(fw.x + fw.x, 0.0) : make_double2(fw.x, sgn * fw.y);
-                  CT val = cmul<T>(v[n], mk<T>(T(fw.x), T(fw.y)));
-                  if (!first) val = add<T>(val, ld2<T>(acc + n * N2 + pp));
-                  st2<T>(acc + n * N2 + pp, val);
-                }
-              }
-            }
-          }
-        }
-        if constexpr (CL > 1) {
-          if (split && k < tk.n_grp) cluster_wait(); else cluster_sync<CL>();
-        } else {
-          cluster_sync<CL>();
-        }
-      }
-      if (vss) continue;
-      // step C: forward transform of P along x, weight, accumulate
-      for (int u = tid; u < G::PENCILS; u += NT) {
-        const int pp = pencil0 + u;
+    if (!self || role == 0) {
+      for (int xl = grp; xl < G::PLANES; xl += GP) {
+        CT* const vol = FS + (plane0 + xl) * N + t;
         CT v[N];
 #pragma unroll
-        for (int n = 0; n < N; ++n) v[n] = ld2<T>(PV + n * N2 + pp);
-        fft_line<T, N, -1>(v);
+        for (int n = 0; n < N; ++n) v[n] = ld2<T>(vol + n * N2);
+        line_fft<T, N, -1>(v);
+#pragma unroll
+        for (int n = 0; n < N; ++n) st2<T>(vol + n * N2, scale<T>(v[n], inv_n3));
+      }
+    }
+    cluster_sync<CL>();
+    const CT* const Fr = FS + (self ? c : t);     // this thread's column of f_hat
+    const CT fe = ld2<T>(Fr + h * N2 + h * N);    // its value on the edge k_x = k_y = N/2
+
+    // ---- gain ---------------------------------------------------------------------------------
+    T P[G::PSM || G::VSS ? 1 : N];
+    for (int q = q0; q < q1; ++q) {
+      const CT* const phq = static_cast<const CT*>(p.phase) + (size_t(task) * p.n_rho + q) * p.max_ent * PB;
+      if (ph_smem) {
+        for (int u = tid; u < tk.n_ent * PB; u += NT) phs[u] = __ldg(phq + u);
+        __syncthreads();
+      }
+      const CT* const phb = ph_smem ? phs : phq;
+
+      // faces of the entries whose shift along the face's axis is not zero, spread over the
+      // cluster's CTAs first; code 2 e + kind.  kind 0: k_x = N/2 (y and z shifted), kind 1:
+      // k_y = N/2 (x and z shifted)
+      for (int f0 = 0; f0 < tk.n_face; f0 += CL * GP) {
+        // groups that share a barrier run the same number of rounds: one without a face of its own
+        // repeats the last and stores nothing
+        const int f = f0 + grp * CL + rank;
+        const bool live = f < tk.n_face;
+        if (N % 32 == 0 && !live) break;
+        const int code = p.faces[tk.face_off + (live ? f : tk.n_face - 1)];
+        const int e = code >> 1, kind = code & 1;
+        const CT* const pe = phb + e * PB;
+        CT* const fc = FC + size_t(e) * G::FACE;
+        {
+          const CT* const src = Fr + (kind == 0 ? h * N2 : h * N);
+          const int step = kind == 0 ? N : N2;
+          CT v[N];
+#pragma unroll
+          for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + r * step);
+          shift_line<T, N>(v, pe + (kind == 0 ? N : 0) + role);
+          line_fft<T, N, +1>(v);
+          group_sync<N, GP>();
+#pragma unroll
+          for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
+          group_sync<N, GP>();
+        }
+        const CT* const row = tb + t * PITCH;
+        const CT cta = pe[2 * N], ctb = pe[2 * N + h];
+        const CT a0 = row[0], b0 = row[h];
+        Rows<T, N> y;
+        rows_c2r<N>(row, pe + 2 * N, mk<T>(a0.x, pe[3 * N].x * b0.x), mk<T>(cta.x * a0.y, ctb.x * b0.y), y);
+        const CT sc = mk<T>(pe[kind == 0 ? 0 : N].y, pe[kind == 0 ? 1 : N + 1].y);
+        if (!live) {
+        } else if (kind == 0) {
+#pragma unroll
+          for (int z = 0; z < N; ++z) st2<T>(fc + z * N + t, mul_each(sc, y.at(z)));
+          st2<T>(fc + 2 * N2 + t, mk<T>(sc.x * a0.y, sc.y * b0.y));
+        } else {
+#pragma unroll
+          for (int z = 0; z < N; ++z) st2<T>(fc + N2 + t * N + z, mul_each(sc, y.at(z)));
+        }
+      }
+
+      for (int k = 0; k <= tk.n_grp + (G::VSS ? 1 : 0); ++k) {
+        // step A of group k: x pass of this thread's pencils with the group's x phases
+        if (k < tk.n_grp && !p.groups[tk.grp_off + k].zero) {
+          const GroupDesc gd = p.groups[tk.grp_off + k];
+          CT* const dst = H0 + size_t(k % G::NBH) * N3;
+          const CT* const phx = phb + gd.first * PB + role;
+          for (int xl = grp; xl < G::PLANES; xl += GP) {
+            const int r = plane0 + xl;
+            CT v[N];
+#pragma unroll
+            for (int n = 0; n < N; ++n) v[n] = ld2<T>(Fr + n * N2 + r * N);
+            shift_line<T, N>(v, phx);
+            line_fft<T, N, +1>(v);
+#pragma unroll
+            for (int n = 0; n < N; ++n) st2<T>(dst + n * N2 + r * N + t, v[n]);
+          }
+        }
+        // split barrier: step B of group k - 1 covers the other CTAs' lag in step A of group k
+        const bool halves = G::SPLIT && k > 0 && k < tk.n_grp;
+        if (halves) cluster_arrive();
+        // step B of group k - 1: this group's planes
+        if (k > 0 && k <= tk.n_grp) {
+          const GroupDesc gd = p.groups[tk.grp_off + k - 1];
+          const bool zero = gd.zero != 0;
+          const CT* const src = zero ? HZ : H0 + size_t((k - 1) % G::NBH) * N3;
+          const int col = zero && self ? c : t;  // (a self pair's roles share the unshifted columns)
+          const bool fresh = k == 1, last = k == tk.n_grp;
+          for (int xl = grp; xl < G::PLANES; xl += GP) {
+            const int x = plane0 + xl;
+            if constexpr (G::PF) {
+              if (t == 0 && xl + GP < G::PLANES) prefetch_l2(src + size_t(x + GP) * N2, N2 * sizeof(CT));
+            }
+            const T sgx = (x & 1) ? T(-1) : T(1), sgy = (t & 1) ? T(-1) : T(1);
+            if constexpr (G::VSS) {
+              // no sum over the entries
+            } else if constexpr (G::PSM) {
+              if (fresh || !G::KEEP) {
+#pragma unroll
+                for (int z = 0; z < N; ++z) pb[z * N + t] = fresh ? T(0) : __ldcg(PS + size_t(x) * N2 + z * N + t);
+              }
+            } else {
+              if (fresh) {
+#pragma unroll
+                for (int z = 0; z < N; ++z) P[z] = T(0);
+              } else if constexpr (G::TMP) {
+                __syncwarp();
+                tm_load<N>(tm_p + uint32_t((xl / GP) * N), reinterpret_cast<float*>(P));
+              } else if constexpr (!G::KEEP) {
+#pragma unroll
+                for (int z = 0; z < N; ++z) P[z] = __ldcg(PS + size_t(x) * N2 + z * N + t);
+              }
+            }
+            for (int e = gd.first; e < gd.first + gd.count; ++e) {
+              const CT* const pe = phb + e * PB;
+              const CT* const fc = FC + size_t(e) * G::FACE;
+              // a shift of zero along an axis has no face there
+              const T txa = pe[0].y, txb = pe[1].y, tya = pe[N].y, tyb = pe[N + 1].y;
+              const bool has_x = has_face<T>(pe), has_y = tya != T(0) || tyb != T(0);
+              const CT uy = has_y ? __ldca(fc + N2 + x * N + t) : mk<T>(0, 0);
+              const CT en = has_x ? __ldca(fc + 2 * N2 + t) : mk<T>(0, 0);
+              {
+                CT v[N];
+                if (!G::TMR || e == gd.first) {
+#pragma unroll
+                  for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + size_t(x) * N2 + r * N + col);
+                  if constexpr (G::TMR) {
+                    if (gd.count > 1) {
+                      __syncwarp();
+                      tm_store<2 * N>(tm_raw, reinterpret_cast<const float*>(v));
+                    }
+                  }
+                } else if constexpr (G::TMR) {
+                  __syncwarp();
+                  tm_load<2 * N>(tm_raw, reinterpret_cast<float*>(v));
+                }
+                const T corner = v[h].y;  // of column 0: f on the edge k_y = k_z = N/2
+                shift_line<T, N>(v, pe + N + role);
+                const T w = sgx * (role == 0 ? txa * tya : txb * tyb);
+                v[h] = mk<T>(v[h].x - w * fe.x, v[h].y - w * fe.y);
+                line_fft<T, N, +1>(v);
+                group_sync<N, GP>();  // the previous entry's rows have been read
+#pragma unroll
+                for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
+                uyb[t] = uy;
+                if (c == 0) tb[role * PITCH + N] = mk<T>(corner, T(0));
+                group_sync<N, GP>();
+              }
+              const CT* const row = tb + t * PITCH;
+              const CT cta = pe[2 * N], ctb = pe[2 * N + h];
+              const CT a0 = row[0], b0 = row[h];
+              const CT m = mk<T>(cta.y * a0.y, ctb.y * b0.y);
+              Rows<T, N> y;
+              rows_c2r<N>(row, pe + 2 * N, mk<T>(a0.x, pe[3 * N].x * b0.x),
+                          mk<T>(cta.x * a0.y - cta.y * (sgx * en.x + sgy * tya * tb[N].x),
+                                ctb.x * b0.y - ctb.y * (sgx * en.y + sgy * tyb * tb[PITCH + N].x)),
+                          y);
+              if constexpr (G::VSS) {
+                // the product is complex; forward z and y transforms, all N columns
+                CT pr[N];
+#pragma unroll
+              for (int z = 0; z < N; z += 2) {
+                CT uz[2];
+                load_two(uyb + z, uz[0], uz[1]);
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                  // read by every plane of the CTA: through L1
+                  const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
+                  const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
+                  const CT re = y.at(z + d);
+                  pr[z + d] = mk<T>(fma_(-im.x, im.y, re.x * re.y), fma_(re.x, im.y, im.x * re.y));
+                }
+              }
+                line_fft<T, N, -1>(pr);
+                group_sync<N, GP>();
+#pragma unroll
+                for (int z = 0; z < N; ++z) tb[t * PITCH + z] = pr[z];
+                group_sync<N, GP>();
+#pragma unroll
+                for (int r = 0; r < N; ++r) pr[r] = tb[r * PITCH + t];
+                line_fft<T, N, -1>(pr);
+                CT* const dst = PV + size_t(2 * ((k - 1) & 1) + e - gd.first) * N3 + size_t(x) * N2 + t;
+#pragma unroll
+                for (int r = 0; r < N; ++r) st2<T>(dst + r * N, pr[r]);
+              } else {
+#pragma unroll
+              for (int z = 0; z < N; z += 2) {
+                CT uz[2];
+                load_two(uyb + z, uz[0], uz[1]);
+#pragma unroll
+                for (int d = 0; d < 2; ++d) {
+                  // read by every plane of the CTA: through L1
+                  const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
+                  const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
+                  const CT re = y.at(z + d);
+                  if constexpr (G::PSM) pb[(z + d) * N + t] = fma_(-im.x, im.y, fma_(re.x, re.y, pb[(z + d) * N + t]));
+                  else P[z + d] = fma_(-im.x, im.y, fma_(re.x, re.y, P[z + d]));
+                }
+              }
+              }
+            }
+            if constexpr (G::VSS) {
+              // done entry by entry
+            } else if (last) {
+              group_sync<N, GP>();
+              {
+                CT z[h];
+                T y[N];
+#pragma unroll
+                for (int n = 0; n < N; ++n) {
+                  if constexpr (G::PSM) y[n] = pb[n * N + t]; else y[n] = P[n];
+                }
+                r2c_line<T, N>(y, z);
+#pragma unroll
+                for (int kz = 0; kz < h; ++kz) tb[t * PITCH + kz] = z[kz];
+              }
+              group_sync<N, GP>();
+              if (role == 0) {
+                CT v[N];
+#pragma unroll
+                for (int r = 0; r < N; ++r) v[r] = tb[r * PITCH + t];
+                line_fft<T, N, -1>(v);
+                CT* const dst = PV + size_t(x) * HN2 + c;
+                if (c != 0) {
+#pragma unroll
+                  for (int r = 0; r < N; ++r) st2<T>(dst + r * h, v[r]);
+                } else {  // C form -> N form
+                  st2<T>(dst, mk<T>(v[0].x, v[h].x));
+                  st2<T>(dst + h * h, mk<T>(v[0].y, v[h].y));
+#pragma unroll
+                  for (int r = 1; r < h; ++r) {
+                    const CT m = conj_<T>(v[N - r]);
+                    const CT d = sub<T>(v[r], m);
+                    st2<T>(dst + r * h, scale<T>(add<T>(v[r], m), T(0.5)));
+                    st2<T>(dst + (h + r) * h, mk<T>(T(0.5) * d.y, T(-0.5) * d.x));
+                  }
+                }
+              }
+            } else if constexpr (G::TMP) {
+              __syncwarp();
+              tm_store<N>(tm_p + uint32_t((xl / GP) * N), reinterpret_cast<const float*>(P));
+            } else if constexpr (!G::KEEP) {
+#pragma unroll
+              for (int z = 0; z < N; ++z) {
+                T val;
+                if constexpr (G::PSM) val = pb[z * N + t]; else val = P[z];
+                __stcg(PS + size_t(x) * N2 + z * N + t, val);
+              }
+            }
+          }
+        }
+        if constexpr (G::VSS) {
+          if (k >= 2) {
+            const GroupDesc gd = p.groups[tk.grp_off + k - 2];
+            for (int j = 0; j < gd.count; ++j)
+              vss_step_c<T, N, W>(p, tk, q, gd.first + j, PV + size_t(2 * (k & 1) + j) * N3, QA, QB, plane0, tid);
+          }
+        }
+        if (halves) cluster_wait(); else cluster_sync<CL>();
+      }
+      if constexpr (G::VSS) continue;
+
+      // step C: x pass of the product spectrum, weights, accumulation
+      for (int u = tid; u < G::PLANES * h; u += NT) {
+        const int r = plane0 + u / h, cc = u % h;
+        const size_t pp = size_t(r) * h + cc;
+        CT v[N];
+#pragma unroll
+        for (int n = 0; n < N; ++n) v[n] = ld2<T>(PV + n * HN2 + pp);
+        line_fft<T, N, -1>(v);
+        // modes of the pencil (N form): column 0 holds k_z = 0 in rows 1..N/2-1 and k_z = N/2 above
+        // them; rows 0 and N/2 hold two real pencils, k_y = 0 and N/2, as one
+        const bool pair_row = cc == 0 && (r == 0 || r == h);
+        const int ky = cc == 0 && r >= h ? r - h : r;
+        const int kz = cc == 0 && r >= h ? h : cc;
+        if (split) {
+#pragma unroll
+          for (int n = 0; n < N; ++n) st2<T>(PT + q * HN3 + n * HN2 + pp, v[n]);
+          continue;
+        }
         for (int o = 0; o < 2; ++o) {
           const int pair = o == 0 ? tk.out0 : tk.out1;
           if (pair < 0) break;
-          // the table is in the plan's real type (FP32 plans: rounded once at plan creation)
-          const T* Fw = static_cast<const T*>(p.Fw) + (size_t(pair) * p.n_rho + q) * N3;
-          CT* acc = o == 0 ? QA : QB;
+          const T* const Fw = static_cast<const T*>(p.Fw) + (size_t(pair) * p.n_rho + q) * N3 + ky * N + kz;
+          CT* const acc = (o == 0 ? QA : QB) + pp;
+          if (!pair_row) {
 #pragma unroll
-          for (int n = 0; n < N; ++n) {
-            const T fw = __ldg(Fw + n * N2 + pp);
-            CT val = scale<T>(v[n], fw);
-            if (q > 0) val = add<T>(val, ld2<T>(acc + n * N2 + pp));
-            st2<T>(acc + n * N2 + pp, val);
+            for (int n = 0; n < N; ++n) {
+              const CT old = q > 0 ? ld2<T>(acc + n * HN2) : mk<T>(0, 0);
+              st2<T>(acc + n * HN2, add_gain<T>(old, __ldg(Fw + n * N2), v[n], q == 0));
+            }
+          } else {
+#pragma unroll
+            for (int n = 0; n < N; ++n) {
+              const CT old = q > 0 ? ld2<T>(acc + n * HN2) : mk<T>(0, 0);
+              st2<T>(acc + n * HN2, add_gain_pair<T>(old, __ldg(Fw + n * N2), __ldg(Fw + n * N2 + h * N), v[n],
+                                                     v[(N - n) % N], q == 0));
+            }
           }
+        }
+      }
+    }
+    if (split) {
+      // the cluster that stores the last of the item's products adds them up and finishes the item
+      __threadfence();
+      cluster_sync<CL>();
+      if (rank == 0 && tid == 0) {
+        unsigned* const done = p.work_counter + kDoneWord + whole;
+        s_last = atomicAdd(done, 1u) + 1 == unsigned(p.chunks) ? 1 : 0;
+        if (s_last) *done = 0;  // ready for the next launch
+        __threadfence();
+      }
+      cluster_sync<CL>();
+      if ((CL == 1 ? s_last : ld_rank0(&s_last)) == 0) {
+        cluster_sync<CL>();  // s_last has been read
+        continue;
+      }
+      __threadfence();
+      for (int u = tid; u < N * G::PLANES * h; u += NT) {  // element by element: every load independent
+        const int n = u / (G::PLANES * h), pp = plane0 * h + u % (G::PLANES * h);
+        const int r = pp / h, cc = pp % h;
+        const bool pair_row = cc == 0 && (r == 0 || r == h);
+        const int ky = cc == 0 && r >= h ? r - h : r;
+        const int kz = cc == 0 && r >= h ? h : cc;
+        const CT* const pv = PT + n * HN2 + pp;
+        const CT* const pm = PT + (n == 0 ? 0 : N - n) * HN2 + pp;
+        for (int o = 0; o < 2; ++o) {
+          const int pair = o == 0 ? tk.out0 : tk.out1;
+          if (pair < 0) break;
+          const T* const Fw = static_cast<const T*>(p.Fw) + size_t(pair) * p.n_rho * N3 + n * N2 + ky * N + kz;
+          CT acc = mk<T>(0, 0);
+          if (!pair_row) {
+#pragma unroll 8
+            for (int q = 0; q < p.n_rho; ++q) acc = add_gain<T>(acc, __ldg(Fw + q * N3), ld2<T>(pv + q * HN3), q == 0);
+          } else {
+            for (int q = 0; q < p.n_rho; ++q)
+              acc = add_gain_pair<T>(acc, __ldg(Fw + q * N3), __ldg(Fw + q * N3 + h * N), ld2<T>(pv + q * HN3),
+                                     ld2<T>(pm + q * HN3), q == 0);
+          }
+          st2<T>((o == 0 ? QA : QB) + n * HN2 + pp, acc);
         }
       }
     }
     __syncthreads();
 
-    // ---- finish: Q_ij = Re IFFT(Q_hat^+) - f_i Re IFFT(G^- f_hat_j) --------------------------
+    // ---- finish: Q_ij = IDFT(Q_hat) - f_i IDFT(G^- f_hat_j); role 0 the gain, role 1 the loss ----
     for (int o = 0; o < 2; ++o) {
       const int pair = o == 0 ? tk.out0 : tk.out1;
       if (pair < 0) break;
       const int io = o == 0 ? tk.i : tk.j;
       const int jo = o == 0 ? tk.j : tk.i;
-      const CT* acc = o == 0 ? QA : QB;
-      const CT* Fj = jo == tk.i ? FI : FJs;
-      const T* Gm = static_cast<const T*>(p.Gm) + size_t(pair) * N3;
-      for (int u = tid; u < G::PENCILS; u += NT) {
-        const int pp = pencil0 + u;
+      const CT* const acc = o == 0 ? QA : QB;
+      const CT* const Fj = FS + (jo == tk.i ? 0 : h);
+      const T* const Gm = static_cast<const T*>(p.Gm) + size_t(pair) * N3;
+      for (int xl = grp; xl < G::PLANES; xl += GP) {
+        const int r = plane0 + xl;
         CT v[N];
+        if (role == 0 && G::VSS) {  // the Hermitian part, in C form
+          constexpr int HP = h + 1;
+          auto at = [&](int n, int row, int kz) {
+            return ld2<T>(acc + n * G::QROW + (kz <= h ? row * HP + kz : N * HP + kz - HP));
+          };
+          auto herm = [](CT a, CT m) { return mk<T>(T(0.5) * (a.x + m.x), T(0.5) * (a.y - m.y)); };
+          const int rm = r == 0 ? 0 : N - r;
+          for (int n = 0; n < N; ++n) {
+            const int nm = n == 0 ? 0 : N - n;
+            CT a = at(n, r, c);
+            if (r == h) a = herm(a, at(nm, h, c == 0 ? 0 : N - c));
+            if (c == 0) {
+              const CT d = herm(at(n, r, h), at(nm, rm, h));
+              a = mk<T>(a.x - d.y, a.y + d.x);
+            }
+            st2<T>(H0 + n * N2 + r * N + t, a);
+          }
 #pragma unroll
-        for (int n = 0; n < N; ++n) v[n] = ld2<T>(acc + n * N2 + pp);
-        fft_line<T, N, +1>(v);
+          for (int n = 0; n < N; ++n) v[n] = ld2<T>(H0 + n * N2 + r * N + t);
+        } else if (role == 0) {
 #pragma unroll
-        for (int n = 0; n < N; ++n) st2<T>(HA0 + n * N2 + pp, v[n]);
+          for (int n = 0; n < N; ++n) v[n] = ld2<T>(acc + n * HN2 + r * h + c);
+        } else if (c != 0) {
 #pragma unroll
-        for (int n = 0; n < N; ++n) v[n] = scale<T>(ld2<T>(Fj + n * N2 + pp), __ldg(Gm + n * N2 + pp));
-        fft_line<T, N, +1>(v);
+          for (int n = 0; n < N; ++n) v[n] = scale<T>(ld2<T>(Fj + n * N2 + r * N + c), __ldg(Gm + n * N2 + r * N + c));
+        } else {  // C form: the two parts of column 0 have weights of their own
+          const int rm = r == 0 ? 0 : N - r;
 #pragma unroll
-        for (int n = 0; n < N; ++n) st2<T>(HB0 + n * N2 + pp, v[n]);
+          for (int n = 0; n < N; ++n) {
+            const T ga = __ldg(Gm + n * N2 + r * N), gh = __ldg(Gm + n * N2 + r * N + h);
+            const T gp = T(0.5) * (ga + gh), gm = T(0.5) * (ga - gh);
+            const CT a = ld2<T>(Fj + n * N2 + r * N), m = ld2<T>(Fj + ((N - n) % N) * N2 + rm * N);
+            v[n] = mk<T>(gp * a.x + gm * m.x, gp * a.y - gm * m.y);
+          }
+        }
+        line_fft<T, N, +1>(v);
+#pragma unroll
+        for (int n = 0; n < N; ++n) st2<T>(H0 + n * N2 + r * N + t, v[n]);
       }
       cluster_sync<CL>();
-      T* Qout = reinterpret_cast<T*>(p.Q) + ((size_t(b) * p.s + io) * p.s + jo) * N3;
-      const T* fi = fb + size_t(io) * N3;
+      T* const Qout = reinterpret_cast<T*>(p.Q) + ((size_t(b) * p.s + io) * p.s + jo) * N3;
+      const T* const fi = fb + size_t(io) * N3;
       for (int xl = grp; xl < G::PLANES; xl += GP) {
         const int x = plane0 + xl;
-        CT v[N];
-        T gain[N];
+        const CT* const src = H0 + size_t(x) * N2;
+        {
+          CT v[N];
+          if (t != 0 || G::VSS) {
 #pragma unroll
-        for (int r = 0; r < N; ++r) v[r] = ld2<T>(HA0 + x * N2 + r * N + t);
-        plane_pass2<T, N, GP, +1, true>(v, tb, t, nullptr);
+            for (int r = 0; r < N; ++r) v[r] = ld2<T>(src + r * N + t);
+          } else {  // N form -> C form
+            const CT a = ld2<T>(src), d = ld2<T>(src + h * N);
+            v[0] = mk<T>(a.x, d.x);
+            v[h] = mk<T>(a.y, d.y);
 #pragma unroll
-        for (int c = 0; c < N; ++c) gain[c] = v[c].x;
+            for (int r = 1; r < h; ++r) {
+              const CT al = ld2<T>(src + r * N), be = ld2<T>(src + (h + r) * N);
+              v[r] = mk<T>(al.x - be.y, al.y + be.x);
+              v[N - r] = mk<T>(al.x + be.y, be.x - al.y);
+            }
+          }
+          line_fft<T, N, +1>(v);
+          group_sync<N, GP>();
 #pragma unroll
-        for (int r = 0; r < N; ++r) v[r] = ld2<T>(HB0 + x * N2 + r * N + t);
-        plane_pass2<T, N, GP, +1, true>(v, tb, t, nullptr);
-        // row t of this plane; stage through shared memory for a coalesced store
-        T* rb = reinterpret_cast<T*>(tb);
+          for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
+          group_sync<N, GP>();
+        }
+        const CT g0 = tb[t * PITCH], l0 = tb[t * PITCH + h];
+        Rows<T, N> y;
+        rows_c2r<N>(tb + t * PITCH, static_cast<const CT*>(nullptr), mk<T>(g0.x, l0.x), mk<T>(g0.y, l0.y), y);
+        group_sync<N, GP>();
+        // stage the row through shared memory for a coalesced store
+        T* const rb = reinterpret_cast<T*>(tb);
 #pragma unroll
-        for (int c = 0; c < N; ++c) rb[t * PITCH + c] = gain[c] - __ldg(fi + x * N2 + t * N + c) * v[c].x;
+        for (int z = 0; z < N; ++z) {
+          const CT gl = y.at(z);
+          rb[t * PITCH + z] = gl.x - __ldg(fi + size_t(x) * N2 + t * N + z) * gl.y;
+        }
         group_sync<N, GP>();
 #pragma unroll
-        for (int r = 0; r < N; ++r) Qout[x * N2 + r * N + t] = rb[r * PITCH + t];
+        for (int r = 0; r < N; ++r) Qout[size_t(x) * N2 + r * N + t] = rb[r * PITCH + t];
         group_sync<N, GP>();
       }
       cluster_sync<CL>();
     }
   }
-  // a group that gave up waiting lets its copies in flight land (bounded) before it leaves
-  if constexpr (G::STAGE) {
-    if (stalled && t == 0) {
-      for (int b = 0; b < 2; ++b)
-        if ((fill_out >> b) & 1u) tc::mbar_wait_bounded(&s_fill[2 * grp + b], (fill_par >> b) & 1u, 2000000000LL);
-    }
-  }
-  if constexpr (G::TM) {
+  if constexpr (G::TM_ALLOC > 0) {
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -817,83 +922,172 @@ __global__ void __launch_bounds__(Geo<T, N>::THREADS, Geo<T, N>::MINB) collision
   }
   // no CTA leaves while another may still read its shared memory (the last item index)
   if constexpr (CL > 1) cluster_sync<CL>();
+  // every cluster has taken its last item once all have come here: the last one readies the counter
+  // for the next launch
+  if (rank == 0 && tid == 0 && atomicAdd(p.work_counter + kExitWord, 1u) + 1 == gridDim.x / CL) {
+    p.work_counter[0] = 0;
+    p.work_counter[kExitWord] = 0;
+  }
 }
 
-// ------------------------------------------------------------------------------------------
-template <typename T, int N>
-int configure_impl(Plan& pl) {
-  using G = Geo<T, N>;
-  auto kern = collision_kernel<T, N>;
-  // stage the phase block of the current (task, rho) in shared memory when it fits
-  // (with YSH: only while the SM still holds G::RES CTAs with it)
-  const size_t ph_bytes = size_t(pl.max_ent) * 6 * N * sizeof(C<T>);
-  // (with YSH: only while the SM still holds G::RES CTAs with it, else the z phases only)
-  const size_t z_bytes = size_t(pl.max_ent) * 2 * N * sizeof(C<T>);
-  int ph_mode = 0;
-  if (G::YSH) {
-    if (G::RES * (G::SMEM + ph_bytes + 1024) <= size_t(228) * 1024) ph_mode = 1;
-    else if (G::RES * (G::SMEM + z_bytes + 1024) <= size_t(228) * 1024) ph_mode = 2;
-  } else if (G::MINB * (G::SMEM + ph_bytes) <= size_t(200) * 1024) {
-    ph_mode = 1;
-  }
-  const size_t smem = G::SMEM + (ph_mode == 1 ? ph_bytes : ph_mode == 2 ? z_bytes : 0);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+// dynamic shared memory of a shape: the plane buffers and, while MINB CTAs still fit, the phase block
+// of the current (task, rho)
+template <typename T, int N, int W>
+size_t kernel_smem(const Plan& pl, KernelShape& s) {
+  using G = VGeo<T, N, W>;
+  const size_t limit = size_t(226) * 1024 / G::MINB - 2048;  // per CTA while MINB CTAs still fit
+  const size_t ph_bytes = (size_t(pl.max_ent) * G::PB + 1) / 2 * 2 * sizeof(C<T>);
+  s.phase_smem = G::SMEM + ph_bytes <= limit ? 1 : 0;
+  const size_t used = G::SMEM + (s.phase_smem ? ph_bytes : 0);
+  return used;
+}
+
+inline void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cluster, int clusters, const KernelShape& s,
+                       cudaStream_t st) {
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(clusters * cluster);
+  cfg.blockDim = dim3(s.threads);
+  cfg.dynamicSmemBytes = s.smem;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+}
+
+template <typename T, int N, int W>
+int configure_shape(Plan& pl) {
+  using G = VGeo<T, N, W>;
+  auto kern = collision_kernel<T, N, W>;
+  KernelShape& s = pl.shapes[W == 2 ? 0 : W];
+  s.threads = G::THREADS;
+  s.smem = kernel_smem<T, N, W>(pl, s);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
     return DGFS_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = G::CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(G::CL);
-  cfg.blockDim = dim3(G::THREADS);
-  cfg.dynamicSmemBytes = smem;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters <= 0) {
+  launch_config(cfg, attr, G::CL, 1, s, nullptr);
+  if (cudaOccupancyMaxActiveClusters(&s.clusters, kern, &cfg) != cudaSuccess || s.clusters <= 0) {
     cudaGetLastError();
     return DGFS_ERR_CUDA;
   }
-  if constexpr (G::TM) {
-    // The CTAs an SM can hold by the built kernel's registers, shared memory and threads must
-    // stay within the TMEM columns: a CTA that could not allocate would wait inside its
-    // cluster.  (The launch bounds size the registers for RES CTAs, whose allocations fit; a
-    // build with fewer registers could let more in.)
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return DGFS_ERR_CUDA;
-    const int warps = (G::THREADS + 31) / 32;
-    const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
-    const int by_regs = regs_warp > 0 ? 65536 / (regs_warp * warps) : 32;
-    const int by_smem = int(size_t(228) * 1024 / (smem + fa.sharedSizeBytes + 1024));
-    int most = 2048 / G::THREADS;
-    if (by_regs < most) most = by_regs;
-    if (by_smem < most) most = by_smem;
-    if (most < 1 || most * G::TM_ALLOC > 512) return DGFS_ERR_CUDA;
+  if constexpr (G::TM_ALLOC > 0) {
     // The occupancy calculator grants a kernel that allocates tensor memory one CTA per SM; the
-    // device co-schedules `most`.  Clusters beyond what it places wait, and the work counter
-    // leaves them the items still open when they start.
+    // device co-schedules what registers, shared memory and threads allow.
+    cudaFuncAttributes fa;
     int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return DGFS_ERR_CUDA;
+    if (G::CL > 1) {
+      // A CTA that waits for columns inside a cluster must not wait for another waiting cluster:
+      // each CTA asks for at least its columns' share of the SM's shared memory, so whatever mix of
+      // such kernels an SM holds, their columns fit.  (A kernel without clusters waits for nobody
+      // once it has its columns.)
+      const size_t least = (size_t(228) * 1024 * G::TM_ALLOC + 511) / 512 - 1024 - fa.sharedSizeBytes;
+      if (s.smem < least) s.smem = least;
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
+        return DGFS_ERR_CUDA;
+    }
+    const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
+    int most = 65536 / (regs_warp * ((G::THREADS + 31) / 32));
+    const int by_smem = int(size_t(228) * 1024 / (s.smem + fa.sharedSizeBytes + 1024));
+    if (by_smem < most) most = by_smem;
+    if (2048 / G::THREADS < most) most = 2048 / G::THREADS;
+    if (512 / G::TM_ALLOC < most) most = 512 / G::TM_ALLOC;
+    if (most < 1) return DGFS_ERR_CUDA;
     const int cap = most * sms / G::CL;
-    if (cap > clusters) clusters = cap;
+    if (cap > s.clusters) s.clusters = cap;
   }
-  pl.shape.cluster = G::CL;
-  pl.shape.groups = G::GP;
-  pl.shape.threads = G::THREADS;
-  pl.shape.smem = smem;
-  pl.shape.phase_smem = ph_mode;
-  pl.shape.clusters = clusters;
-  pl.scratch_bytes = size_t(clusters) * G::SLOT * G::N3 * sizeof(C<T>);
   return DGFS_OK;
 }
 
 template <typename T, int N>
-int launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
-  using G = Geo<T, N>;
-  KernelParams kp;
+int vhs_configure_impl(Plan& pl) {
+  using G = VGeo<T, N, 0>;
+  if (int rc = configure_shape<T, N, 0>(pl)) return rc;
+  if constexpr (HasWide<T, N>::value) {
+    if (int rc = configure_shape<T, N, 1>(pl)) return rc;
+  }
+  pl.shape.cluster = G::CL;
+  pl.shape.groups = G::GP;
+  pl.shape.threads = G::THREADS;
+  pl.shape.smem = pl.shapes[0].smem;
+  pl.shape.clusters = pl.shapes[0].clusters;
+  pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
+  // one workspace per cluster of either shape, then the products of split items
+  int most = pl.shapes[0].clusters;
+  if (pl.shapes[1].clusters > most) most = pl.shapes[1].clusters;
+  pl.part_off = size_t(most) * pl.shape.slot;
+  pl.part_slots = kPartsPerCluster * most;
+  pl.scratch_bytes = (pl.part_off + size_t(pl.part_slots) * G::HN3) * sizeof(C<T>);
+  return DGFS_OK;
+}
+
+template <typename T, int N>
+int vss_configure_impl(Plan& pl) {
+  using G = VGeo<T, N, 2>;
+  if (int rc = configure_shape<T, N, 2>(pl)) return rc;
+  pl.shape.cluster = G::CL;
+  pl.shape.groups = G::GP;
+  pl.shape.threads = G::THREADS;
+  pl.shape.smem = pl.shapes[0].smem;
+  pl.shape.clusters = pl.shapes[0].clusters;
+  pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
+  pl.scratch_bytes = size_t(pl.shapes[0].clusters) * pl.shape.slot * sizeof(C<T>);
+  return DGFS_OK;
+}
+
+// How a launch of `items` work items (task, node) runs: the shape W and the number of chunks each
+// item's radial nodes are split into, by a cost model in units of one radial node of the dearest
+// task on a full device.  A chunk of `len` nodes costs len + 1/2 (its own f_hat).  Chunks go out one
+// by one, so a launch takes its share of the device, sum of costs / clusters, and about 0.38 of the
+// last chunk; a chunk on a nearly idle device runs at 0.6 of its cost.  Fitted to N = 24, 45 nodes
+// (W = 0: 1.42, 1.21, 1.11, 0.98, 1.10 ms with 1, 2, 4, 6, 12 chunks) and N = 32, 5 nodes, 3 species
+// (W = 0: 2.30, 1.22, 0.99, 1.11 ms with 1, 4, 8, 16; W = 1: 0.97, 0.74, 0.75, 0.84 with 1, 2, 4, 16).
+// The wide shape takes `slow` times longer per node and cluster-share of the device.  All products
+// of all items must fit the parts buffer.
+struct LaunchPlan {
+  int wide = 0, chunks = 1;
+};
+inline LaunchPlan plan_launch(int items, int n_rho, int clusters0, int clusters1, double slow, double mean_cost,
+                           int part_slots) {
+  LaunchPlan best;
+  double best_t = 1e300;
+  for (int w = 0; w < 2; ++w) {
+    const int C = w == 0 ? clusters0 : clusters1;
+    if (C <= 0) continue;
+    const double unit = w == 0 ? 1.0 : slow * double(clusters1) / double(clusters0);
+    for (int s = 1; s <= n_rho; ++s) {
+      if (s > 1 && double(items) * n_rho > double(part_slots)) break;
+      const int len = (n_rho + s - 1) / s;
+      if (s > 1 && (n_rho + s - 2) / (s - 1) == len) continue;  // no shorter than with s - 1 chunks
+      const double one = 0.5 + len, share = double(items) * s * mean_cost * one / C + 0.38 * one;
+      const double t = (share > 0.6 * one ? share : 0.6 * one) * unit;
+      if (t < best_t * (1.0 - 1e-9)) {
+        best_t = t;
+        best.wide = w;
+        best.chunks = s;
+      }
+    }
+  }
+  return best;
+}
+
+template <typename T, int N, int W>
+int launch_shape(const Plan& pl, KernelParams& kp, int items, int limit, cudaStream_t st) {
+  using G = VGeo<T, N, W>;
+  const KernelShape& s = pl.shapes[W == 2 ? 0 : W];
+  kp.phase_smem = s.phase_smem;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  launch_config(cfg, attr, G::CL, items < limit ? items : limit, s, st);
+  return cudaLaunchKernelEx(&cfg, collision_kernel<T, N, W>, kp) == cudaSuccess ? DGFS_OK : DGFS_ERR_CUDA;
+}
+
+inline KernelParams kernel_params(const Plan& pl, const void* f, void* Q, int batch, int ws) {
+  KernelParams kp{};
   kp.f = f;
   kp.Q = Q;
   kp.batch = batch;
@@ -903,37 +1097,48 @@ int launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t 
   kp.max_ent = pl.max_ent;
   kp.tasks = pl.d_tasks;
   kp.groups = pl.d_groups;
-  kp.ent_w = pl.d_ent_w;
+  kp.faces = pl.d_faces;
   kp.phase = pl.d_phase;
   kp.Fw = pl.d_Fwf ? static_cast<const void*>(pl.d_Fwf) : static_cast<const void*>(pl.d_Fw);
-  kp.Gm = pl.d_Gmf ? static_cast<const void*>(pl.d_Gmf) : static_cast<const void*>(pl.d_Gm);
-  kp.scratch = pl.scratch_of(ws);
-  kp.phase_smem = pl.shape.phase_smem;
-  kp.work_counter = pl.counter_of(ws);
-  kp.vss = pl.vss ? 1 : 0;
-  kp.n_fslot = pl.n_fslot;
   kp.Fv = pl.d_Fvf ? static_cast<const void*>(pl.d_Fvf) : static_cast<const void*>(pl.d_Fv);
+  kp.Gm = pl.d_Gmf ? static_cast<const void*>(pl.d_Gmf) : static_cast<const void*>(pl.d_Gm);
   kp.ent_m = pl.d_ent_m;
-  kp.ent_ysh = pl.d_ent_ysh;
+  kp.n_fslot = pl.n_fslot;
+  kp.scratch = pl.scratch_of(ws);
+  kp.slot = pl.shape.slot;
+  kp.work_counter = pl.counter_of(ws);
+  kp.chunks = 1;
+  return kp;
+}
+
+template <typename T, int N>
+int vss_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
+  KernelParams kp = kernel_params(pl, f, Q, batch, ws);
+  const int n = int(pl.shapes[0].clusters * pl.shape.share);
+  return launch_shape<T, N, 2>(pl, kp, batch * kp.n_tasks, n < 1 ? 1 : n, st);
+}
+
+template <typename T, int N>
+int vhs_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
+  KernelParams kp = kernel_params(pl, f, Q, batch, ws);
+  kp.parts = static_cast<C<T>*>(pl.scratch_of(ws)) + pl.part_off;
+  auto share_of = [&](int clusters) {
+    const int n = int(clusters * pl.shape.share);
+    return n < 1 ? 1 : n;
+  };
   const int items = batch * kp.n_tasks;
-  int limit = int(pl.shape.clusters * pl.shape.share);
-  if (limit < 1) limit = 1;
-  const int clusters = items < limit ? items : limit;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = G::CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(clusters * G::CL);
-  cfg.blockDim = dim3(G::THREADS);
-  cfg.dynamicSmemBytes = pl.shape.smem;
-  cfg.stream = st;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if (cudaMemsetAsync(kp.work_counter, 0, sizeof(unsigned), st) != cudaSuccess) return DGFS_ERR_CUDA;
-  if (cudaLaunchKernelEx(&cfg, collision_kernel<T, N>, kp) != cudaSuccess) return DGFS_ERR_CUDA;
-  return DGFS_OK;
+  const int c0 = share_of(pl.shapes[0].clusters), c1 = pl.shapes[1].clusters > 0 ? share_of(pl.shapes[1].clusters) : 0;
+  double cost = 0.0, most = 0.0;
+  for (const TaskDesc& t : pl.tasks) {
+    cost += t.n_ent;
+    most = t.n_ent > most ? t.n_ent : most;
+  }
+  const LaunchPlan run = plan_launch(items, pl.N_rho, c0, c1, HasWide<T, N>::slow, cost / (kp.n_tasks * most), pl.part_slots);
+  kp.chunks = run.chunks;
+  if constexpr (HasWide<T, N>::value) {
+    if (run.wide) return launch_shape<T, N, 1>(pl, kp, items * run.chunks, c1, st);
+  }
+  return launch_shape<T, N, 0>(pl, kp, items * run.chunks, c0, st);
 }
 
 }  // namespace dgfs

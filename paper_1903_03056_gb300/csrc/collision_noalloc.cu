@@ -19,7 +19,8 @@
 
 #include <cuda.h>
 
-#include "collision_kernel.cuh"
+#include "dgfs_internal.h"
+#include "group_sync.cuh"
 
 namespace dgfs {
 namespace {
@@ -67,6 +68,28 @@ template <int N>
 __device__ __forceinline__ float kabs(int n0, int pp) {
   const float kx = float(centred(n0, N)), ky = float(centred(pp / N, N)), kz = float(centred(pp % N, N));
   return sqrtf(kx * kx + ky * ky + kz * kz);
+}
+
+// transpose a plane held as column t (x[r] = V[r][t]) into row t (x[c] = V[t][c]) and back
+template <typename T, int N, int GP>
+__device__ __forceinline__ void cols_to_rows(C<T> (&x)[N], C<T>* tb, int t) {
+  constexpr int P = N + 1;
+#pragma unroll
+  for (int r = 0; r < N; ++r) tb[r * P + t] = x[r];
+  group_sync<N, GP>();
+#pragma unroll
+  for (int c = 0; c < N; ++c) x[c] = tb[t * P + c];
+  group_sync<N, GP>();
+}
+template <typename T, int N, int GP>
+__device__ __forceinline__ void rows_to_cols(C<T> (&x)[N], C<T>* tb, int t) {
+  constexpr int P = N + 1;
+#pragma unroll
+  for (int c = 0; c < N; ++c) tb[t * P + c] = x[c];
+  group_sync<N, GP>();
+#pragma unroll
+  for (int r = 0; r < N; ++r) x[r] = tb[r * P + t];
+  group_sync<N, GP>();
 }
 
 // one work item per CTA at a time (no cluster); plane groups of N threads, one plane each

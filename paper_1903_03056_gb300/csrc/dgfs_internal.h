@@ -55,20 +55,17 @@ struct KernelParams {
   const GroupDesc* groups;
   const int* faces;       // face codes of the tasks: 2 e + kind, e the entry within its task, kind 0
                           // (k_x = N/2) if sigma_x != 0, kind 1 (k_y = N/2) if sigma_y != 0
-  const double* ent_w;    // [entries] sigma weight (x2 for halved self pairs)
-  const void* phase;      // complex: [task][rho][max_ent][role 2][axis 3][N]
+  const void* phase;      // complex: [task][rho][max_ent] phase blocks (VGeo::PB, plan.cpp)
   const void* Fw;         // [s*s][n_rho][N^3]: w_rho F^(ij)(k, rho) / N^3, in the plan's real
                           // type (FP32 plans: each FP64 value rounded once)
   const void* Gm;         // [s*s][N^3]: G^(ij)-(k), in the plan's real type
   void* scratch;          // complex: [clusters][slot]
-  size_t slot;            // complex values of workspace per cluster (VHS kernel)
-  void* parts;            // complex: [item][rho][N^3 / 2] products of split work items (VHS kernel)
-  int chunks;             // chunks a work item's radial nodes are split into (VHS kernel)
-  int phase_smem;         // 1: the task's phase block of the current rho is staged in smem;
-                          // 2: only its z phases are
-  unsigned* work_counter; // next work item (reset to 0 before every launch)
+  size_t slot;            // complex values of workspace per cluster
+  void* parts;            // complex: [item][rho][N^3 / 2] products of split work items
+  int chunks;             // chunks a work item's radial nodes are split into
+  int phase_smem;         // the phase block of the current (task, rho) is staged in shared memory
+  unsigned* work_counter; // next work item, device status, exits, finished chunks (kExitWord, kDoneWord)
   // VSS (alpha != 1): sigma-dependent complex gain weights, one forward transform per entry
-  int vss;
   int n_fslot;            // table slots per (pair, rho): M, or M / 2 with an antipodal design
   const void* Fv;         // [s*s][n_rho][n_fslot][N^3]: w_rho F^(ij)(k, rho, sigma) / N^3,
                           // complex in the plan's real type; with an antipodal design a slot
@@ -78,9 +75,6 @@ struct KernelParams {
   const int* ent_m;       // [entries][2]: slot code (2 slot + conjugation bit) of the entry's
                           // direction and of its antipode (-1: none); a self pair's entry with
                           // an antipode takes F(sigma) + F(-sigma)
-  const int* ent_ysh;     // [entries]: 1 when the entry has the previous entry's sigma_x and
-                          // sigma_y (same group), so both its shifted volumes share that
-                          // entry's x and y passes
 };
 
 // Conservation projection of one self pair (rows = 5) or one stacked cross pair (rows = 6):
@@ -108,8 +102,8 @@ constexpr int kExitWord = 2, kDoneWord = 64;
 // products (one radial node of one item) the VHS workspace holds per resident cluster
 constexpr int kPartsPerCluster = 6;
 
-// one launch shape of the VHS kernel
-struct VhsShape {
+// one launch shape of the collision kernel
+struct KernelShape {
   int threads = 0, phase_smem = 0, clusters = 0;
   size_t smem = 0;
 };
@@ -165,7 +159,6 @@ struct Plan {
   float2* d_Fvf = nullptr;
   float* d_Gmf = nullptr;
   int* d_ent_m = nullptr;
-  int* d_ent_ysh = nullptr;
   int* d_faces = nullptr;
   double* d_Gm = nullptr;
   double* d_ent_w = nullptr;
@@ -176,7 +169,7 @@ struct Plan {
 
   // workspace
   LaunchShape shape;
-  VhsShape vhs[2];                 // VHS plans: the batch shape and the wide one (clusters = 0: none)
+  KernelShape shapes[2];           // the batch shape and (VHS) the wide one (clusters = 0: none)
   size_t part_off = 0;             // VHS plans: the split items' products in the workspace (complex values)
   int part_slots = 0;              // and how many there is room for
   size_t counter_bytes() const { return (kDoneWord + size_t(part_slots)) * sizeof(unsigned); }
@@ -228,14 +221,14 @@ int upload_plan(Plan& p);
 void free_plan(Plan& p);
 
 // kernel configuration and launch, per precision (collision_f32.cu / collision_f64.cu)
+int configure_vss_f32(Plan& p);
+int configure_vss_f64(Plan& p);
 int configure_f32(Plan& p);
 int configure_f64(Plan& p);
-int configure_vhs_f32(Plan& p);
-int configure_vhs_f64(Plan& p);
-int launch_vhs_f32(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
-int launch_vhs_f64(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
 int launch_f32(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
 int launch_f64(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
+int launch_vss_f32(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
+int launch_vss_f64(const Plan& p, const void* f, void* Q, int batch, cudaStream_t st, int ws = 0);
 
 // on-device FP64 weight tables on the plan's stream (tables.cu)
 int launch_vhs_tables(Plan& p, const double* d_fcoef, const double* d_gcoef, const double* d_gscale, int n_loss);

@@ -548,11 +548,31 @@ int upload_plan(Plan& p) {
       }
     }
   // phase factors exp(i pi shift_d k / L) per task, radial node, entry, role, axis
-  // the VHS kernel takes its tasks in order of falling cost
-  const bool vhs = !p.vss && p.precision != DGFS_BF16X3;
+  // the collision kernel takes its tasks in order of falling cost
+  const bool fft = p.precision != DGFS_BF16X3;
   std::vector<TaskDesc> tasks = p.tasks;
-  if (vhs)
+  if (fft)
     std::stable_sort(tasks.begin(), tasks.end(), [](const TaskDesc& a, const TaskDesc& c) { return a.n_ent > c.n_ent; });
+  // VSS: two neighbouring entries with the same sigma_x share a group, and with it the x pass, the
+  // barriers of a phase and the accumulators in L2
+  std::vector<GroupDesc> groups = p.groups;
+  if (p.vss) {
+    groups.clear();
+    for (TaskDesc& tk : tasks) {
+      const int off = tk.grp_off, n = tk.n_grp;
+      tk.grp_off = int(groups.size());
+      for (int g = 0; g < n; ++g) {
+        const GroupDesc& gd = p.groups[size_t(off) + g];
+        auto sx = [&](int e) { return p.sigma[3 * size_t(p.ent_sigma[tk.ent_off + e])]; };
+        GroupDesc* last = int(groups.size()) > tk.grp_off ? &groups.back() : nullptr;
+        if (last && last->count == 1 && last->zero == gd.zero && std::fabs(sx(last->first) - sx(gd.first)) <= 1e-12)
+          last->count = 2;
+        else
+          groups.push_back(gd);
+      }
+      tk.n_grp = int(groups.size()) - tk.grp_off;
+    }
+  }
   const int NT = int(tasks.size());
   auto phase_of = [&](int t, int q, int e, int role, int ax, int n) {
     const TaskDesc& tk = tasks[t];
@@ -565,7 +585,7 @@ int upload_plan(Plan& p) {
     return std::complex<double>(std::cos(arg), std::sin(arg));
   };
   std::vector<std::complex<double>> ph;
-  if (!vhs) {
+  if (!fft) {
     // [task][rho][entry][role][axis][N]
     ph.assign(size_t(NT) * NR * p.max_ent * 2 * 3 * N, std::complex<double>(0.0, 0.0));
     for (int t = 0; t < NT; ++t)
@@ -576,7 +596,7 @@ int upload_plan(Plan& p) {
               for (int n = 0; n < N; ++n)
                 ph[((((size_t(t) * NR + q) * p.max_ent + e) * 2 + role) * 3 + ax) * N + n] = phase_of(t, q, e, role, ax, n);
   } else {
-    // [task][rho][entry] blocks of the VHS kernel: x [N/2][role], y [N/2][role], z [role][N/2] (role 1
+    // [task][rho][entry] blocks of the collision kernel: x [N/2][role], y [N/2][role], z [role][N/2] (role 1
     // times the weight w_e), then (w_e, 0) and a pad.  Modes 1..N/2-1 (their negatives take the
     // conjugate); the slot of mode 0, whose phase is 1, holds the unpaired mode's c + i t
     const size_t PB = 3 * size_t(N) + 2;
@@ -756,10 +776,9 @@ int upload_plan(Plan& p) {
       total = total - nF * sizeof(double) + nF * sizeof(float);
     }
   }
-  if ((rc = upload(p, p.ent_w.data(), p.ent_w.size(), (void**)&p.d_ent_w, total))) return rc;
+  if (p.precision == DGFS_BF16X3 && (rc = upload(p, p.ent_w.data(), p.ent_w.size(), (void**)&p.d_ent_w, total))) return rc;
   if ((rc = upload(p, tasks.data(), tasks.size(), (void**)&p.d_tasks, total))) return rc;
-  if ((rc = upload(p, p.groups.data(), p.groups.size(), (void**)&p.d_groups, total))) return rc;
-  if ((rc = upload(p, p.ent_ysh.data(), p.ent_ysh.size(), (void**)&p.d_ent_ysh, total))) return rc;
+  if ((rc = upload(p, groups.data(), groups.size(), (void**)&p.d_groups, total))) return rc;
   if (!p.faces.empty() && (rc = upload(p, p.faces.data(), p.faces.size(), (void**)&p.d_faces, total))) return rc;
   if (!mats.empty() && (rc = upload(p, mats.data(), mats.size(), (void**)&p.d_mats, total))) return rc;
   if (p.f32io()) {
@@ -799,7 +818,7 @@ int upload_plan(Plan& p) {
 void free_plan(Plan& p) {
   void* ptrs[] = {p.d_Fw,      p.d_Gm,      p.d_ent_w,   p.d_phase, p.d_tasks, p.d_groups, p.d_Fv,
                   p.d_scratch_raw, p.d_stage_f, p.d_stage_Q, p.d_cons, p.d_kappa, p.d_Qfull, p.d_ent_m,
-                  p.d_counter, p.d_rk,      p.d_ent_ysh, p.d_Fwf,    p.d_Fvf,   p.d_Gmf,   p.d_mats,
+                  p.d_counter, p.d_rk,      p.d_Fwf,    p.d_Fvf,   p.d_Gmf,   p.d_mats,
                   p.d_scratch2_raw, p.d_counter2, p.d_faces, p.d_lam};
   if (p.home) {
     for (void* q : ptrs)
@@ -838,7 +857,6 @@ void free_plan(Plan& p) {
   p.d_Fvf = nullptr;
   p.d_Gmf = nullptr;
   p.d_ent_m = nullptr;
-  p.d_ent_ysh = nullptr;
   p.d_counter = nullptr;
   p.d_rk = nullptr;
   p.d_mats = nullptr;

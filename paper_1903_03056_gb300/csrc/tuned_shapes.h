@@ -1,21 +1,51 @@
-// Launch shape of collision_kernel<T, N>: thread-block cluster size, plane groups per CTA and
-// the CTAs per SM the registers are sized for.  Written by paper_1903_03056_gb300/tune.py from
-// timings on the device (record: tuned_shapes.json); edit by re-running the tuner.
+// Launch shapes of collision_kernel<T, N, W>: thread-block cluster size, plane groups per CTA and the
+// CTAs per SM the registers are sized for.  DGFS_SHAPE3: VHS batches, written by
+// paper_1903_03056_gb300/tune.py from timings on the device (record: tuned_shapes.json); DGFS_WIDE: the
+// shape of small VHS batches where they use one of their own; DGFS_VSS: VSS plans.
 #pragma once
 
-DGFS_SHAPE(float, 4, 1, 4)
-DGFS_SHAPE(float, 6, 1, 6)
-DGFS_SHAPE(float, 8, 1, 8)
-DGFS_SHAPE(float, 12, 1, 12)
-DGFS_SHAPE3(float, 16, 1, 8, 3)
+DGFS_SHAPE3(float, 4, 1, 4, 1)
+DGFS_SHAPE3(float, 6, 1, 6, 1)
+DGFS_SHAPE3(float, 8, 1, 8, 1)
+DGFS_SHAPE3(float, 12, 1, 12, 1)
+DGFS_SHAPE3(float, 16, 1, 8, 4)
 DGFS_SHAPE3(float, 24, 1, 8, 2)
-DGFS_SHAPE3(float, 32, 8, 4, 3)
-DGFS_SHAPE3(float, 48, 2, 4, 1)
-DGFS_SHAPE(double, 4, 1, 4)
-DGFS_SHAPE(double, 6, 1, 6)
-DGFS_SHAPE(double, 8, 1, 8)
-DGFS_SHAPE(double, 12, 1, 12)
-DGFS_SHAPE(double, 16, 1, 8)
-DGFS_SHAPE(double, 24, 2, 6)
-DGFS_SHAPE(double, 32, 4, 4)
-DGFS_SHAPE(double, 48, 4, 1)
+DGFS_SHAPE3(float, 32, 2, 4, 3)
+DGFS_SHAPE3(float, 48, 4, 4, 2)
+DGFS_SHAPE3(double, 4, 1, 4, 1)
+DGFS_SHAPE3(double, 6, 1, 6, 1)
+DGFS_SHAPE3(double, 8, 1, 8, 1)
+DGFS_SHAPE3(double, 12, 1, 12, 1)
+DGFS_SHAPE3(double, 16, 1, 8, 1)
+DGFS_SHAPE3(double, 24, 6, 4, 1)
+DGFS_SHAPE3(double, 32, 4, 4, 2)
+DGFS_SHAPE3(double, 48, 4, 1, 1)
+
+// ... and how many times longer the wide shape takes per radial node on a full device (measured:
+// N = 16 7.16 / 4.72 ms, 24 15.2 / 10.6, 32 14.1 / 12.4, 48 13.9 / 10.8; FP64 8 6.70 / 3.25,
+// 12 10.7 / 9.47, 16 12.7 / 11.2)
+DGFS_WIDE(float, 16, 8, 2, 1, 1.5)
+DGFS_WIDE(float, 24, 6, 4, 5, 1.43)
+DGFS_WIDE(float, 32, 8, 4, 3, 1.14)
+DGFS_WIDE(float, 48, 8, 6, 1, 1.29)
+DGFS_WIDE(double, 8, 4, 2, 1, 2.06)
+DGFS_WIDE(double, 12, 6, 2, 1, 1.13)
+DGFS_WIDE(double, 16, 8, 2, 1, 1.13)
+
+// VSS plans (W = 2)
+DGFS_VSS(float, 4, 1, 4, 1)
+DGFS_VSS(float, 6, 1, 6, 1)
+DGFS_VSS(float, 8, 1, 8, 1)
+DGFS_VSS(float, 12, 1, 12, 1)
+DGFS_VSS(float, 16, 2, 8, 4)
+DGFS_VSS(float, 24, 1, 8, 2)
+DGFS_VSS(float, 32, 2, 4, 3)
+DGFS_VSS(float, 48, 8, 2, 4)
+DGFS_VSS(double, 4, 1, 4, 1)
+DGFS_VSS(double, 6, 1, 6, 1)
+DGFS_VSS(double, 8, 1, 8, 1)
+DGFS_VSS(double, 12, 1, 12, 1)
+DGFS_VSS(double, 16, 1, 8, 1)
+DGFS_VSS(double, 24, 6, 4, 1)
+DGFS_VSS(double, 32, 4, 4, 2)
+DGFS_VSS(double, 48, 4, 1, 1)

@@ -13,7 +13,8 @@ thread computes a line, never the arithmetic of a line), and keeps the fastest. 
 in csrc/tuned_shapes.json; rebuild afterwards.
 
 With --radix it times, per N, every order of the radices 8, 4, 2, 3 in the candidate list
-(tuned_radix.h codes) of the FP32 kernel instead.  A schedule changes the rounding of a line,
+(tuned_radix.h codes) of the FP32 kernel instead; a line of N runs as transforms of N / 2 points, so
+the schedule of N / 2 is the one that is tried.  A schedule changes the rounding of a line,
 so its output is checked against the FP64 path on the first nodes of the workload (the largest
 per-node max |Q - Q_fp64| / max |Q_fp64| must stay below the FP32 bar, 1e-5); the fastest
 schedule that passes is kept.  (FP64 schedules stay at the default order: an FP64 variant has
@@ -53,6 +54,7 @@ CANDIDATES = {
 RADIX_H = os.path.join(CSRC, "tuned_radix.h")
 # orders of the radix multisets of each N (4-stage and longer schedules left out)
 RADIX_CANDIDATES = {
+    8: [42, 24, 8, 222],
     12: [43, 34, 223, 232, 322],
     16: [44, 82, 28, 422, 242, 224],
     24: [423, 83, 38, 432, 243, 342, 234, 324],
@@ -84,9 +86,10 @@ def _patch_radix(text, T, N, line):
 
 
 def geometry(N, C, GP, MB, csize):
-    """The kernel's compile-time geometry of a shape (the same rules as its Geo template):
-    P in registers, CTAs per SM, y-pass sharing, tensor-memory accumulators, plane buffers per
-    group and the shared memory of the plane buffers.  csize = bytes of one complex element."""
+    """Geometry rules of the complex-transform kernel that the records up to the real-transform
+    kernel were taken with: P in registers, CTAs per SM, y-pass sharing, tensor-memory
+    accumulators, plane buffers per group and their shared memory.  Kept to read those records;
+    ``valid`` follows the present kernel.  csize = bytes of one complex element."""
     preg = (csize == 8 and N <= 48) or N <= 16
     buf = N * (N + 1) * csize
     threads = GP * N
@@ -105,14 +108,19 @@ def geometry(N, C, GP, MB, csize):
             "smem": GP * nbuf * buf}
 
 
+def kernel_smem(N, GP, csize):
+    """Shared memory of a CTA's plane groups (VGeo::SMEM without its few bytes of padding): a padded
+    plane and a face row each, and P where an FP64 line leaves it no registers."""
+    return GP * ((N * (N + 1) + N) * csize + (N * N * 8 if csize == 16 and N >= 48 else 0))
+
+
 def valid(N, C, GP, MB, csize):
     """Shape constraints of the kernel: planes and pencils split evenly over the cluster and
     the plane groups, at most 1024 threads, the plane buffers of MB CTAs in one SM's shared
     memory, and at least 64 registers a thread at MB CTAs per SM."""
     if N % C or (N * N) % C or (N // C) % GP or GP * N > 1024:
         return False
-    g = geometry(N, C, GP, MB, csize)
-    return MB * g["smem"] <= 227 * 1024 and 65536 // (g["threads"] * MB) >= 64
+    return MB * kernel_smem(N, GP, csize) <= 227 * 1024 and 65536 // (GP * N * MB) >= 64
 
 
 def _ctype(precision):
@@ -153,7 +161,7 @@ def _variant(tmp, precision, N, shape, radix=None):
         with open(rh) as fh:
             text = fh.read()
         with open(rh, "w") as fh:
-            fh.write(_patch_radix(text, T, N, _radix_line(T, N, radix)))
+            fh.write(_patch_radix(text, T, N // 2, _radix_line(T, N // 2, radix)))
     tu = "collision_f32" if precision == "fp32" else "collision_f64"
     obj = os.path.join(pkg, "_build", tu + ".o")
     cmd = ([build.nvcc()] + build.ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC",
@@ -253,15 +261,15 @@ def tune_radix(precision="fp32", sizes=(16, 24, 32, 48), write=False, jobs=8):
     with open(RADIX_H) as fh:
         header = fh.read()
     with tempfile.TemporaryDirectory(prefix="dgfs_tune_") as tmp:
-        todo = [(N, code) for N in sizes for code in RADIX_CANDIDATES.get(N, []) if radix_code_valid(N, code)]
+        todo = [(N, code) for N in sizes for code in RADIX_CANDIDATES.get(N // 2, []) if radix_code_valid(N // 2, code)]
         with ThreadPoolExecutor(max_workers=jobs) as ex:
             roots = dict(zip(todo, ex.map(lambda t: _variant(tmp, precision, t[0], current_shape(precision, t[0]),
                                                              radix=t[1]), todo)))
         for N in sizes:
             workload, batch = WORKLOAD_FOR_N[N]
-            cur = current_radix(precision, N)
+            cur = current_radix(precision, N // 2)
             rows = []
-            for code in RADIX_CANDIDATES.get(N, []):
+            for code in RADIX_CANDIDATES.get(N // 2, []):
                 if (N, code) not in roots:
                     continue
                 r = _time(roots[(N, code)], workload, batch, precision, compare=RADIX_CHECK_NODES)
@@ -276,7 +284,7 @@ def tune_radix(precision="fp32", sizes=(16, 24, 32, 48), write=False, jobs=8):
             record["radix/%s/%d" % (precision, N)] = {"workload": workload, "batch": batch, "previous": cur,
                                                      "shape": list(current_shape(precision, N)), "best": best,
                                                      "candidates": rows}
-            header = _patch_radix(header, T, N, _radix_line(T, N, best["radix"]))
+            header = _patch_radix(header, T, N // 2, _radix_line(T, N // 2, best["radix"]))
     if write:
         with open(RADIX_H, "w") as fh:
             fh.write(header)
