@@ -134,6 +134,8 @@ struct VGeo {
   static constexpr bool TMR = TMOK && fits(SETS * (2 * N + (TMP ? P_COLS : 0)));
   static constexpr int TM_SET = (TMR ? 2 * N : 0) + (TMP ? P_COLS : 0);  // columns of a thread
   static constexpr int TM_ALLOC = TM_SET > 0 ? alloc_of(SETS * TM_SET) : 0;
+  static constexpr bool CALL = sizeof(T) == 4 && W == 0 && (N == 24 || N == 32);  // add_parts
+  static constexpr int QU = W == 1 || N <= 12 ? 8 : CALL || sizeof(T) == 8 ? 4 : 2;
   // shared memory per group: one padded plane, the entry's row of the k_y face, P if PSM
   // (FP32: the groups' stride is 2 N words modulo 32, so that the lanes of a warp that spans two
   // groups hit distinct banks: N = 24)
@@ -230,12 +232,26 @@ template <int N>
 __device__ __forceinline__ void rows_c2r(const double2* row, const double2* phz, double2 x0, double2 xh,
                                          Rows<double, N>& y) {
   constexpr int h = N / 2;
+  // a shift of zero along z leaves role 0 as it is and scales role 1 by its weight (bound by the FP64
+  // pipe: half the multiplications of those rows)
+  const bool plain = phz == nullptr || (phz[0].y == 0.0 && phz[h].y == 0.0);
   double2 x[h];
+  if (plain) {
 #pragma unroll
-  for (int k = 1; k < h; ++k) x[k] = phz != nullptr ? cmul<double>(row[k], phz[k]) : row[k];
+    for (int k = 1; k < h; ++k) x[k] = row[k];
+  } else {
+#pragma unroll
+    for (int k = 1; k < h; ++k) x[k] = cmul<double>(row[k], phz[k]);
+  }
   c2r_line<double, N>(x, x0.x, xh.x, y.a);
+  if (plain) {
+    const double w = phz != nullptr ? phz[h].x : 1.0;
 #pragma unroll
-  for (int k = 1; k < h; ++k) x[k] = phz != nullptr ? cmul<double>(row[h + k], phz[h + k]) : row[h + k];
+    for (int k = 1; k < h; ++k) x[k] = scale<double>(row[h + k], w);
+  } else {
+#pragma unroll
+    for (int k = 1; k < h; ++k) x[k] = cmul<double>(row[h + k], phz[h + k]);
+  }
   c2r_line<double, N>(x, x0.y, xh.y, y.b);
 }
 
@@ -363,6 +379,76 @@ __device__ __forceinline__ void vss_step_c(const KernelParams& p, const TaskDesc
   }
 }
 
+// Gain of a split work item from its stored products PT [rho][k_x][pencil], this CTA's pencils, QU radial
+// nodes of loads in flight per thread.  It runs once per split item, but inside the kernel its pointers
+// and loads cost the inner loops registers, so the batch shapes trade: N = 24 and 32 call it out of line
+// with QU = 4 (45 nodes of N = 24 0.80 ms; inline 8: 0.81, but batches 36.6 -> 37.2 ms), N = 16 and 48
+// inline it with QU = 2 (batches 16.3 and 35.6 ms; out of line 16.6 and 36.7).
+template <typename T, int N, int W>
+__device__ __forceinline__ void add_parts(const C<T>* PT, const T* Fp, C<T>* QA, C<T>* QB, int out0, int out1, int n_rho,
+                                       int plane0, int tid) {
+  using G = VGeo<T, N, W>;
+  using CT = C<T>;
+  constexpr int h = G::h, N2 = G::N2, HN2 = G::HN2, NT = G::THREADS;
+  constexpr size_t N3 = G::N3, HN3 = G::HN3;
+  // (bound by L2 latency: one cluster reads all products and weights of the item)
+  constexpr int total = N * G::PLANES * h, QU = G::QU;
+  const T* const F0 = Fp + size_t(out0) * n_rho * N3;
+  const T* const F1 = Fp + size_t(out1 >= 0 ? out1 : out0) * n_rho * N3;
+#pragma unroll 1
+  for (int u = tid; u < total; u += NT) {
+    const int n = u / (G::PLANES * h), pp = plane0 * h + u % (G::PLANES * h);
+    const int r = pp / h, cc = pp % h;
+    if (cc == 0 && (r == 0 || r == h)) continue;  // the pencils that hold two real ones, below
+    const int at = n * HN2 + pp;
+    const int fo = n * N2 + (cc == 0 && r >= h ? (r - h) * N + h : r * N + cc);
+    CT a0 = mk<T>(0, 0), a1 = mk<T>(0, 0);
+#pragma unroll 1
+    for (int q = 0; q < n_rho; q += QU) {
+      CT v[QU];
+      T wa[QU], wb[QU];
+#pragma unroll
+      for (int j = 0; j < QU; ++j)
+        if (q + j < n_rho) {
+          v[j] = ld2<T>(PT + (q + j) * HN3 + at);
+          wa[j] = __ldg(F0 + (q + j) * N3 + fo);
+          wb[j] = __ldg(F1 + (q + j) * N3 + fo);
+        }
+#pragma unroll
+      for (int j = 0; j < QU; ++j)
+        if (q + j < n_rho) {
+          a0 = add_gain<T>(a0, wa[j], v[j], q + j == 0);
+          a1 = add_gain<T>(a1, wb[j], v[j], q + j == 0);
+        }
+    }
+    st2<T>(QA + at, a0);
+    if (out1 >= 0) st2<T>(QB + at, a1);
+  }
+  for (int u = tid; u < 2 * N; u += NT) {  // the pencils (0, 0) and (N/2, 0)
+    const int n = u >> 1, pp = (u & 1) * h * h;
+    if (pp / h < plane0 || pp / h >= plane0 + G::PLANES) continue;
+    const CT* const pv = PT + n * HN2 + pp;
+    const CT* const pm = PT + (n == 0 ? 0 : N - n) * HN2 + pp;
+    for (int o = 0; o < 2; ++o) {
+      const int pair = o == 0 ? out0 : out1;
+      if (pair < 0) break;
+      const T* const Fw = Fp + size_t(pair) * n_rho * N3 + n * N2 + (u & 1) * h;
+      CT acc = mk<T>(0, 0);
+#pragma unroll 4
+      for (int q = 0; q < n_rho; ++q)
+        acc = add_gain_pair<T>(acc, __ldg(Fw + q * N3), __ldg(Fw + q * N3 + h * N), ld2<T>(pv + q * HN3),
+                               ld2<T>(pm + q * HN3), q == 0);
+      st2<T>((o == 0 ? QA : QB) + n * HN2 + pp, acc);
+    }
+  }
+}
+
+template <typename T, int N, int W>
+__device__ __noinline__ void add_parts_call(const C<T>* PT, const T* Fp, C<T>* QA, C<T>* QB, int out0, int out1, int n_rho,
+                                            int plane0, int tid) {
+  add_parts<T, N, W>(PT, Fp, QA, QB, out0, out1, n_rho, plane0, tid);
+}
+
 template <typename T, int N, int W>
 __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) collision_kernel(const KernelParams p) {
   using G = VGeo<T, N, W>;
@@ -426,7 +512,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
     const int whole = item / p.chunks;
     const int b = whole % p.batch;
     const int task = whole / p.batch;
-    const bool split = p.chunks > 1;
+    const bool split = !G::VSS && p.chunks > 1;
     const int q0 = chunk * p.n_rho / p.chunks, q1 = (chunk + 1) * p.n_rho / p.chunks;
     CT* const PT = static_cast<CT*>(p.parts) + size_t(whole) * p.n_rho * HN3;  // P_hat of every radial node
     const TaskDesc tk = p.tasks[task];
@@ -608,7 +694,9 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
                   tm_load<2 * N>(tm_raw, reinterpret_cast<float*>(v));
                 }
                 const T corner = v[h].y;  // of column 0: f on the edge k_y = k_z = N/2
-                shift_line<T, N>(v, pe + N + role);
+                // (a shift of zero has phase 1 throughout; measured: skipping it N = 32 -2.3 %, FP64 N = 32 -1 %,
+                // N = 16, 24, 48 +0.7 to 3 %)
+                if (!(sizeof(T) == 8 || N == 32) || has_y) shift_line<T, N>(v, pe + N + role);
                 const T w = sgx * (role == 0 ? txa * tya : txb * tyb);
                 v[h] = mk<T>(v[h].x - w * fe.x, v[h].y - w * fe.y);
                 line_fft<T, N, +1>(v);
@@ -789,30 +877,10 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
         continue;
       }
       __threadfence();
-      for (int u = tid; u < N * G::PLANES * h; u += NT) {  // element by element: every load independent
-        const int n = u / (G::PLANES * h), pp = plane0 * h + u % (G::PLANES * h);
-        const int r = pp / h, cc = pp % h;
-        const bool pair_row = cc == 0 && (r == 0 || r == h);
-        const int ky = cc == 0 && r >= h ? r - h : r;
-        const int kz = cc == 0 && r >= h ? h : cc;
-        const CT* const pv = PT + n * HN2 + pp;
-        const CT* const pm = PT + (n == 0 ? 0 : N - n) * HN2 + pp;
-        for (int o = 0; o < 2; ++o) {
-          const int pair = o == 0 ? tk.out0 : tk.out1;
-          if (pair < 0) break;
-          const T* const Fw = static_cast<const T*>(p.Fw) + size_t(pair) * p.n_rho * N3 + n * N2 + ky * N + kz;
-          CT acc = mk<T>(0, 0);
-          if (!pair_row) {
-#pragma unroll 8
-            for (int q = 0; q < p.n_rho; ++q) acc = add_gain<T>(acc, __ldg(Fw + q * N3), ld2<T>(pv + q * HN3), q == 0);
-          } else {
-            for (int q = 0; q < p.n_rho; ++q)
-              acc = add_gain_pair<T>(acc, __ldg(Fw + q * N3), __ldg(Fw + q * N3 + h * N), ld2<T>(pv + q * HN3),
-                                     ld2<T>(pm + q * HN3), q == 0);
-          }
-          st2<T>((o == 0 ? QA : QB) + n * HN2 + pp, acc);
-        }
-      }
+      if constexpr (G::CALL)
+        add_parts_call<T, N, W>(PT, static_cast<const T*>(p.Fw), QA, QB, tk.out0, tk.out1, p.n_rho, plane0, tid);
+      else
+        add_parts<T, N, W>(PT, static_cast<const T*>(p.Fw), QA, QB, tk.out0, tk.out1, p.n_rho, plane0, tid);
     }
     __syncthreads();
 
