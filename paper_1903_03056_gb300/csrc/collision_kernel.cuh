@@ -45,8 +45,8 @@
 // Groups hold one or two entries.
 //
 // Measured on the GB300 against the complex-transform kernel this one replaced: 4096 nodes of N = 32
-// FP32 285 -> 144.6 ms, 3001 of N = 24 75.1 -> 36.5, 8192 of N = 16 28.7 -> 16.2, 61 three-species nodes
-// of N = 48 86.0 -> 36.0, 61 nodes of N = 32 FP64 201 -> 85.7, VSS 37 three-species nodes of N = 48
+// FP32 285 -> 145 ms, 3001 of N = 24 75.1 -> 36.6, 8192 of N = 16 28.7 -> 16.3, 61 three-species nodes
+// of N = 48 86.0 -> 35.8, 61 nodes of N = 32 FP64 201 -> 82, VSS 37 three-species nodes of N = 48
 // (M = 32) 339 -> 161 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
 // FMA pipes run half their cycles (N = 16: the L1 data path three quarters), the stalls are L2 loads
 // of the x-passed spectra, whose workspaces together exceed L2 from N = 24 on.
@@ -1010,6 +1010,16 @@ size_t kernel_smem(const Plan& pl, KernelShape& s) {
   return used;
 }
 
+// raise a kernel's dynamic shared memory limit to `smem` (never lower it: plans of one shape share the
+// kernel, and their phase blocks differ)
+template <typename K>
+bool allow_smem(K kern, size_t smem) {
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return false;
+  if (fa.maxDynamicSharedSizeBytes >= int(smem)) return true;
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) == cudaSuccess;
+}
+
 inline void launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int cluster, int clusters, const KernelShape& s,
                        cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -1031,8 +1041,7 @@ int configure_shape(Plan& pl) {
   KernelShape& s = pl.shapes[W == 2 ? 0 : W];
   s.threads = G::THREADS;
   s.smem = kernel_smem<T, N, W>(pl, s);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
-    return DGFS_ERR_CUDA;
+  if (!allow_smem(kern, s.smem)) return DGFS_ERR_CUDA;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   launch_config(cfg, attr, G::CL, 1, s, nullptr);
@@ -1055,8 +1064,7 @@ int configure_shape(Plan& pl) {
       // once it has its columns.)
       const size_t least = (size_t(228) * 1024 * G::TM_ALLOC + 511) / 512 - 1024 - fa.sharedSizeBytes;
       if (s.smem < least) s.smem = least;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem)) != cudaSuccess)
-        return DGFS_ERR_CUDA;
+      if (!allow_smem(kern, s.smem)) return DGFS_ERR_CUDA;
     }
     const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
     int most = 65536 / (regs_warp * ((G::THREADS + 31) / 32));
@@ -1071,6 +1079,14 @@ int configure_shape(Plan& pl) {
   return DGFS_OK;
 }
 
+// Fewer clusters where their workspaces would pass 16 GB: the faces grow with the sphere rule (a
+// thousand directions at N = 32: 17 MB a cluster), and rules of any size stay accepted.
+inline void cap_clusters(Plan& pl, size_t slot_bytes) {
+  const size_t cap = (size_t(16) << 30) / slot_bytes;
+  for (KernelShape& s : pl.shapes)
+    if (size_t(s.clusters) > cap) s.clusters = cap > 0 ? int(cap) : 1;
+}
+
 template <typename T, int N>
 int vhs_configure_impl(Plan& pl) {
   using G = VGeo<T, N, 0>;
@@ -1082,11 +1098,12 @@ int vhs_configure_impl(Plan& pl) {
   pl.shape.groups = G::GP;
   pl.shape.threads = G::THREADS;
   pl.shape.smem = pl.shapes[0].smem;
-  pl.shape.clusters = pl.shapes[0].clusters;
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
   // one workspace per cluster of either shape, then the products of split items
+  cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
   int most = pl.shapes[0].clusters;
   if (pl.shapes[1].clusters > most) most = pl.shapes[1].clusters;
+  pl.shape.clusters = pl.shapes[0].clusters;
   pl.part_off = size_t(most) * pl.shape.slot;
   pl.part_slots = kPartsPerCluster * most;
   pl.scratch_bytes = (pl.part_off + size_t(pl.part_slots) * G::HN3) * sizeof(C<T>);
@@ -1103,6 +1120,8 @@ int vss_configure_impl(Plan& pl) {
   pl.shape.smem = pl.shapes[0].smem;
   pl.shape.clusters = pl.shapes[0].clusters;
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
+  cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
+  pl.shape.clusters = pl.shapes[0].clusters;
   pl.scratch_bytes = size_t(pl.shapes[0].clusters) * pl.shape.slot * sizeof(C<T>);
   return DGFS_OK;
 }

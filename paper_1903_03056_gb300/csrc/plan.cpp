@@ -437,8 +437,8 @@ int build_plan(const dgfs_plan_desc* d, Plan& p) {
       tk.ent_off = int(p.ent_w.size());
       tk.n_ent = int(ent.size());
       tk.grp_off = int(p.groups.size());
-      // groups share sigma_x (VHS); with VSS every entry needs its own forward transform and
-      // is its own group
+      // groups share sigma_x (VHS); with VSS every entry needs its own forward transform and is its
+      // own group here (upload_plan pairs neighbours of equal sigma_x)
       int first = 0;
       for (int e = 1; e <= int(ent.size()); ++e) {
         if (e == int(ent.size()) || p.vss ||

@@ -46,3 +46,19 @@ def test_a_split_evaluation_replays_from_a_graph():
         torch.cuda.synchronize()
         assert torch.equal(Q, ref)
     plan.close()
+
+
+def test_plans_of_one_shape_with_different_sphere_rules_stay_usable():
+    """Two plans share a kernel and differ in its shared memory (phase blocks of 32 and 6 directions):
+    creating and running the smaller one leaves the larger one usable."""
+    import torch
+    w = synth.Workload("split", 2, 16, 5.0, (1.0, 2.1), 0.7, 1.0, 6, 3, "bimaxwellian", 0.05, 92)
+    f = torch.from_numpy(synth.batch_distribution(w)).to(device="cuda", dtype=torch.float32)
+    large = dgfs.Plan(16, 5.0, [1.0, 2.1], 0.7, M=32, N_rho=3, precision="fp32")
+    ref = large.eval(f)
+    small = dgfs.Plan(16, 5.0, [1.0, 2.1], 0.7, M=6, N_rho=3, precision="fp32")
+    small.eval(f)
+    assert torch.equal(large.eval(f), ref)
+    torch.cuda.synchronize()
+    large.close()
+    small.close()
