@@ -497,7 +497,8 @@ def gpu_arm(args):
 
     f64 = synth.batch_distribution(w, nodes=rank_nodes(rank, B))  # [B, s, N, N, N]
     stream = torch.cuda.Stream()
-    flops_node = transforms_per_node(w) * flops_per_transform(w.N)
+    # every transform of the method has real data on one side: half the flops of a complex one
+    flops_node = 0.5 * transforms_per_node(w) * flops_per_transform(w.N)
 
     with torch.cuda.stream(stream):
         f32 = torch.from_numpy(f64.astype(np.float32)).cuda()

@@ -47,7 +47,7 @@
 // Measured on the GB300 against the complex-transform kernel this one replaced: 4096 nodes of N = 32
 // FP32 285 -> 145 ms, 3001 of N = 24 75.1 -> 36.6, 8192 of N = 16 28.7 -> 16.3, 61 three-species nodes
 // of N = 48 86.0 -> 35.8, 61 nodes of N = 32 FP64 201 -> 82, VSS 37 three-species nodes of N = 48
-// (M = 32) 339 -> 161 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
+// (M = 32) 339 -> 163 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
 // FMA pipes run half their cycles (N = 16: the L1 data path three quarters), the stalls are L2 loads
 // of the x-passed spectra, whose workspaces together exceed L2 from N = 24 on.
 #pragma once
