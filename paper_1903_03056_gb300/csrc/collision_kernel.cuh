@@ -47,7 +47,7 @@
 // Measured on the GB300 against the complex-transform kernel this one replaced: 4096 nodes of N = 32
 // FP32 285 -> 145 ms, 3001 of N = 24 75.1 -> 36.6, 8192 of N = 16 28.7 -> 16.3, 61 three-species nodes
 // of N = 48 86.0 -> 35.8, 61 nodes of N = 32 FP64 201 -> 82, VSS 37 three-species nodes of N = 48
-// (M = 32) 339 -> 163 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
+// (M = 32) 339 -> 147 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
 // FMA pipes run half their cycles (N = 16: the L1 data path three quarters), the stalls are L2 loads
 // of the x-passed spectra, whose workspaces together exceed L2 from N = 24 on.
 #pragma once
@@ -153,11 +153,12 @@ struct VGeo {
   static constexpr bool SPLIT = CL > 1 && (sizeof(T) == 8 || N >= 48) && !VSS;
   static constexpr int NBH = SPLIT ? 3 : 2;
   // VSS: complex product spectra [x][k_y][k_z] of up to two entries a group, double buffered, and
-  // accumulators per k_x: pencils [k_y][0..N/2], then (k_y = N/2, k_z = N/2+1..N-1)
+  // accumulators (total and current part of the radial nodes) per k_x: pencils [k_y][0..N/2], then
+  // (k_y = N/2, k_z = N/2+1..N-1)
   static constexpr size_t PVN = VSS ? 4 * N3 : HN3;
   static constexpr int QROW = VSS ? N * (h + 1) + h - 1 : HN2;
   static constexpr size_t QN = VSS ? (size_t(N) * QROW + 1) / 2 * 2 : HN3;
-  static constexpr size_t SLOT = VSS ? (2 + 2) * N3 + PVN + 2 * QN : (2 + 3) * N3 + 4 * HN3;
+  static constexpr size_t SLOT = VSS ? (2 + 2) * N3 + PVN + 4 * QN : (2 + 3) * N3 + 4 * HN3;
   static constexpr size_t FACE = 2 * N2 + N;
 };
 
@@ -319,14 +320,13 @@ __device__ __forceinline__ void tm_store(uint32_t ta, const float* v) {
 // and weights only its element k_x = N/2 apart (two alternating sums over x).  The pencils with k_y or
 // k_z = N/2 keep Q_hat itself, partner included, until the finish.
 template <typename T, int N, int W>
-__device__ __forceinline__ void vss_step_c(const KernelParams& p, const TaskDesc& tk, int q, int e, const C<T>* PV,
-                                           C<T>* QA, C<T>* QB, int plane0, int tid) {
+__device__ __forceinline__ void vss_step_c(const KernelParams& p, const TaskDesc& tk, int q, int e, bool first,
+                                           const C<T>* PV, C<T>* QA, C<T>* QB, int plane0, int tid) {
   using G = VGeo<T, N, W>;
   using CT = C<T>;
   constexpr int h = G::h, N2 = G::N2, QS = G::QROW, HP = h + 1;
   const int c0 = p.ent_m[2 * (tk.ent_off + e)], c1 = p.ent_m[2 * (tk.ent_off + e) + 1];
   const bool self_sum = tk.i == tk.j && c1 >= 0;
-  const bool first = q == 0 && e == 0;
   const int own = G::PLANES * HP;
   const int all = own + (plane0 <= h && h < plane0 + G::PLANES ? h - 1 : 0);
   for (int u = tid; u < all; u += G::THREADS) {
@@ -388,6 +388,27 @@ __device__ __forceinline__ void vss_step_c(const KernelParams& p, const TaskDesc
           st2<T>(acc + n * QS, val);
         }
       }
+    }
+  }
+}
+
+// VSS: total += part (or its copy), both accumulators, this CTA's pencils.  A radial sum is the sum, in
+// order, of the sums of at most kVssParts parts of the radial nodes, whether one cluster runs them all or
+// several run some each: a node's bits do not depend on how its item was split.  (Out of line, so that its
+// pointers and loads cost the inner loops no registers.)
+template <typename T, int N, int W>
+__device__ __noinline__ void vss_add_part(C<T>* total, const C<T>* part, bool copy, bool both, int plane0, int tid) {
+  using G = VGeo<T, N, W>;
+  constexpr int HP = G::h + 1, own = G::PLANES * HP;
+  const int all = own + (plane0 <= G::h && G::h < plane0 + G::PLANES ? G::h - 1 : 0);
+  for (int o = 0; o < (both ? 2 : 1); ++o) {
+#pragma unroll 4
+    for (int v0 = tid; v0 < N * all; v0 += G::THREADS) {
+      const int n = v0 / all, u = v0 % all;
+      const size_t at = size_t(o) * G::QN + n * G::QROW + (u < own ? plane0 * HP + u : N * HP + u - own);
+      C<T> v = ld2<T>(part + at);
+      if (!copy) v = add<T>(ld2<T>(total + at), v);
+      st2<T>(total + at, v);
     }
   }
 }
@@ -525,9 +546,15 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
     const int whole = item / p.chunks;
     const int b = whole % p.batch;
     const int task = whole / p.batch;
-    const bool split = !G::VSS && p.chunks > 1;
-    const int q0 = chunk * p.n_rho / p.chunks, q1 = (chunk + 1) * p.n_rho / p.chunks;
-    CT* const PT = static_cast<CT*>(p.parts) + size_t(whole) * p.n_rho * HN3;  // P_hat of every radial node
+    const bool split = p.chunks > 1;
+    // VSS: the chunk is a range of the plan's parts of the radial nodes
+    const int n_part = G::VSS ? vss_parts(p.n_rho) : p.chunks;
+    int part = G::VSS ? chunk * n_part / p.chunks : chunk;
+    const int part_end = G::VSS ? (chunk + 1) * n_part / p.chunks : chunk + 1;
+    const int q0 = part * p.n_rho / n_part, q1 = part_end * p.n_rho / n_part;
+    int part_q0 = q0;
+    // split items: P_hat of every radial node; VSS: both accumulators of every part
+    CT* const PT = static_cast<CT*>(p.parts) + (G::VSS ? size_t(whole) * n_part * 2 * G::QN : size_t(whole) * p.n_rho * HN3);
     const TaskDesc tk = p.tasks[task];
     const T* fb = reinterpret_cast<const T*>(p.f) + size_t(b) * p.s * N3;
     const bool self = tk.i == tk.j;
@@ -580,6 +607,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
 
     // ---- gain ---------------------------------------------------------------------------------
     T P[G::PSM || G::VSS ? 1 : N];
+    auto part_acc = [&]() { return split ? PT + size_t(part) * 2 * G::QN : QB + G::QN; };
     for (int q = q0; q < q1; ++q) {
       const CT* const phq = static_cast<const CT*>(p.phase) + (size_t(task) * p.n_rho + q) * p.max_ent * PB;
       if (ph_smem) {
@@ -827,12 +855,20 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
           if (k >= 2) {
             const GroupDesc gd = p.groups[tk.grp_off + k - 2];
             for (int j = 0; j < gd.count; ++j)
-              vss_step_c<T, N, W>(p, tk, q, gd.first + j, PV + size_t(2 * (k & 1) + j) * N3, QA, QB, plane0, tid);
+              vss_step_c<T, N, W>(p, tk, q, gd.first + j, q == part_q0 && gd.first + j == 0,
+                                  PV + size_t(2 * (k & 1) + j) * N3, part_acc(), part_acc() + G::QN, plane0, tid);
           }
         }
         if (halves) cluster_wait(); else cluster_sync<CL>();
       }
-      if constexpr (G::VSS) continue;
+      if constexpr (G::VSS) {
+        if (q + 1 == (part + 1) * p.n_rho / n_part) {  // the part's last
+          if (!split) vss_add_part<T, N, W>(QA, part_acc(), part == 0, tk.out1 >= 0, plane0, tid);
+          ++part;
+          part_q0 = q + 1;
+        }
+        continue;
+      }
 
       // step C: x pass of the product spectrum, weights, accumulation
       for (int u = tid; u < G::PLANES * h; u += NT) {
@@ -890,12 +926,15 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
         continue;
       }
       __threadfence();
-      if constexpr (G::CALL)
+      if constexpr (G::VSS) {
+        for (int j = 0; j < n_part; ++j)
+          vss_add_part<T, N, W>(QA, PT + size_t(j) * 2 * G::QN, j == 0, tk.out1 >= 0, plane0, tid);
+      } else if constexpr (G::CALL)
         add_parts_call<T, N, W>(PT, static_cast<const T*>(p.Fw), QA, QB, tk.out0, tk.out1, p.n_rho, plane0, tid);
       else
         add_parts<T, N, W>(PT, static_cast<const T*>(p.Fw), QA, QB, tk.out0, tk.out1, p.n_rho, plane0, tid);
     }
-    __syncthreads();
+    if constexpr (G::VSS) cluster_sync<CL>(); else __syncthreads();
 
     // ---- finish: Q_ij = IDFT(Q_hat) - f_i IDFT(G^- f_hat_j); role 0 the gain, role 1 the loss ----
     for (int o = 0; o < 2; ++o) {
@@ -1135,7 +1174,9 @@ int vss_configure_impl(Plan& pl) {
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
   cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
   pl.shape.clusters = pl.shapes[0].clusters;
-  pl.scratch_bytes = size_t(pl.shapes[0].clusters) * pl.shape.slot * sizeof(C<T>);
+  pl.part_off = size_t(pl.shapes[0].clusters) * pl.shape.slot;
+  pl.part_slots = kVssPartsPerCluster * pl.shapes[0].clusters;
+  pl.scratch_bytes = (pl.part_off + size_t(pl.part_slots) * 2 * G::QN) * sizeof(C<T>);
   return DGFS_OK;
 }
 
@@ -1211,11 +1252,40 @@ inline KernelParams kernel_params(const Plan& pl, const void* f, void* Q, int ba
   return kp;
 }
 
+// VSS: chunks of whole parts, in units of one radial node of the dearest task.  A chunk's f_hat costs
+// little beside its entries' three transforms each, so finer chunks cost only the sums of the parts; they fill
+// the chip with few items.  One three-species node of N = 48, 24 radial nodes, M = 32: 31.3 -> 6.6 ms with
+// 8 parts (4: 10.2).  Adding up the parts costs items that run whole 0.8 % (256 nodes 986 -> 994 ms).
+inline int vss_chunks(int items, int n_rho, int clusters, double mean_cost, int part_slots) {
+  const int parts = vss_parts(n_rho);
+  if (double(items) * parts > double(part_slots)) return 1;
+  int best = 1;
+  double best_t = 1e300;
+  for (int s = 1; s <= parts; s *= 2) {
+    const double one = 0.1 + double((parts + s - 1) / s) * n_rho / parts;
+    const double share = double(items) * s * mean_cost * one / clusters + 0.4 * one;
+    const double t = share > one ? share : one;
+    if (t < best_t * (1.0 - 1e-9)) {
+      best_t = t;
+      best = s;
+    }
+  }
+  return best;
+}
+
 template <typename T, int N>
 int vss_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
   KernelParams kp = kernel_params(pl, f, Q, batch, ws);
-  const int n = int(pl.shapes[0].clusters * pl.shape.share);
-  return launch_shape<T, N, 2>(pl, kp, batch * kp.n_tasks, n < 1 ? 1 : n, st);
+  kp.parts = static_cast<C<T>*>(pl.scratch_of(ws)) + pl.part_off;
+  const int n = int(pl.shapes[0].clusters * pl.shape.share), limit = n < 1 ? 1 : n;
+  double cost = 0.0, most = 0.0;
+  for (const TaskDesc& t : pl.tasks) {
+    cost += t.n_ent;
+    most = t.n_ent > most ? t.n_ent : most;
+  }
+  const int items = batch * kp.n_tasks;
+  kp.chunks = vss_chunks(items, pl.N_rho, limit, cost / (kp.n_tasks * most), pl.part_slots);
+  return launch_shape<T, N, 2>(pl, kp, items * kp.chunks, limit, st);
 }
 
 template <typename T, int N>

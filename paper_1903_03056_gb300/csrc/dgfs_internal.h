@@ -101,6 +101,10 @@ struct LaunchShape {
 constexpr int kExitWord = 2, kDoneWord = 64;
 // products (one radial node of one item) the VHS workspace holds per resident cluster
 constexpr int kPartsPerCluster = 6;
+// VSS: the radial sum is made of this many parts (fewer radial nodes: one each), and the split items' buffer
+// holds the accumulators of this many per cluster (three items' worth)
+constexpr int kVssParts = 8, kVssPartsPerCluster = 24;
+constexpr __host__ __device__ int vss_parts(int n_rho) { return n_rho < kVssParts ? n_rho : kVssParts; }
 
 // one launch shape of the collision kernel
 struct KernelShape {

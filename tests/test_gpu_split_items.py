@@ -62,3 +62,30 @@ def test_plans_of_one_shape_with_different_sphere_rules_stay_usable():
     torch.cuda.synchronize()
     large.close()
     small.close()
+
+
+@pytest.mark.parametrize("N,N_rho,s,M,few,many,precision", [
+    (8, 10, 2, 6, 3, 1500, "fp32"),   # parts of one and two radial nodes
+    (8, 3, 2, 12, 2, 3000, "fp64"),    # fewer radial nodes than parts
+    (12, 9, 2, 6, 40, 1200, "fp32"),  # groups that share a barrier
+    (16, 8, 3, 32, 1, 400, "fp32"),   # clusters of two, three species
+    (24, 17, 2, 12, 2, 700, "fp32"),
+    (6, 1, 1, 6, 1, 5, "fp32"),       # one radial node: never split
+])
+def test_vss_nodes_do_not_depend_on_the_split(N, N_rho, s, M, few, many, precision):
+    """A VSS node's bits are the same alone, where its items split over the parts of the radial sum,
+    and in a batch whose items run whole."""
+    import torch
+    masses = [1.0, 2.1, 0.6][:s]
+    w = synth.Workload("vss_split", few, N, 5.0, tuple(masses), 0.7, 1.4, M, N_rho, "bimaxwellian", 0.05, 17)
+    dt = torch.float64 if precision == "fp64" else torch.float32
+    f = torch.from_numpy(synth.batch_distribution(w)).to(device="cuda", dtype=dt)
+    plan = dgfs.Plan(N, 5.0, masses, 0.7, alpha=1.4, M=M, N_rho=N_rho, precision=precision)
+    ref = plan.eval(f)
+    batch = f.repeat((many + few - 1) // few, 1, 1, 1, 1)[:many].contiguous()
+    Q = plan.eval(batch)
+    torch.cuda.synchronize()
+    for b in range(many):
+        assert torch.equal(Q[b], ref[b % few])
+    assert torch.equal(plan.eval(f), ref)
+    plan.close()
