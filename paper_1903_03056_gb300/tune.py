@@ -138,6 +138,13 @@ def _patch(text, T, N, line):
     return pat.sub(line, text)
 
 
+def other_objects(tu):
+    """The current build's objects that a variant of translation unit `tu` links: one per source of the
+    library (objects of sources that were renamed or removed may still lie beside them)."""
+    names = (os.path.splitext(f)[0] for f in build.SOURCES)
+    return [os.path.join(build.BUILD, n + ".o") for n in names if n != tu]
+
+
 def _variant(tmp, precision, N, shape, radix=None):
     """Build a variant tree under tmp; returns its root (with the package inside).  With
     `radix` the shape stays and the radix schedule of (precision, N) becomes `radix`."""
@@ -170,10 +177,8 @@ def _variant(tmp, precision, N, shape, radix=None):
     res = subprocess.run(cmd, capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(res.stderr[-2000:])
-    others = [os.path.join(build.BUILD, f) for f in os.listdir(build.BUILD)
-              if f.endswith(".o") and f != tu + ".o"]
-    res = subprocess.run([build.nvcc()] + build.ARCH + ["-shared", "-o", os.path.join(pkg, "libdgfs.so"), obj] + others,
-                         capture_output=True, text=True)
+    res = subprocess.run([build.nvcc()] + build.ARCH + ["-shared", "-o", os.path.join(pkg, "libdgfs.so"), obj]
+                         + other_objects(tu) + ["-ldl"], capture_output=True, text=True)
     if res.returncode != 0:
         raise RuntimeError(res.stderr[-2000:])
     os.utime(os.path.join(pkg, "libdgfs.so"))

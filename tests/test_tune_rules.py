@@ -1,0 +1,14 @@
+"""The tuner's rules on the CPU: which objects a variant links."""
+
+import os
+
+from paper_1903_03056_gb300 import build, tune
+
+
+def test_a_variant_links_the_librarys_own_objects_only(tmp_path, monkeypatch):
+    monkeypatch.setattr(build, "BUILD", str(tmp_path))
+    names = [os.path.splitext(f)[0] for f in build.SOURCES]
+    for n in names + ["left_over"]:  # the object of a source that is no longer there
+        (tmp_path / (n + ".o")).write_bytes(b"")
+    linked = [os.path.splitext(os.path.basename(f))[0] for f in tune.other_objects("collision_f32")]
+    assert sorted(linked) == sorted(n for n in names if n != "collision_f32")
