@@ -16,8 +16,8 @@ With --radix it times, per N, every order of the radices 8, 4, 2, 3 in the candi
 (tuned_radix.h codes) of the FP32 kernel instead; a line of N runs as transforms of N / 2 points, so
 the schedule of N / 2 is the one that is tried.  A schedule changes the rounding of a line,
 so its output is checked against the FP64 path on the first nodes of the workload (the largest
-per-node max |Q - Q_fp64| / max |Q_fp64| must stay below the FP32 bar, 1e-5); the fastest
-schedule that passes is kept.  (FP64 schedules stay at the default order: an FP64 variant has
+per-node max |Q - Q_fp64| / max |Q_fp64| must stay below the FP32 bar, 1e-5); of the schedules that
+pass and run within 1 % of the fastest, the one of smallest error is kept.  (FP64 schedules stay at the default order: an FP64 variant has
 no more accurate path to be checked against on the device.)
 """
 
@@ -63,6 +63,7 @@ RADIX_CANDIDATES = {
 }
 RADIX_BAR = 1e-5
 RADIX_CHECK_NODES = 4
+RADIX_TIE = 1.01  # times that count as equal
 
 
 def radix_code_valid(N, code):
@@ -143,6 +144,12 @@ def other_objects(tu):
     library (objects of sources that were renamed or removed may still lie beside them)."""
     names = (os.path.splitext(f)[0] for f in build.SOURCES)
     return [os.path.join(build.BUILD, n + ".o") for n in names if n != tu]
+
+
+def best_radix(rows):
+    """The row with the smallest error among those within RADIX_TIE of the fastest's time."""
+    fastest = min(r["ms"] for r in rows)
+    return min((r for r in rows if r["ms"] <= RADIX_TIE * fastest), key=lambda r: (r["err_vs_fp64"], r["ms"]))
 
 
 def _variant(tmp, precision, N, shape, radix=None):
@@ -253,8 +260,9 @@ def current_radix(precision, N):
 
 
 def tune_radix(precision="fp32", sizes=(16, 24, 32, 48), write=False, jobs=8):
-    """Time every candidate radix schedule of each N at the current launch shape; keep the fastest
-    whose output stays within RADIX_BAR of the FP64 path."""
+    """Time every candidate radix schedule of each N at the current launch shape; among those whose output
+    stays within RADIX_BAR of the FP64 path and whose time is within 1 % of the fastest's, keep the one of
+    smallest error."""
     if precision != "fp32":
         raise ValueError("radix schedules are tuned for the FP32 kernel")
     build.build()
@@ -285,7 +293,7 @@ def tune_radix(precision="fp32", sizes=(16, 24, 32, 48), write=False, jobs=8):
             good = [r for r in rows if r["ok"]]
             if not good:
                 continue
-            best = min(good, key=lambda r: r["ms"])
+            best = best_radix(good)
             record["radix/%s/%d" % (precision, N)] = {"workload": workload, "batch": batch, "previous": cur,
                                                      "shape": list(current_shape(precision, N)), "best": best,
                                                      "candidates": rows}

@@ -1,4 +1,4 @@
-"""The tuner's rules on the CPU: which objects a variant links."""
+"""The tuner's rules on the CPU: which objects a variant links and which radix schedule it keeps."""
 
 import os
 
@@ -12,3 +12,10 @@ def test_a_variant_links_the_librarys_own_objects_only(tmp_path, monkeypatch):
         (tmp_path / (n + ".o")).write_bytes(b"")
     linked = [os.path.splitext(os.path.basename(f))[0] for f in tune.other_objects("collision_f32")]
     assert sorted(linked) == sorted(n for n in names if n != "collision_f32")
+
+
+def test_equal_times_are_decided_by_the_error():
+    rows = [{"radix": 28, "ms": 145.5, "err_vs_fp64": 1.32e-6}, {"radix": 44, "ms": 146.0, "err_vs_fp64": 1.21e-6},
+            {"radix": 422, "ms": 147.5, "err_vs_fp64": 1.0e-6}]
+    assert tune.best_radix(rows)["radix"] == 44
+    assert tune.best_radix(rows[::2])["radix"] == 28
