@@ -56,6 +56,7 @@
 
 #include <cuda_runtime.h>
 
+#include "dd_line.cuh"
 #include "dgfs_internal.h"
 #include "group_sync.cuh"
 #include "real_line.cuh"
@@ -134,6 +135,16 @@ struct VGeo {
   static constexpr bool TMR = TMOK && fits(SETS * (2 * N + (TMP ? P_COLS : 0)));
   static constexpr int TM_SET = (TMR ? 2 * N : 0) + (TMP ? P_COLS : 0);  // columns of a thread
   static constexpr int TM_ALLOC = TM_SET > 0 ? alloc_of(SETS * TM_SET) : 0;
+  // FP32: passes of the finish whose sums carry their rounding errors along (dd_line.cuh).  Gain and loss
+  // are larger than their difference, so the rounding of these last transforms is in every result; real
+  // transforms alone round more than the complex ones they replaced (a complex transform of real data leaves
+  // half its error in the part that is dropped): 2-norm error 1.04 to 1.19 times theirs, N = 48 0.84 to 0.96.
+  // These are the fewest passes that bring it below theirs (N = 6 to 32: 0.78 to 0.98).  Measured: 4096 nodes
+  // of N = 32 145.2 -> 149.9 ms, 3001 of N = 24 36.6 -> 37.5, 8192 of N = 16 16.3 -> 16.7, one N = 16
+  // relaxation step 144 -> 155 us; in FP64 the same passes took 3 to 5 times that.
+  static constexpr bool FINE_Z = sizeof(T) == 4 && (N <= 16 || N == 32 || (N == 24 && !VSS));
+  static constexpr bool FINE_Y = FINE_Z && N != 24;
+  static constexpr bool FINE_X = FINE_Y && N <= 8 && !VSS;
   static constexpr bool CALL = sizeof(T) == 4 && W == 0 && (N == 24 || N == 32);  // add_parts
   static constexpr int QU = W == 1 || N <= 12 ? 8 : CALL || sizeof(T) == 8 ? 4 : 2;
   // shared memory per group: one padded plane, the entry's row of the k_y face, P if PSM
@@ -254,6 +265,24 @@ __device__ __forceinline__ void rows_c2r(const double2* row, const double2* phz,
     for (int k = 1; k < h; ++k) x[k] = cmul<double>(row[h + k], phz[h + k]);
   }
   c2r_line<double, N>(x, x0.y, xh.y, y.b);
+}
+
+// the last z pass of a row (gain in row, loss in row + N/2): out[z] = gain - f loss
+template <int N>
+__device__ __forceinline__ void dd_finish_row(const float2* row, const float* f, float (&out)[N]) {
+  constexpr int h = N / 2;
+  CDD<F2> x[h];
+  DD<F2> y[N];
+#pragma unroll
+  for (int k = 1; k < h; ++k) x[k] = dd_of(pack2(row[k].x, row[h + k].x), pack2(row[k].y, row[h + k].y));
+  const float2 g0 = row[0], l0 = row[h];
+  c2r_line<DD<F2>, N>(x, dd_of(pack2(g0.x, l0.x)), dd_of(pack2(g0.y, l0.y)), y);
+#pragma unroll
+  for (int z = 0; z < N; ++z) {
+    const float2 hi = unpack2(y[z].hi), lo = unpack2(y[z].lo);
+    const float fz = __ldg(f + z);
+    out[z] = fmaf(-fz, hi.y, hi.x) + fmaf(-fz, lo.y, lo.x);
+  }
 }
 
 __device__ __forceinline__ float fma_(float a, float b, float c) { return fmaf(a, b, c); }
@@ -983,7 +1012,7 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
             v[n] = mk<T>(gp * a.x + gm * m.x, gp * a.y - gm * m.y);
           }
         }
-        line_fft<T, N, +1>(v);
+        if constexpr (G::FINE_X) dd_line_fft<N, +1>(v); else line_fft<T, N, +1>(v);
 #pragma unroll
         for (int n = 0; n < N; ++n) st2<T>(H0 + n * N2 + r * N + t, v[n]);
       }
@@ -1009,22 +1038,31 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
               v[N - r] = mk<T>(al.x + be.y, be.x - al.y);
             }
           }
-          line_fft<T, N, +1>(v);
+          if constexpr (G::FINE_Y) dd_line_fft<N, +1>(v); else line_fft<T, N, +1>(v);
           group_sync<N, GP>();
 #pragma unroll
           for (int r = 0; r < N; ++r) tb[r * PITCH + t] = v[r];
           group_sync<N, GP>();
         }
-        const CT g0 = tb[t * PITCH], l0 = tb[t * PITCH + h];
-        Rows<T, N> y;
-        rows_c2r<N>(tb + t * PITCH, static_cast<const CT*>(nullptr), mk<T>(g0.x, l0.x), mk<T>(g0.y, l0.y), y);
-        group_sync<N, GP>();
         // stage the row through shared memory for a coalesced store
         T* const rb = reinterpret_cast<T*>(tb);
+        const T* const fr = fi + size_t(x) * N2 + t * N;
+        if constexpr (G::FINE_Z) {
+          T y[N];
+          dd_finish_row<N>(tb + t * PITCH, fr, y);
+          group_sync<N, GP>();
 #pragma unroll
-        for (int z = 0; z < N; ++z) {
-          const CT gl = y.at(z);
-          rb[t * PITCH + z] = gl.x - __ldg(fi + size_t(x) * N2 + t * N + z) * gl.y;
+          for (int z = 0; z < N; ++z) rb[t * PITCH + z] = y[z];
+        } else {
+          const CT g0 = tb[t * PITCH], l0 = tb[t * PITCH + h];
+          Rows<T, N> y;
+          rows_c2r<N>(tb + t * PITCH, static_cast<const CT*>(nullptr), mk<T>(g0.x, l0.x), mk<T>(g0.y, l0.y), y);
+          group_sync<N, GP>();
+#pragma unroll
+          for (int z = 0; z < N; ++z) {
+            const CT gl = y.at(z);
+            rb[t * PITCH + z] = gl.x - __ldg(fr + z) * gl.y;
+          }
         }
         group_sync<N, GP>();
 #pragma unroll
