@@ -57,8 +57,8 @@ def flops_per_transform(N):
 
 # the sources that define the collision kernel's code and launch shape
 COLLISION_KERNEL_SOURCES = ("collision_kernel.cuh", "real_line.cuh", "dd_line.cuh", "simd2.cuh", "group_sync.cuh", "fft_line.cuh",
-                            "tcgen05.cuh", "collision_f32.cu", "collision_f64.cu", "dgfs_internal.h", "tuned_shapes.h",
-                            "tuned_radix.h")
+                            "tcgen05.cuh", "collision_f32.cu", "collision_f64.cu", "dgfs_internal.h", "launch_plan.h",
+                            "tuned_shapes.h", "tuned_radix.h")
 
 
 def kernel_sources_sha1():

@@ -59,6 +59,7 @@
 #include "dd_line.cuh"
 #include "dgfs_internal.h"
 #include "group_sync.cuh"
+#include "launch_plan.h"
 #include "real_line.cuh"
 #include "tcgen05.cuh"
 
@@ -1218,42 +1219,6 @@ int vss_configure_impl(Plan& pl) {
   return DGFS_OK;
 }
 
-// How a launch of `items` work items (task, node) runs: the shape W and the number of chunks each
-// item's radial nodes are split into, by a cost model in units of one radial node of the dearest
-// task on a full device.  A chunk of `len` nodes costs len + 1/2 (its own f_hat).  Chunks go out one
-// by one, so a launch takes its share of the device, sum of costs / clusters, and about 0.38 of the
-// last chunk; a chunk on a nearly idle device runs at 0.6 of its cost.  Fitted to N = 24, 45 nodes
-// (W = 0: 1.42, 1.21, 1.11, 0.98, 1.10 ms with 1, 2, 4, 6, 12 chunks) and N = 32, 5 nodes, 3 species
-// (W = 0: 2.30, 1.22, 0.99, 1.11 ms with 1, 4, 8, 16; W = 1: 0.97, 0.74, 0.75, 0.84 with 1, 2, 4, 16).
-// The wide shape takes `slow` times longer per node and cluster-share of the device.  All products
-// of all items must fit the parts buffer.
-struct LaunchPlan {
-  int wide = 0, chunks = 1;
-};
-inline LaunchPlan plan_launch(int items, int n_rho, int clusters0, int clusters1, double slow, double mean_cost,
-                           int part_slots) {
-  LaunchPlan best;
-  double best_t = 1e300;
-  for (int w = 0; w < 2; ++w) {
-    const int C = w == 0 ? clusters0 : clusters1;
-    if (C <= 0) continue;
-    const double unit = w == 0 ? 1.0 : slow * double(clusters1) / double(clusters0);
-    for (int s = 1; s <= n_rho; ++s) {
-      if (s > 1 && double(items) * n_rho > double(part_slots)) break;
-      const int len = (n_rho + s - 1) / s;
-      if (s > 1 && (n_rho + s - 2) / (s - 1) == len) continue;  // no shorter than with s - 1 chunks
-      const double one = 0.5 + len, share = double(items) * s * mean_cost * one / C + 0.38 * one;
-      const double t = (share > 0.6 * one ? share : 0.6 * one) * unit;
-      if (t < best_t * (1.0 - 1e-9)) {
-        best_t = t;
-        best.wide = w;
-        best.chunks = s;
-      }
-    }
-  }
-  return best;
-}
-
 template <typename T, int N, int W>
 int launch_shape(const Plan& pl, KernelParams& kp, int items, int limit, cudaStream_t st) {
   using G = VGeo<T, N, W>;
@@ -1290,39 +1255,13 @@ inline KernelParams kernel_params(const Plan& pl, const void* f, void* Q, int ba
   return kp;
 }
 
-// VSS: chunks of whole parts, in units of one radial node of the dearest task.  A chunk's f_hat costs
-// little beside its entries' three transforms each, so finer chunks cost only the sums of the parts; they fill
-// the chip with few items.  One three-species node of N = 48, 24 radial nodes, M = 32: 31.3 -> 6.6 ms with
-// 8 parts (4: 10.2).  Adding up the parts costs items that run whole 0.8 % (256 nodes 986 -> 994 ms).
-inline int vss_chunks(int items, int n_rho, int clusters, double mean_cost, int part_slots) {
-  const int parts = vss_parts(n_rho);
-  if (double(items) * parts > double(part_slots)) return 1;
-  int best = 1;
-  double best_t = 1e300;
-  for (int s = 1; s <= parts; s *= 2) {
-    const double one = 0.1 + double((parts + s - 1) / s) * n_rho / parts;
-    const double share = double(items) * s * mean_cost * one / clusters + 0.4 * one;
-    const double t = share > one ? share : one;
-    if (t < best_t * (1.0 - 1e-9)) {
-      best_t = t;
-      best = s;
-    }
-  }
-  return best;
-}
-
 template <typename T, int N>
 int vss_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStream_t st, int ws) {
   KernelParams kp = kernel_params(pl, f, Q, batch, ws);
   kp.parts = static_cast<C<T>*>(pl.scratch_of(ws)) + pl.part_off;
   const int n = int(pl.shapes[0].clusters * pl.shape.share), limit = n < 1 ? 1 : n;
-  double cost = 0.0, most = 0.0;
-  for (const TaskDesc& t : pl.tasks) {
-    cost += t.n_ent;
-    most = t.n_ent > most ? t.n_ent : most;
-  }
   const int items = batch * kp.n_tasks;
-  kp.chunks = vss_chunks(items, pl.N_rho, limit, cost / (kp.n_tasks * most), pl.part_slots);
+  kp.chunks = vss_chunks(items, pl.N_rho, limit, task_load(pl), pl.part_slots);
   return launch_shape<T, N, 2>(pl, kp, items * kp.chunks, limit, st);
 }
 
@@ -1336,12 +1275,7 @@ int vhs_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStrea
   };
   const int items = batch * kp.n_tasks;
   const int c0 = share_of(pl.shapes[0].clusters), c1 = pl.shapes[1].clusters > 0 ? share_of(pl.shapes[1].clusters) : 0;
-  double cost = 0.0, most = 0.0;
-  for (const TaskDesc& t : pl.tasks) {
-    cost += t.n_ent;
-    most = t.n_ent > most ? t.n_ent : most;
-  }
-  const LaunchPlan run = plan_launch(items, pl.N_rho, c0, c1, HasWide<T, N>::slow, cost / (kp.n_tasks * most), pl.part_slots);
+  const LaunchPlan run = plan_launch(items, pl.N_rho, c0, c1, HasWide<T, N>::slow, task_load(pl), pl.part_slots);
   kp.chunks = run.chunks;
   if constexpr (HasWide<T, N>::value) {
     if (run.wide) return launch_shape<T, N, 1>(pl, kp, items * run.chunks, c1, st);
