@@ -140,11 +140,11 @@ struct VGeo {
   // are larger than their difference, so the rounding of these last transforms is in every result; real
   // transforms alone round more than the complex ones they replaced (a complex transform of real data leaves
   // half its error in the part that is dropped): 2-norm error 1.04 to 1.19 times theirs, N = 48 0.84 to 0.96.
-  // These are the fewest passes that bring it below theirs (N = 6 to 32: 0.78 to 0.98).  Measured: 4096 nodes
-  // of N = 32 145.2 -> 149.9 ms, 3001 of N = 24 36.6 -> 37.5, 8192 of N = 16 16.3 -> 16.7, one N = 16
-  // relaxation step 144 -> 155 us; in FP64 the same passes took 3 to 5 times that.
+  // These are the fewest passes that bring it below theirs (N = 6 to 32: 0.78 to 0.99; VSS needs y at N = 6
+  // alone).  Measured: 4096 nodes of N = 32 145.2 -> 149.9 ms, 3001 of N = 24 36.6 -> 37.5, 8192 of N = 16
+  // 16.3 -> 16.7, one N = 16 relaxation step 144 -> 155 us; in FP64 the same passes took 3 to 5 times that.
   static constexpr bool FINE_Z = sizeof(T) == 4 && (N <= 16 || N == 32 || (N == 24 && !VSS));
-  static constexpr bool FINE_Y = FINE_Z && N != 24;
+  static constexpr bool FINE_Y = FINE_Z && (VSS ? N == 6 : N != 24);
   static constexpr bool FINE_X = FINE_Y && N <= 8 && !VSS;
   static constexpr bool CALL = sizeof(T) == 4 && W == 0 && (N == 24 || N == 32);  // add_parts
   static constexpr int QU = W == 1 || N <= 12 ? 8 : CALL || sizeof(T) == 8 ? 4 : 2;
