@@ -52,6 +52,7 @@
 // of the x-passed spectra, whose workspaces together exceed L2 from N = 24 on.
 #pragma once
 
+#include <algorithm>
 #include <cmath>
 
 #include <cuda_runtime.h>
@@ -1192,12 +1193,9 @@ int vhs_configure_impl(Plan& pl) {
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
   // one workspace per cluster of either shape, then the products of split items
   cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
-  int most = pl.shapes[0].clusters;
-  if (pl.shapes[1].clusters > most) most = pl.shapes[1].clusters;
-  pl.shape.clusters = pl.shapes[0].clusters;
-  pl.part_off = size_t(most) * pl.shape.slot;
-  pl.part_slots = kPartsPerCluster * most;
-  pl.scratch_bytes = (pl.part_off + size_t(pl.part_slots) * G::HN3) * sizeof(C<T>);
+  pl.part_slots = kPartsPerCluster * std::max(pl.shapes[0].clusters, pl.shapes[1].clusters);
+  pl.part_size = G::HN3;
+  size_workspace(pl);
   return DGFS_OK;
 }
 
@@ -1209,13 +1207,11 @@ int vss_configure_impl(Plan& pl) {
   pl.shape.groups = G::GP;
   pl.shape.threads = G::THREADS;
   pl.shape.smem = pl.shapes[0].smem;
-  pl.shape.clusters = pl.shapes[0].clusters;
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
   cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
-  pl.shape.clusters = pl.shapes[0].clusters;
-  pl.part_off = size_t(pl.shapes[0].clusters) * pl.shape.slot;
   pl.part_slots = kVssPartsPerCluster * pl.shapes[0].clusters;
-  pl.scratch_bytes = (pl.part_off + size_t(pl.part_slots) * 2 * G::QN) * sizeof(C<T>);
+  pl.part_size = 2 * G::QN;
+  size_workspace(pl);
   return DGFS_OK;
 }
 

@@ -176,6 +176,7 @@ struct Plan {
   KernelShape shapes[2];           // the batch shape and (VHS) the wide one (clusters = 0: none)
   size_t part_off = 0;             // VHS plans: the split items' products in the workspace (complex values)
   int part_slots = 0;              // and how many there is room for
+  size_t part_size = 0;            // complex values of one
   size_t counter_bytes() const { return (kDoneWord + size_t(part_slots)) * sizeof(unsigned); }
   void* d_scratch = nullptr;       // kGuardBytes into d_scratch_raw
   void* d_scratch_raw = nullptr;   // guard | workspace | guard
@@ -223,6 +224,12 @@ void gauss_legendre_rule(int n, double* x, double* w);
 int build_plan(const dgfs_plan_desc* d, Plan& p);
 int upload_plan(Plan& p);
 void free_plan(Plan& p);
+// bytes of the workspace from the clusters of the launch shapes and the room for split items
+void size_workspace(Plan& p);
+// Allocate the workspace and its counters with `alloc`.  Where the memory does not suffice the room for
+// split items goes first (small batches then run their items whole, with the same results), then
+// clusters do, down to one: a plan is refused only when the smallest workspace does not fit.
+int alloc_workspace(Plan& p, int (*alloc)(Plan& p, void** dptr, size_t bytes));
 
 // kernel configuration and launch, per precision (collision_f32.cu / collision_f64.cu)
 int configure_vss_f32(Plan& p);

@@ -508,6 +508,28 @@ static int upload(Plan& p, const V* host, size_t count, void** dptr, size_t& tot
   return DGFS_OK;
 }
 
+void size_workspace(Plan& p) {
+  const int most = std::max(p.shapes[0].clusters, p.shapes[1].clusters);
+  p.shape.clusters = p.shapes[0].clusters;
+  p.part_off = size_t(most) * p.shape.slot;
+  p.scratch_bytes = (p.part_off + size_t(p.part_slots) * p.part_size) * 2 * real_size(p);
+}
+
+int alloc_workspace(Plan& p, int (*alloc)(Plan& p, void** dptr, size_t bytes)) {
+  for (;;) {
+    int rc = alloc(p, &p.d_scratch_raw, p.scratch_bytes + 2 * Plan::kGuardBytes);
+    if (rc == DGFS_OK) rc = alloc(p, (void**)&p.d_counter, p.counter_bytes());
+    const bool least = p.part_slots == 0 && p.shapes[0].clusters <= 1 && p.shapes[1].clusters <= 1;
+    // (the tensor-core path sizes its own)
+    if (rc != DGFS_ERR_OOM || p.d_scratch_raw || p.shape.slot == 0 || least) return rc;
+    if (p.part_slots > 0)
+      p.part_slots = 0;
+    else
+      for (KernelShape& s : p.shapes) s.clusters = (s.clusters + 1) / 2;
+    size_workspace(p);
+  }
+}
+
 // Device memory of the plan is stream-ordered on the plan's own stream (cudaMallocAsync /
 // cudaFreeAsync), so creating and destroying plans never synchronises other streams; the
 // function returns after the plan's stream has finished the uploads and table builds.
@@ -796,7 +818,7 @@ int upload_plan(Plan& p) {
   }
   // the workspace between two guard blocks of a fixed byte pattern: dgfs_plan_check reads
   // them back to detect a kernel write outside the workspace
-  if ((rc = dalloc(p, &p.d_scratch_raw, p.scratch_bytes + 2 * Plan::kGuardBytes))) return rc;
+  if ((rc = alloc_workspace(p, dalloc))) return rc;
   p.d_scratch = static_cast<char*>(p.d_scratch_raw) + Plan::kGuardBytes;
   if (cudaMemsetAsync(p.d_scratch_raw, Plan::kGuardByte, Plan::kGuardBytes, p.home) != cudaSuccess ||
       cudaMemsetAsync(static_cast<char*>(p.d_scratch) + p.scratch_bytes, Plan::kGuardByte, Plan::kGuardBytes,
@@ -804,7 +826,6 @@ int upload_plan(Plan& p) {
     cudaGetLastError();
     return DGFS_ERR_CUDA;
   }
-  if ((rc = dalloc(p, (void**)&p.d_counter, p.counter_bytes()))) return rc;
   // the counters and the device status word start at zero
   if (cudaMemsetAsync(p.d_counter, 0, p.counter_bytes(), p.home) != cudaSuccess) {
     cudaGetLastError();

@@ -1,0 +1,61 @@
+"""The collision workspace under short memory, with an allocator that refuses what passes a limit (CPU): a plan is refused only when the smallest workspace does not fit."""
+
+import json
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_1903_03056_gb300 import build, dgfs
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA_INC = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include")
+GUARDS = 2 * 4096
+# the VSS workspace of three species at N = 48 (M = 32): 76 clusters, 24 parts each
+VSS48 = dict(N=48, s=3, precision=1, flags=0, max_batch=0, c0=76, c1=0, slot=1200000, slots=1824, size=117456)
+
+
+@pytest.fixture(scope="module")
+def probe(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if cxx is None or not os.path.isdir(CUDA_INC):
+        pytest.skip("needs g++ and the CUDA headers")
+    libdir = os.path.dirname(build.build())
+    exe = str(tmp_path_factory.mktemp("probe") / "workspace_probe")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I", os.path.join(ROOT, "include"), "-I", build.CSRC, "-I", CUDA_INC,
+                    os.path.join(ROOT, "tests", "workspace_probe.cpp"), "-o", exe, "-L", libdir, "-ldgfs",
+                    "-Wl,-rpath," + libdir], check=True)
+
+    def run(limit=1 << 60, batch=0, **kw):
+        words = list(kw.values()) + [limit, batch]
+        return json.loads(subprocess.run([exe], input=" ".join(map(str, words)), capture_output=True, text=True,
+                                         check=True).stdout)
+
+    return run
+
+
+def test_enough_memory_keeps_the_whole_workspace(probe):
+    r = probe(**VSS48)
+    assert r["rc"] == 0 and r["scratch"] == r["wanted"] == (76 * 1200000 + 1824 * 117456) * 8
+    assert r["clusters"] == [76, 0] and r["part_slots"] == 1824
+
+
+@pytest.mark.parametrize("limit,clusters,slots", [
+    (2_300_000_000, 76, 0),   # no room for split items
+    (400_000_000, 38, 0),     # half the clusters
+    (10_000_000, 1, 0),       # one
+])
+def test_short_memory_shrinks_the_workspace(probe, limit, clusters, slots):
+    r = probe(limit=limit, **VSS48)
+    assert r["rc"] == 0 and r["clusters"] == [clusters, 0] and r["part_slots"] == slots
+    assert r["scratch"] == clusters * 1200000 * 8 and r["used"] == r["scratch"] + GUARDS + r["counters"] <= limit
+
+
+def test_two_shapes_share_the_smaller_workspace(probe):
+    r = probe(limit=200 << 20, N=32, s=2, precision=1, flags=0, max_batch=0, c0=228, c1=57, slot=254000, slots=1368, size=16384)
+    assert r["rc"] == 0 and r["clusters"] == [57, 15] and r["part_off"] == 57 * 254000
+
+
+def test_less_than_one_cluster_is_refused(probe):
+    assert probe(limit=9_000_000, **VSS48)["rc"] == dgfs.DGFS_ERR_OOM

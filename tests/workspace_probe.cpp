@@ -1,0 +1,38 @@
+// Host-side probe of the workspace's allocation (test infrastructure, no GPU needed): a plan whose launch
+// shapes are given, an allocator that refuses what passes a limit, and the sizes that result.
+//
+// stdin: N s precision flags max_batch clusters0 clusters1 slot part_slots part_size limit batch
+#include <cstdio>
+
+#include "dgfs_internal.h"
+
+namespace {
+size_t limit_bytes = 0, used = 0;
+char memory[1];
+int refuse_above_limit(dgfs::Plan&, void** p, size_t bytes) {
+  if (used + bytes > limit_bytes) {
+    *p = nullptr;
+    return DGFS_ERR_OOM;
+  }
+  used += bytes;
+  *p = memory;
+  return DGFS_OK;
+}
+}  // namespace
+
+int main() {
+  dgfs::Plan p;
+  int batch;
+  if (std::scanf("%d %d %d %u %d %d %d %zu %d %zu %zu %d", &p.N, &p.s, &p.precision, &p.flags, &p.max_batch,
+                 &p.shapes[0].clusters, &p.shapes[1].clusters, &p.shape.slot, &p.part_slots, &p.part_size, &limit_bytes,
+                 &batch) != 12)
+    return 2;
+  dgfs::size_workspace(p);
+  const size_t wanted = p.scratch_bytes;
+  const int rc = dgfs::alloc_workspace(p, refuse_above_limit);
+  std::printf("{\"rc\": %d, \"wanted\": %zu, \"scratch\": %zu, \"used\": %zu, \"clusters\": [%d, %d], \"part_slots\": %d, "
+              "\"part_off\": %zu, \"counters\": %zu}\n",
+              rc, wanted, p.scratch_bytes, used, p.shapes[0].clusters, p.shapes[1].clusters, p.part_slots, p.part_off,
+              p.counter_bytes());
+  return 0;
+}
