@@ -290,14 +290,8 @@ int dgfs_plan_set_sm_share(dgfs_plan plan, double share) {
 
 int dgfs_plan_bytes(dgfs_plan plan, int batch, size_t* tables, size_t* workspace) {
   if (!plan || batch < 0) return DGFS_ERR_INVALID_ARG;
-  const dgfs::Plan& p = plan->plan;
-  const size_t n3 = size_t(p.N) * p.N * p.N;
-  if (tables) *tables = p.table_bytes;
-  if (workspace)
-    *workspace = p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes + (p.d_Qfull ? size_t(p.max_batch) * p.s * p.s * n3 * dgfs::real_size(p) : 0) +
-                 (batch > 0 ? size_t(batch) * (p.s + output_pairs(p)) * n3 * dgfs::real_size(p) +
-                                  p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes + p.counter_bytes()
-                            : 0);
+  if (tables) *tables = plan->plan.table_bytes;
+  if (workspace) *workspace = dgfs::workspace_bytes(plan->plan, batch);
   return DGFS_OK;
 }
 

@@ -230,6 +230,8 @@ void size_workspace(Plan& p);
 // split items goes first (small batches then run their items whole, with the same results), then
 // clusters do, down to one: a plan is refused only when the smallest workspace does not fit.
 int alloc_workspace(Plan& p, int (*alloc)(Plan& p, void** dptr, size_t bytes));
+// device bytes of the workspace, and of what a host-buffer call of `batch` nodes adds to it
+size_t workspace_bytes(const Plan& p, int batch);
 
 // kernel configuration and launch, per precision (collision_f32.cu / collision_f64.cu)
 int configure_vss_f32(Plan& p);

@@ -530,6 +530,16 @@ int alloc_workspace(Plan& p, int (*alloc)(Plan& p, void** dptr, size_t bytes)) {
   }
 }
 
+size_t workspace_bytes(const Plan& p, int batch) {
+  const size_t node = size_t(p.N) * p.N * p.N * real_size(p), ss = size_t(p.s) * p.s;
+  const size_t one = p.scratch_bytes + 2 * Plan::kGuardBytes + p.counter_bytes();
+  size_t bytes = one;
+  if (p.d_Qfull) bytes += size_t(p.max_batch) * ss * node;
+  if (p.d_lam) bytes += size_t(p.max_batch) * p.cons.size() * 6 * sizeof(double);
+  if (batch > 0) bytes += one + size_t(batch) * (p.s + ((p.flags & DGFS_SUM_SPECIES) ? size_t(p.s) : ss)) * node;
+  return bytes;
+}
+
 // Device memory of the plan is stream-ordered on the plan's own stream (cudaMallocAsync /
 // cudaFreeAsync), so creating and destroying plans never synchronises other streams; the
 // function returns after the plan's stream has finished the uploads and table builds.

@@ -1,4 +1,5 @@
-"""The collision workspace under short memory, with an allocator that refuses what passes a limit (CPU): a plan is refused only when the smallest workspace does not fit."""
+"""The collision workspace under short memory and the bytes a plan reports, with an allocator that refuses
+what passes a limit (CPU): a plan is refused only when the smallest workspace does not fit."""
 
 import json
 import os
@@ -59,3 +60,17 @@ def test_two_shapes_share_the_smaller_workspace(probe):
 
 def test_less_than_one_cluster_is_refused(probe):
     assert probe(limit=9_000_000, **VSS48)["rc"] == dgfs.DGFS_ERR_OOM
+
+
+@pytest.mark.parametrize("batch", [0, 700])
+def test_reported_bytes_hold_every_array_of_the_workspace(probe, batch):
+    """Workspace, guards and counters, the staged operators and the projection's multipliers; for a host-buffer
+    call the second workspace and its counters, inputs and outputs."""
+    flags = dgfs.DGFS_CONSERVE | dgfs.DGFS_SUM_SPECIES
+    r = probe(batch=batch, N=24, s=2, precision=1, flags=flags, max_batch=1000, c0=304, c1=90, slot=100000, slots=1824, size=6912)
+    n3 = 24 ** 3 * 4
+    one = r["scratch"] + GUARDS + (64 + 1824) * 4
+    want = one + 1000 * 4 * n3 + 1000 * 3 * 6 * 8
+    if batch:
+        want += one + batch * (2 + 2) * n3
+    assert r["reported"] == want

@@ -30,9 +30,13 @@ int main() {
   dgfs::size_workspace(p);
   const size_t wanted = p.scratch_bytes;
   const int rc = dgfs::alloc_workspace(p, refuse_above_limit);
+  if ((p.flags & DGFS_SUM_SPECIES) && (p.flags & DGFS_CONSERVE)) {
+    p.cons.resize(size_t(p.s) * (p.s + 1) / 2);
+    p.d_Qfull = p.d_lam = reinterpret_cast<double*>(memory);
+  }
   std::printf("{\"rc\": %d, \"wanted\": %zu, \"scratch\": %zu, \"used\": %zu, \"clusters\": [%d, %d], \"part_slots\": %d, "
-              "\"part_off\": %zu, \"counters\": %zu}\n",
+              "\"part_off\": %zu, \"counters\": %zu, \"reported\": %zu}\n",
               rc, wanted, p.scratch_bytes, used, p.shapes[0].clusters, p.shapes[1].clusters, p.part_slots, p.part_off,
-              p.counter_bytes());
+              p.counter_bytes(), dgfs::workspace_bytes(p, batch));
   return 0;
 }
