@@ -147,7 +147,8 @@ int dgfs_eval_collision(dgfs_plan plan, const void* f_dev, void* Q_dev, int batc
  * workspace of its own, so one chunk's kernel starts while the previous one ends.  The call
  * is ordered after the work already on `stream` and after the plan's previous evaluation.
  * batch <= max_batch, else DGFS_ERR_BUDGET.  The plan's staging buffers and second workspace
- * are allocated at the first call. */
+ * are allocated at the first call; where the second workspace does not fit, the chunks run one
+ * after another on the first. */
 int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, int batch,
                              void* stream);
 

@@ -164,26 +164,29 @@ int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, i
     p.stage_batch = p.max_batch;
   }
   if (!p.d_scratch2_raw) {
-    // the second workspace (with its guard blocks) and work counter of the pipelined chunks
-    if (cudaMallocAsync(&p.d_scratch2_raw, p.scratch_bytes + 2 * dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
-        cudaMallocAsync((void**)&p.d_counter2, p.counter_bytes(), p.home) != cudaSuccess) {
+    // the second workspace (with its guard blocks) and work counter of the pipelined chunks; where it
+    // does not fit, the chunks run one after another on the first
+    const size_t bytes = p.scratch_bytes_of(1), counters = p.counter_bytes(1);
+    if (cudaMallocAsync(&p.d_scratch2_raw, bytes + 2 * dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
+        cudaMallocAsync((void**)&p.d_counter2, counters, p.home) != cudaSuccess) {
       cudaGetLastError();
       if (p.d_scratch2_raw) cudaFreeAsync(p.d_scratch2_raw, p.home);
-      if (p.d_counter2) cudaFreeAsync(p.d_counter2, p.home);
       cudaStreamSynchronize(p.home);
       p.d_scratch2_raw = nullptr;
       p.d_counter2 = nullptr;
-      return DGFS_ERR_OOM;
-    }
-    p.d_scratch2 = static_cast<char*>(p.d_scratch2_raw) + dgfs::Plan::kGuardBytes;
-    if (cudaMemsetAsync(p.d_scratch2_raw, dgfs::Plan::kGuardByte, dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
-        cudaMemsetAsync(static_cast<char*>(p.d_scratch2) + p.scratch_bytes, dgfs::Plan::kGuardByte,
-                        dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
-        cudaMemsetAsync(p.d_counter2, 0, p.counter_bytes(), p.home) != cudaSuccess || cudaStreamSynchronize(p.home) != cudaSuccess) {
-      cudaGetLastError();
-      return DGFS_ERR_CUDA;
+    } else {
+      p.d_scratch2 = static_cast<char*>(p.d_scratch2_raw) + dgfs::Plan::kGuardBytes;
+      if (cudaMemsetAsync(p.d_scratch2_raw, dgfs::Plan::kGuardByte, dgfs::Plan::kGuardBytes, p.home) != cudaSuccess ||
+          cudaMemsetAsync(static_cast<char*>(p.d_scratch2) + bytes, dgfs::Plan::kGuardByte, dgfs::Plan::kGuardBytes,
+                          p.home) != cudaSuccess ||
+          cudaMemsetAsync(p.d_counter2, 0, counters, p.home) != cudaSuccess ||
+          cudaStreamSynchronize(p.home) != cudaSuccess) {
+        cudaGetLastError();
+        return DGFS_ERR_CUDA;
+      }
     }
   }
+  const int n_ws = p.d_scratch2_raw ? 2 : 1;
   if (!p.h2d) {
     bool ok = cudaStreamCreateWithFlags(&p.h2d, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&p.d2h, cudaStreamNonBlocking) == cudaSuccess &&
@@ -220,7 +223,7 @@ int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, i
     const int b0 = k * chunk;
     const int nb = batch - b0 < chunk ? batch - b0 : chunk;
     if (nb <= 0) break;
-    cudaStream_t es = evs[k & 1];
+    cudaStream_t es = evs[k % n_ws];
     char* sf = static_cast<char*>(p.d_stage_f) + size_t(b0) * f_node;
     char* sq = static_cast<char*>(p.d_stage_Q) + size_t(b0) * q_node;
     if (cudaMemcpyAsync(sf, static_cast<const char*>(f_host) + size_t(b0) * f_node, size_t(nb) * f_node,
@@ -229,7 +232,7 @@ int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, i
       return DGFS_ERR_CUDA;
     {
       dgfs::NvtxRange range("dgfs collision");
-      const int rc = launch_core(p, sf, sq, nb, es, k & 1, b0, &launches);
+      const int rc = launch_core(p, sf, sq, nb, es, k % n_ws, b0, &launches);
       if (rc != DGFS_OK) return rc;
     }
     if (cudaEventRecord(p.ev_done[k], es) != cudaSuccess || cudaStreamWaitEvent(p.d2h, p.ev_done[k], 0) != cudaSuccess ||
@@ -324,7 +327,7 @@ int dgfs_plan_check(dgfs_plan plan, int* intact) {
     const char* body = static_cast<const char*>(p.scratch_of(ws));
     unsigned st = 0;
     if (cudaMemcpyAsync(host, raw, G, cudaMemcpyDeviceToHost, p.home) != cudaSuccess ||
-        cudaMemcpyAsync(host + G, body + p.scratch_bytes, G, cudaMemcpyDeviceToHost, p.home) != cudaSuccess ||
+        cudaMemcpyAsync(host + G, body + p.scratch_bytes_of(ws), G, cudaMemcpyDeviceToHost, p.home) != cudaSuccess ||
         cudaMemcpyAsync(&st, p.counter_of(ws) + 1, sizeof(unsigned), cudaMemcpyDeviceToHost, p.home) != cudaSuccess ||
         cudaStreamSynchronize(p.home) != cudaSuccess) {
       cudaGetLastError();

@@ -1257,7 +1257,7 @@ int vss_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStrea
   kp.parts = static_cast<C<T>*>(pl.scratch_of(ws)) + pl.part_off;
   const int n = int(pl.shapes[0].clusters * pl.shape.share), limit = n < 1 ? 1 : n;
   const int items = batch * kp.n_tasks;
-  kp.chunks = vss_chunks(items, pl.N_rho, limit, task_load(pl), pl.part_slots);
+  kp.chunks = vss_chunks(items, pl.N_rho, limit, task_load(pl), pl.part_slots_of(ws));
   return launch_shape<T, N, 2>(pl, kp, items * kp.chunks, limit, st);
 }
 
@@ -1271,7 +1271,8 @@ int vhs_launch_impl(const Plan& pl, const void* f, void* Q, int batch, cudaStrea
   };
   const int items = batch * kp.n_tasks;
   const int c0 = share_of(pl.shapes[0].clusters), c1 = pl.shapes[1].clusters > 0 ? share_of(pl.shapes[1].clusters) : 0;
-  const LaunchPlan run = plan_launch(items, pl.N_rho, c0, c1, HasWide<T, N>::slow, task_load(pl), pl.part_slots);
+  const LaunchPlan run = plan_launch(items, pl.N_rho, c0, c1, HasWide<T, N>::slow, task_load(pl),
+                                     pl.part_slots_of(ws));
   kp.chunks = run.chunks;
   if constexpr (HasWide<T, N>::value) {
     if (run.wide) return launch_shape<T, N, 1>(pl, kp, items * run.chunks, c1, st);

@@ -460,7 +460,7 @@ int configure_gemm_impl(Plan& p) {
   p.shape.smem = G::SMEM;
   p.shape.phase_smem = 0;
   p.shape.clusters = sms * per_sm;
-  p.scratch_bytes = size_t(p.shape.clusters) * 6 * G::N3 * sizeof(float2);
+  p.scratch_bytes = p.scratch2_bytes = size_t(p.shape.clusters) * 6 * G::N3 * sizeof(float2);
   return DGFS_OK;
 }
 

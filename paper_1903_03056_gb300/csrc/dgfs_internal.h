@@ -177,7 +177,8 @@ struct Plan {
   size_t part_off = 0;             // VHS plans: the split items' products in the workspace (complex values)
   int part_slots = 0;              // and how many there is room for
   size_t part_size = 0;            // complex values of one
-  size_t counter_bytes() const { return (kDoneWord + size_t(part_slots)) * sizeof(unsigned); }
+  int part_slots_of(int ws) const { return ws == 0 ? part_slots : part_slots2; }
+  size_t counter_bytes(int ws = 0) const { return (kDoneWord + size_t(part_slots_of(ws))) * sizeof(unsigned); }
   void* d_scratch = nullptr;       // kGuardBytes into d_scratch_raw
   void* d_scratch_raw = nullptr;   // guard | workspace | guard
   static constexpr size_t kGuardBytes = 4096;
@@ -195,6 +196,10 @@ struct Plan {
   void* scratch_of(int ws) const { return ws == 0 ? d_scratch : d_scratch2; }
   unsigned* counter_of(int ws) const { return ws == 0 ? d_counter : d_counter2; }
   size_t scratch_bytes = 0;
+  int part_slots2 = 0;              // the second one's room for split items: the same, or none where no
+                                    // chunk of a pipelined batch is small enough to split
+  size_t scratch2_bytes = 0;
+  size_t scratch_bytes_of(int ws) const { return ws == 0 ? scratch_bytes : scratch2_bytes; }
   void* d_rk = nullptr;             // SSP-RK2 workspace: f1 and the right-hand side
   void* d_stage_f = nullptr;
   void* d_stage_Q = nullptr;
@@ -224,7 +229,10 @@ void gauss_legendre_rule(int n, double* x, double* w);
 int build_plan(const dgfs_plan_desc* d, Plan& p);
 int upload_plan(Plan& p);
 void free_plan(Plan& p);
-// bytes of the workspace from the clusters of the launch shapes and the room for split items
+// the fewest nodes of a pipelined host batch's chunk: at most 8 chunks of 256 nodes or more, rounded up,
+// leave the last one 7 short
+constexpr int kPipelinedNodes = 249;
+// bytes of both workspaces from the clusters of the launch shapes and the room for split items
 void size_workspace(Plan& p);
 // Allocate the workspace and its counters with `alloc`.  Where the memory does not suffice the room for
 // split items goes first (small batches then run their items whole, with the same results), then

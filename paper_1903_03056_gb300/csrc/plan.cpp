@@ -512,7 +512,10 @@ void size_workspace(Plan& p) {
   const int most = std::max(p.shapes[0].clusters, p.shapes[1].clusters);
   p.shape.clusters = p.shapes[0].clusters;
   p.part_off = size_t(most) * p.shape.slot;
-  p.scratch_bytes = (p.part_off + size_t(p.part_slots) * p.part_size) * 2 * real_size(p);
+  if (p.shape.slot > 0) p.scratch_bytes = (p.part_off + size_t(p.part_slots) * p.part_size) * 2 * real_size(p);
+  const int pieces = p.vss ? vss_parts(p.N_rho) : p.N_rho;
+  p.part_slots2 = double(kPipelinedNodes) * p.tasks.size() * pieces > p.part_slots ? 0 : p.part_slots;
+  p.scratch2_bytes = p.scratch_bytes - size_t(p.part_slots - p.part_slots2) * p.part_size * 2 * real_size(p);
 }
 
 int alloc_workspace(Plan& p, int (*alloc)(Plan& p, void** dptr, size_t bytes)) {
@@ -532,11 +535,11 @@ int alloc_workspace(Plan& p, int (*alloc)(Plan& p, void** dptr, size_t bytes)) {
 
 size_t workspace_bytes(const Plan& p, int batch) {
   const size_t node = size_t(p.N) * p.N * p.N * real_size(p), ss = size_t(p.s) * p.s;
-  const size_t one = p.scratch_bytes + 2 * Plan::kGuardBytes + p.counter_bytes();
-  size_t bytes = one;
+  auto one = [&p](int ws) { return p.scratch_bytes_of(ws) + 2 * Plan::kGuardBytes + p.counter_bytes(ws); };
+  size_t bytes = one(0);
   if (p.d_Qfull) bytes += size_t(p.max_batch) * ss * node;
   if (p.d_lam) bytes += size_t(p.max_batch) * p.cons.size() * 6 * sizeof(double);
-  if (batch > 0) bytes += one + size_t(batch) * (p.s + ((p.flags & DGFS_SUM_SPECIES) ? size_t(p.s) : ss)) * node;
+  if (batch > 0) bytes += one(1) + size_t(batch) * (p.s + ((p.flags & DGFS_SUM_SPECIES) ? size_t(p.s) : ss)) * node;
   return bytes;
 }
 
