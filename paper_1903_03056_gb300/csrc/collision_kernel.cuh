@@ -1186,10 +1186,6 @@ int vhs_configure_impl(Plan& pl) {
   if constexpr (HasWide<T, N>::value) {
     if (int rc = configure_shape<T, N, 1>(pl)) return rc;
   }
-  pl.shape.cluster = G::CL;
-  pl.shape.groups = G::GP;
-  pl.shape.threads = G::THREADS;
-  pl.shape.smem = pl.shapes[0].smem;
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
   // one workspace per cluster of either shape, then the products of split items
   cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
@@ -1203,10 +1199,6 @@ template <typename T, int N>
 int vss_configure_impl(Plan& pl) {
   using G = VGeo<T, N, 2>;
   if (int rc = configure_shape<T, N, 2>(pl)) return rc;
-  pl.shape.cluster = G::CL;
-  pl.shape.groups = G::GP;
-  pl.shape.threads = G::THREADS;
-  pl.shape.smem = pl.shapes[0].smem;
   pl.shape.slot = G::SLOT + size_t(pl.max_ent) * G::FACE;
   cap_clusters(pl, pl.shape.slot * sizeof(C<T>));
   pl.part_slots = kVssPartsPerCluster * pl.shapes[0].clusters;

@@ -454,11 +454,6 @@ int configure_gemm_impl(Plan& p) {
   }
   // the CTAs of one SM share its 512 tensor-memory columns
   if (per_sm > 512 / G::TMEM_COLS) per_sm = 512 / G::TMEM_COLS;
-  p.shape.cluster = 1;
-  p.shape.groups = G::TILES;
-  p.shape.threads = G::THREADS;
-  p.shape.smem = G::SMEM;
-  p.shape.phase_smem = 0;
   p.shape.clusters = sms * per_sm;
   p.scratch_bytes = p.scratch2_bytes = size_t(p.shape.clusters) * 6 * G::N3 * sizeof(float2);
   return DGFS_OK;

@@ -39,7 +39,7 @@ struct TaskDesc {
   int ent_off, n_ent;  // entries (sigma, weight) of this task
   int grp_off, n_grp;  // groups of entries sharing sigma_x
   int any_zero;        // some group has sigma_x = 0
-  int face_off, n_face;  // faces of the VHS kernel: entries with a shift along x or y
+  int face_off, n_face;  // its faces: entries with a shift along x or y
 };
 
 struct GroupDesc {
@@ -86,20 +86,17 @@ struct ConsBlock {
 };
 
 struct LaunchShape {
-  int cluster = 1;        // CTAs cooperating on one work item
-  int groups = 1;         // plane groups per CTA
-  int threads = 0;        // groups * N
-  size_t smem = 0;        // dynamic shared memory per CTA
-  int phase_smem = 0;     // phases staged in shared memory
   int clusters = 0;       // resident clusters (persistent grid)
-  size_t slot = 0;        // complex values of workspace per cluster (VHS kernel)
+  size_t slot = 0;        // complex values of workspace per cluster (0: the tensor-core path)
   double share = 1.0;     // fraction of the resident clusters one launch may use
 };
 
-// words of the counter array: 0 the work counter, 1 the device status, then (VHS kernel) the
+// words of the counter array: 0 the work counter, 1 the device status, then the
 // clusters that have left and, from kDoneWord on, the finished chunks of every split item
 constexpr int kExitWord = 2, kDoneWord = 64;
-// products (one radial node of one item) the VHS workspace holds per resident cluster
+// VHS: products (one radial node of one item) the workspace holds per resident cluster.  Splitting pays while
+// a launch has fewer items than clusters, or about that many of few radial nodes; 6 cover N_rho = 12 up to half an
+// item a cluster
 constexpr int kPartsPerCluster = 6;
 // VSS: the radial sum is made of this many parts (fewer radial nodes: one each), and the split items' buffer
 // holds the accumulators of this many per cluster (three items' worth)
@@ -145,7 +142,8 @@ struct Plan {
   double vss_a_max = 0;         // largest argument pi rho c_j |k| / L of that table
   bool vss_grid = false;        // the table was built from the grid of Phi_alpha(p, q)
   bool antipodal = false;       // every direction has an antipode of equal weight
-  std::vector<int> ent_ysh;     // [entries] shares the previous entry's y pass
+  std::vector<int> ent_ysh;     // [entries] repeats the previous entry's sigma_x and sigma_y (VHS; no kernel
+                                // reads it, the host tests of the entry lists do)
   int max_ent = 0;
   bool vss = false;             // some alpha_ij != 1
 
@@ -174,7 +172,7 @@ struct Plan {
   // workspace
   LaunchShape shape;
   KernelShape shapes[2];           // the batch shape and (VHS) the wide one (clusters = 0: none)
-  size_t part_off = 0;             // VHS plans: the split items' products in the workspace (complex values)
+  size_t part_off = 0;             // where the split items' products (VHS) or parts (VSS) start in the workspace (complex values)
   int part_slots = 0;              // and how many there is room for
   size_t part_size = 0;            // complex values of one
   int part_slots_of(int ws) const { return ws == 0 ? part_slots : part_slots2; }

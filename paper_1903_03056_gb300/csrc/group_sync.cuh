@@ -54,13 +54,6 @@ __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// Order this thread's generic-proxy accesses to global memory before later async-proxy (bulk
-// copy) accesses: the workspace planes are written with ordinary stores and read back by bulk
-// copies after a barrier.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
-
 // Barrier of one plane group.  A group of N threads that divides a warp lives inside one warp
 // and synchronises only that warp.  Otherwise SG = lcm(N, 32) / N consecutive groups form a
 // warp-aligned super-group that synchronises on its own named barrier (ids 1, 2, ...), so
