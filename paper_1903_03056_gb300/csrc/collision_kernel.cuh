@@ -792,18 +792,18 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
                 // the product is complex; forward z and y transforms, all N columns
                 CT pr[N];
 #pragma unroll
-              for (int z = 0; z < N; z += 2) {
-                CT uz[2];
-                load_two(uyb + z, uz[0], uz[1]);
+                for (int z = 0; z < N; z += 2) {
+                  CT uz[2];
+                  load_two(uyb + z, uz[0], uz[1]);
 #pragma unroll
-                for (int d = 0; d < 2; ++d) {
-                  // read by every plane of the CTA: through L1
-                  const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
-                  const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
-                  const CT re = y.at(z + d);
-                  pr[z + d] = mk<T>(fma_(-im.x, im.y, re.x * re.y), fma_(re.x, im.y, im.x * re.y));
+                  for (int d = 0; d < 2; ++d) {
+                    // read by every plane of the CTA: through L1
+                    const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
+                    const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
+                    const CT re = y.at(z + d);
+                    pr[z + d] = mk<T>(fma_(-im.x, im.y, re.x * re.y), fma_(re.x, im.y, im.x * re.y));
+                  }
                 }
-              }
                 line_fft<T, N, -1>(pr);
                 group_sync<N, GP>();
 #pragma unroll
@@ -817,19 +817,19 @@ __global__ void __launch_bounds__(VGeo<T, N, W>::THREADS, VGeo<T, N, W>::MINB) c
                 for (int r = 0; r < N; ++r) st2<T>(dst + r * N, pr[r]);
               } else {
 #pragma unroll
-              for (int z = 0; z < N; z += 2) {
-                CT uz[2];
-                load_two(uyb + z, uz[0], uz[1]);
+                for (int z = 0; z < N; z += 2) {
+                  CT uz[2];
+                  load_two(uyb + z, uz[0], uz[1]);
 #pragma unroll
-                for (int d = 0; d < 2; ++d) {
-                  // read by every plane of the CTA: through L1
-                  const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
-                  const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
-                  const CT re = y.at(z + d);
-                  if constexpr (G::PSM) pb[(z + d) * N + t] = fma_(-im.x, im.y, fma_(re.x, re.y, pb[(z + d) * N + t]));
-                  else P[z + d] = fma_(-im.x, im.y, fma_(re.x, re.y, P[z + d]));
+                  for (int d = 0; d < 2; ++d) {
+                    // read by every plane of the CTA: through L1
+                    const CT ux = has_x ? __ldca(fc + (z + d) * N + t) : mk<T>(0, 0);
+                    const CT im = face_sum(sgx, ux, sgy, uz[d], d ? mk<T>(-m.x, -m.y) : m);
+                    const CT re = y.at(z + d);
+                    if constexpr (G::PSM) pb[(z + d) * N + t] = fma_(-im.x, im.y, fma_(re.x, re.y, pb[(z + d) * N + t]));
+                    else P[z + d] = fma_(-im.x, im.y, fma_(re.x, re.y, P[z + d]));
+                  }
                 }
-              }
               }
             }
             if constexpr (G::VSS) {

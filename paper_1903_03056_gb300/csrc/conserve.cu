@@ -7,8 +7,8 @@
 //
 // conserve_kernel: one cluster of CTAs per (node, block).  The moment sums are FP64 and bound by
 // the FP64 pipe (two multiply-adds a cycle and SM), so each thread keeps one pair of v_z nodes and
-// walks over the (x, y) rows: three FP64 additions or multiply-adds per value instead of nine, no
-// index arithmetic per value, and the cluster spreads a block over up to 8 SMs.  The CTAs read each
+// walks over the (x, y) rows: eight FP64 operations and one integer division per pair of values instead
+// of nine operations and two 64-bit divisions per value, and the cluster spreads a block over up to 8 SMs.  The CTAs read each
 // other's partial sums through distributed shared memory, in rank order, so the result does not
 // depend on the batch.  Then each CTA subtracts C^T lambda from its rows (APPLY), or rank 0 stores
 // lambda for the species sum.  Measured (GB300): one N = 16 node 79 us -> 7 us, 45 nodes of N = 24

@@ -1,7 +1,6 @@
 // Radix schedule of the register line transform per (precision, N): the decimal digits of the
-// code, first stage first (442 = radix 4, 4, then 2).  Written by
-// paper_1903_03056_gb300/tune.py --radix from timings on the device (record:
-// tuned_shapes.json, keys "radix/..."); edit by re-running the tuner.
+// code, first stage first (442 = radix 4, 4, then 2).  paper_1903_03056_gb300/tune.py --radix times the
+// orders on the device and writes these lines.
 // FP32 lines of N points run as transforms of N / 2, so the FP32 entry of N / 2 serves grid size N.
 // Where the orders' times agree within 1 %, the one with the smallest error against 64 bits is kept:
 // 16 takes 44 (N = 32: 1.32e-6 -> 1.21e-6 of ||Q|| on 8 two-species nodes, 28 measured 145.5 ms against
