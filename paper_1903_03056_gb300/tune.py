@@ -214,14 +214,14 @@ def tune(precision="fp32", sizes=(16, 24, 32, 48), write=False, jobs=8):
     with open(SHAPES_H) as fh:
         header = fh.read()
     with tempfile.TemporaryDirectory(prefix="dgfs_tune_") as tmp:
-        todo = [(N, sh) for N in sizes for sh in CANDIDATES.get(N, []) if valid(N, *sh, csize)]
+        todo = [(N, sh) for N in sizes for sh in shape_candidates(precision, N) if valid(N, *sh, csize)]
         with ThreadPoolExecutor(max_workers=jobs) as ex:
             roots = dict(zip(todo, ex.map(lambda t: _variant(tmp, precision, t[0], t[1]), todo)))
         for N in sizes:
             workload, batch = WORKLOAD_FOR_N[N]
             ref = _time(ROOT, workload, batch, precision)
             rows = []
-            for sh in CANDIDATES.get(N, []):
+            for sh in shape_candidates(precision, N):
                 if (N, sh) not in roots:
                     continue
                 r = _time(roots[(N, sh)], workload, batch, precision)
@@ -251,6 +251,13 @@ def current_shape(precision, N):
         text = fh.read()
     m = re.search(r"^DGFS_SHAPE(3?)\(%s, %d, (\d+), (\d+)(?:, (\d+))?\)$" % (T, N), text, re.M)
     return int(m.group(2)), int(m.group(3)), int(m.group(4) or 1)
+
+
+def shape_candidates(precision, N):
+    """The shapes a run tries: the list, and the library's own where the list lacks it."""
+    cur = current_shape(precision, N)
+    listed = CANDIDATES.get(N, [])
+    return listed if cur in listed else [cur] + listed
 
 
 def current_radix(precision, N):

@@ -1,4 +1,5 @@
-"""The tuner's rules on the CPU: which objects a variant links, which radix schedule it keeps; the shape table."""
+"""The tuner's rules on the CPU: which objects a variant links, which shapes it tries, which radix
+schedule it keeps; the shape table."""
 
 import os
 import re
@@ -20,6 +21,13 @@ def test_equal_times_are_decided_by_the_error():
             {"radix": 422, "ms": 147.5, "err_vs_fp64": 1.0e-6}]
     assert tune.best_radix(rows)["radix"] == 44
     assert tune.best_radix(rows[::2])["radix"] == 28
+
+
+def test_a_run_tries_the_librarys_own_shape():
+    for precision in ("fp32", "fp64"):
+        for N in tune.WORKLOAD_FOR_N:
+            tried = tune.shape_candidates(precision, N)
+            assert tune.current_shape(precision, N) in tried and set(tune.CANDIDATES[N]) <= set(tried)
 
 
 def test_small_grids_are_sized_for_enough_warps():
