@@ -205,8 +205,8 @@ int dgfs_eval_collision_host(dgfs_plan plan, const void* f_host, void* Q_host, i
   // alternate between two evaluation streams (the caller's and the plan's second one) and two
   // workspaces, so chunk k+1's kernel starts while chunk k's finishes its last work items;
   // chunk k+2 reuses chunk k's stream and workspace and so runs after it.  Measured on the
-  // 4096-node N = 32 batch in 8 chunks: 312.9 ms per batch with two workspaces against
-  // 337.6 ms with one (the device-resident launch: 309.1 ms).
+  // 4096-node N = 32 batch in 8 chunks: 154.2 ms per batch with two workspaces against 158.1 ms with one
+  // (the device-resident launch: 150.9 ms).
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaStream_t evs[2] = {st, p.eval2};
   int nchunks = batch / 256;

@@ -44,10 +44,13 @@
 // runs two phases behind step A, entry by entry, on the half space of its Hermitian part (vss_step_c).
 // Groups hold one or two entries.
 //
+// The finish transforms gain and loss back, whose rounding every result keeps: FP32 carries it along
+// there (VGeo::FINE_Z).
+//
 // Measured on the GB300 against the complex-transform kernel this one replaced: 4096 nodes of N = 32
-// FP32 285 -> 145 ms, 3001 of N = 24 75.1 -> 36.6, 8192 of N = 16 28.7 -> 16.3, 61 three-species nodes
-// of N = 48 86.0 -> 35.8, 61 nodes of N = 32 FP64 201 -> 82, VSS 37 three-species nodes of N = 48
-// (M = 32) 339 -> 147 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
+// FP32 285 -> 151 ms, 3001 of N = 24 74.9 -> 37.7, 8192 of N = 16 28.6 -> 16.7, 61 three-species nodes
+// of N = 48 86.0 -> 35.9, 61 nodes of N = 32 FP64 184 (201 on another device) -> 83, VSS 37 three-species
+// nodes of N = 48 (M = 32) 339 -> 146 ms.  What bounds it: FP64 the FP64 pipe (79 % of its cycles); FP32 latency -- the
 // FMA pipes run half their cycles (N = 16: the L1 data path three quarters), the stalls are L2 loads
 // of the x-passed spectra, whose workspaces together exceed L2 from N = 24 on.
 #pragma once
