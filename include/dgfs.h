@@ -118,7 +118,8 @@ typedef struct {
  * for N outside the list of the N field; DGFS_ERR_INVALID_ARG for a field outside its stated range,
  * a non-finite mass, b_ij, kappa, weight or R, a direction that is not a unit vector, an
  * unknown flag, or R > 0 with DGFS_PER_PAIR_R.  DGFS_ERR_OOM when the tables or the
- * workspace do not fit.  DGFS_ERR_CUDA when a CUDA call fails. */
+ * smallest workspace do not fit (with less memory than the full workspace takes, a plan takes a
+ * smaller one: the same results, in more time).  DGFS_ERR_CUDA when a CUDA call fails. */
 int dgfs_create_plan(const dgfs_plan_desc* desc, dgfs_plan* out);
 
 /* Release the plan's device memory.  Waits for the plan's most recent evaluation (not for
