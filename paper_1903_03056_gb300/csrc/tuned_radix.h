@@ -2,10 +2,9 @@
 // code, first stage first (442 = radix 4, 4, then 2).  paper_1903_03056_gb300/tune.py --radix times the
 // orders on the device and writes these lines.
 // FP32 lines of N points run as transforms of N / 2, so the FP32 entry of N / 2 serves grid size N.
-// Where the orders' times agree within 1 %, the one with the smallest error against 64 bits is kept:
-// 16 takes 44 (N = 32: 1.32e-6 -> 1.21e-6 of ||Q|| on 8 two-species nodes, 28 measured 145.5 ms against
-// 146.0), 24 takes 243 (N = 48: 1.45e-6 -> 1.23e-6, 38 35.8 ms against 36.1); radix 3 last is the better
-// order throughout.
+// Where the orders' times agree within 2 %, the one with the smallest error against 64 bits is kept (64
+// nodes, 2-norm): 16 takes 44 (N = 32: 1.10e-6 of ||Q||, 149.8 ms; 82 1.23e-6, 148.1), 24 takes 243 (N = 48:
+// 9.80e-7, 296.3 ms; 38 1.23e-6, 294.2), 12 takes 43 (N = 24: 8.9e-7; 34 1.06e-6, the same time).
 #pragma once
 
 DGFS_RADIX(float, 4, 4)

@@ -19,7 +19,7 @@ def main():
     ap.add_argument("--checksum", action="store_true", help="add the SHA-1 of the output bytes")
     ap.add_argument("--compare-fp64", type=int, default=0, metavar="K",
                     help="also evaluate the first K nodes with an FP64 plan and report the largest "
-                         "per-node max |Q - Q_fp64| / max |Q_fp64|")
+                         "per-node max |Q - Q_fp64| / max |Q_fp64| and the 2-norm over all of them")
     ap.add_argument("--n-rho", type=int, default=None,
                     help="override the workload's radial nodes (smaller tables for profiling)")
     a = ap.parse_args()
@@ -67,6 +67,7 @@ def main():
         dims = tuple(range(1, Q64.dim()))
         err = ((Q[:K].double() - Q64).abs().amax(dim=dims) / Q64.abs().amax(dim=dims)).max()
         out["err_vs_fp64"] = float(err)
+        out["l2_vs_fp64"] = float((Q[:K].double() - Q64).norm() / Q64.norm())
     print(json.dumps(out))
     plan.close()
 
